@@ -125,7 +125,8 @@ typedef enum {
     RPCHOLQR_OPT_SPIN_LIMIT = 0,    /* polls a device-side pipeline wait makes before it gives up and the
                                        call reports RPCHOLQR_ERR_TIMEOUT (default 2^24, 1 <= value <=
                                        2^40).  A kernel's final wait for its own tensor-core work, before
-                                       it releases its tensor memory, always uses the default. */
+                                       it releases its tensor memory, and the sketch QR's waits inside
+                                       its thread-block cluster always use the default. */
     RPCHOLQR_OPT_SCALE_SAMPLE = 1,  /* 1 (default): the sample is scaled by sqrt(m/s) (Remark r_exp);
                                        0: unscaled.  R is the same in exact arithmetic either way. */
     RPCHOLQR_OPT_DETERMINISTIC = 2, /* 1 (default, the only value built): every reduction is a

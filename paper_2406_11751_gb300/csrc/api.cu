@@ -19,10 +19,13 @@ void launch_sample_indices(uint64_t seed, uint64_t stream_id, int64_t m, int32_t
 void launch_sample_gather(const double* A, int64_t m, int32_t n, int64_t lda, int32_t s, uint64_t seed,
                           uint64_t stream_id, double scale, double* As, int64_t lds, int32_t np,
                           int64_t* idx_out, int32_t* info, cudaStream_t st);
-// smallfactor.cu
-cudaError_t launch_householder(double* W, int64_t lds, int s, int n, int np, double* Rs,
-                               double* Rs_user, int32_t* info, cudaStream_t st);
+// sketchqr.cu
+cudaError_t launch_householder(double* W, int64_t lds, int s, int n, int np, double* Rs, double* Rs_user, double* qws,
+                               int32_t* info, cudaStream_t st);
 size_t householder_smem_bytes(int s, int n);
+int householder_launches(int n);
+size_t householder_ws_bytes(int np);
+// smallfactor.cu
 cudaError_t launch_cholesky(const double* G, int64_t ldg, int n, int np, double* R, double* R_user,
                             int32_t* info, cudaStream_t st);
 void launch_triu_mul(const double* R1, int64_t ld1, const double* Rs, int64_t lds, int n, double* R,
@@ -169,6 +172,7 @@ struct rpcholqr_plan_s {
     double* frag_1 = nullptr;
     double* diag_1 = nullptr;
     double* gpart = nullptr;    // grid x np x np
+    double* qws = nullptr;      // the sketch QR's workspace (householder_ws_bytes)
     int32_t* info_ws = nullptr; // 2 ints (for step calls without a caller info)
     // staging for rpcholqr_factor_host
     double* hA = nullptr;
@@ -242,7 +246,7 @@ struct rpcholqr_plan_s {
 namespace {
 
 struct WsLayout {
-    size_t As, Rs, R1, G, frag_s, diag_s, frag_1, diag_1, gpart, info, total;
+    size_t As, Rs, R1, G, frag_s, diag_s, frag_1, diag_1, gpart, qws, info, total;
 };
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
@@ -274,6 +278,7 @@ WsLayout ws_layout(int32_t max_n, int32_t max_s, int grid) {
     L.frag_1 = take(sizeof(double) * np * np);
     L.diag_1 = take(sizeof(double) * (np / 8) * 64);
     L.gpart = take(sizeof(double) * static_cast<size_t>(grid) * np * np);
+    L.qws = take(householder_ws_bytes(static_cast<int>(np)));
     L.info = take(sizeof(int32_t) * 2);
     L.total = off;
     return L;
@@ -732,6 +737,7 @@ rpcholqr_status rpcholqr_plan_create(rpcholqr_plan* plan, int device, rpcholqr_m
     p->frag_1 = reinterpret_cast<double*>(b + L.frag_1);
     p->diag_1 = reinterpret_cast<double*>(b + L.diag_1);
     p->gpart = reinterpret_cast<double*>(b + L.gpart);
+    p->qws = reinterpret_cast<double*>(b + L.qws);
     p->info_ws = reinterpret_cast<int32_t*>(b + L.info);
     if (mode == RPCHOLQR_SPLIT64) {
         const size_t np = static_cast<size_t>(p->np);
@@ -907,10 +913,10 @@ static rpcholqr_status sketch_internal(rpcholqr_plan p, const double* A, int64_t
     if (pm) pm->mark(RPCHOLQR_PHASE_SKETCH_QR);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_SKETCH_QR, 2.0 * s * n * n - 2.0 * n * n * n / 3.0);
-        if (launch_householder(p->As, lds, s, n, np, p->Rs, Rs_user, info, st) != cudaSuccess)
+        if (launch_householder(p->As, lds, s, n, np, p->Rs, Rs_user, p->qws, info, st) != cudaSuccess)
             return RPCHOLQR_ERR_CUDA;
     }
-    ++p->launches;
+    p->launches += householder_launches(n);
     return RPCHOLQR_OK;
 }
 
@@ -1502,8 +1508,8 @@ rpcholqr_status rpcholqr_factor_f32(rpcholqr_plan p, const float* A, int64_t m, 
         ++p->launches;
     }
     pm.mark(RPCHOLQR_PHASE_SKETCH_QR);
-    if (launch_householder(p->As, s, s, n, np, p->Rs, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
-    ++p->launches;
+    if (launch_householder(p->As, s, s, n, np, p->Rs, nullptr, p->qws, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
+    p->launches += householder_launches(n);
     // pass 1 in FP32: A1 = A R_s^{-1} into Q, then the Gram partials and their FP64 sum
     pm.mark(RPCHOLQR_PHASE_PREP_RS);
     launch_prep_f32(p->Rs, np, n, p->T32, p->rinv32, RPCHOLQR_ERR_SINGULAR_SKETCH, info, st);
@@ -1688,8 +1694,8 @@ static rpcholqr_status factor_host_split(rpcholqr_plan p, const double* A, int64
     }
     launch_sample_rows(p->hrows_dev, n, s, sample_scale(p, m, s), p->As, s, np,
                        info, st);
-    if (launch_householder(p->As, s, s, n, np, p->Rs, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
-    p->launches += 3;
+    if (launch_householder(p->As, s, s, n, np, p->Rs, nullptr, p->qws, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
+    p->launches += 2 + householder_launches(n);
     // pass 1, block by block as A arrives
     launch_fill_noexp(p->colexp, n, st);
     prep_blocks(p, p->Rs, np, n, p->frag_s, p->diag_s, info, st, split_sub(p));
@@ -2011,8 +2017,8 @@ rpcholqr_status rpcholqr_sketch_r_from_sample(rpcholqr_plan p, const double* As,
     if (rc != RPCHOLQR_OK) return rc;
     const int np = pad_np(n);
     launch_sample_to_colmajor(As, ld_as, s, n, np, p->As, s, st);
-    if (launch_householder(p->As, s, s, n, np, p->Rs, Rs, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
-    p->launches += 2;
+    if (launch_householder(p->As, s, s, n, np, p->Rs, Rs, p->qws, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
+    p->launches += 1 + householder_launches(n);
     return check_launch();
 }
 

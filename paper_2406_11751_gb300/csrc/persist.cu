@@ -23,20 +23,20 @@
 // Bits: P_i is the single call's pass-1 grid (one CTA per 128-row panel, at most one per SM), the
 // panels of part b are those CTA b of the single call solves, each part's Gram partial is accumulated
 // by the same code, and the parts are summed in the single call's order; the sample, the Householder
-// QR (the cluster kernel's per-column arithmetic is the same for one CTA of the same size), the
-// Cholesky factorisation (the same virtual-thread layout), the fragment tables and R = R1 R_s are the
+// QR (every sum's order depends on the shape alone, not on the CTAs that share it), the Cholesky factorisation (the same virtual-thread layout), the fragment tables and R = R1 R_s are the
 // same device functions.  So every matrix's Q, R and status are bit-identical to rpcholqr_factor on
 // an FP64 plan, whatever else is in the batch.
 #include <algorithm>
 
 #include "philox.cuh"
 #include "rowpass.cuh"
+#include "sketchqr.cuh"
 #include "smallfactor.cuh"
 
 namespace rpq {
 namespace {
 
-constexpr int kPThreads = kClusterQrThreads;   // the Householder QR's bits are those of 256-thread CTAs
+constexpr int kPThreads = 256;
 constexpr int kBatchMaxNP = 128;
 constexpr int kPanelRowsForParts = 128;        // the single call sizes its pass-1 grid by 128-row panels
 
@@ -67,6 +67,7 @@ struct BatchArgs {
     int64_t max_m;
     int32_t max_n, max_s, sms, scale_sample;
     long spin;
+    size_t smem;           // dynamic shared memory of a CTA
 };
 
 __host__ __device__ inline uint64_t item_code(int type, int i, int64_t b) {
@@ -216,7 +217,7 @@ __device__ void item_sketch(const BatchArgs& a, int i, double* psm) {
     }
     if (__syncthreads_or(bad) && tid == 0) set_status(info, RPCHOLQR_ERR_NONFINITE);
     __syncthreads();
-    if (load_status(info) == 0) hh_factor<false>(w.As, s, s, n, np, w.Rs, nullptr, info, 0u, 1u, psm);
+    if (load_status(info) == 0) qr_factor_one_cta<kPThreads>(w.As, s, s, n, np, w.Rs, info, psm, a.smem);
     __syncthreads();
     if (load_status(info) == 0)
         for (int e = tid; e < np * np + (np / 8) * 64; e += kPThreads)
@@ -381,7 +382,8 @@ size_t batch_smem_bytes(int32_t max_n, int32_t max_s) {
     size_t b = 0;
     for (int np = 16; np <= npm; np += 16) b = std::max(b, rowpass_smem_bytes(np));
     b = std::max(b, static_cast<size_t>(npm + kCholParts) * npm * sizeof(double));
-    b = std::max(b, static_cast<size_t>(max_s + max_n + 34) * sizeof(double));
+    // the sketch: its panels stay in shared memory for samples of up to 3 max_n rows (the paper's choice of s)
+    b = std::max(b, qr_one_bytes(max_n, std::min(max_s, 3 * max_n)));
     b = std::max(b, static_cast<size_t>(max_s) * sizeof(int64_t));
     return b;
 }
@@ -426,13 +428,14 @@ cudaError_t launch_batch_persistent(int32_t count, const double* const* A, const
     a.items = reinterpret_cast<uint64_t*>(w + L.items_off);
     a.queue = reinterpret_cast<int32_t*>(w + L.queue_off);
     a.max_m = max_m; a.max_n = max_n; a.max_s = max_s; a.sms = sms; a.scale_sample = scale_sample; a.spin = spin;
+    a.smem = batch_smem_bytes(max_n, max_s);
     k_batch_setup<<<1, 1024, 0, st>>>(a);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
     cfg.blockDim = dim3(kPThreads, 1, 1);
-    cfg.dynamicSmemBytes = batch_smem_bytes(max_n, max_s);
+    cfg.dynamicSmemBytes = a.smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -1,35 +1,9 @@
 // The small dense steps of Algorithm alg_2 (Section 4):
-//   'factor'   A_s = Q_s R_s   -- Householder QR of the s x n sample on a 16-CTA cluster;
 //   'Cholesky' G_1 = R_1^T R_1 -- n x n upper Cholesky, one CTA;
 //   'recover'  R = R_1 R_s     -- product of upper-triangular factors, one CTA per row.
-#include <cfloat>
-
 #include "smallfactor.cuh"
 
 namespace rpq {
-
-// Block-wide sum of one double per thread (every thread gets the result).
-__device__ __forceinline__ double block_sum(double v, double* red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    const int nw = blockDim.x >> 5;
-    double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += red[w];
-    return s;
-}
-
-__global__ void __launch_bounds__(kClusterQrThreads)
-k_hh_cluster(double* __restrict__ W, int64_t lds, int s, int n, int np, double* __restrict__ Rs,
-             double* __restrict__ Rs_user, const int32_t* info_in, int32_t* info) {
-    extern __shared__ double qsm[];
-    // every CTA of the cluster sees the same status, so all take the same number of barriers
-    if (load_status(info_in) != 0) return;
-    hh_factor<true>(W, lds, s, n, np, Rs, Rs_user, info, cluster_rank(), cluster_size(), qsm);
-}
 
 __global__ void __launch_bounds__(kCholThreads)
 k_cholesky(const double* __restrict__ G, int64_t ldg, int n, int np, double* __restrict__ R,
@@ -232,43 +206,6 @@ __global__ void __launch_bounds__(256) k_triu_inv(const double* __restrict__ T, 
 }
 
 // ---- host launchers ------------------------------------------------------------------------------
-size_t householder_smem_bytes(int s, int n) { return (static_cast<size_t>(s) + n + 40) * sizeof(double); }
-
-// W: s x n column-major (ld lds).  One cluster of kClusterQr CTAs (16 needs the non-portable cluster
-// size; 8 is used where the device refuses 16).
-cudaError_t launch_householder(double* W, int64_t lds, int s, int n, int np, double* Rs,
-                               double* Rs_user, int32_t* info, cudaStream_t st) {
-    const size_t smem = householder_smem_bytes(s, n);
-    cudaError_t err = cudaFuncSetAttribute(k_hh_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(smem));
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(k_hh_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (err != cudaSuccess) return err;
-    for (int csize : {kClusterQr, 8}) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(csize, 1, 1);
-        cfg.blockDim = dim3(kClusterQrThreads, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = csize;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, k_hh_cluster, &cfg) != cudaSuccess || clusters < 1) {
-            cudaGetLastError();
-            continue;
-        }
-        err = cudaLaunchKernelEx(&cfg, k_hh_cluster, W, lds, s, n, np, Rs, Rs_user,
-                                 static_cast<const int32_t*>(info), info);
-        return err == cudaSuccess ? cudaGetLastError() : err;
-    }
-    return cudaErrorInvalidConfiguration;
-}
-
 cudaError_t launch_cholesky(const double* G, int64_t ldg, int n, int np, double* R, double* R_user,
                             int32_t* info, cudaStream_t st) {
     if (np > kMaxNP) {

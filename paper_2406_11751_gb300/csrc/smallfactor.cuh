@@ -1,133 +1,9 @@
-// Device-side pieces of the small dense steps of Algorithm alg_2 (Section 4) -- the Householder QR of
-// the sample and the n x n Cholesky factorisation -- shared by their kernels (smallfactor.cu) and the
-// persistent batched kernel (persist.cu).
+// Device-side pieces of the n x n steps of Algorithm alg_2 (Section 4) -- the Cholesky factorisation and
+// R = R_1 R_s -- shared by their kernels (smallfactor.cu) and the persistent batched kernel (persist.cu).
 #pragma once
-#include <cfloat>
-
 #include "common.cuh"
 
 namespace rpq {
-
-// Householder QR of the sample on one thread-block cluster.  FP64 on GB300 retires one warp-wide
-// DFMA per 64 cycles per SM sub-partition, so a single CTA would run this O(s n^2) step at 1/152 of
-// the GPU; instead kClusterQr CTAs (one per SM) share the columns round-robin and advance one
-// column per hardware cluster barrier:
-//   every CTA: read column j (rows j..s-1), form the reflector (beta = -sign(alpha)||x||,
-//              v = x / (alpha - beta) with v_j = 1, tau = (beta - alpha) / beta; no reflection when
-//              nothing is below the diagonal) -- identical in every CTA;
-//   every CTA: apply it to its own columns k > j;
-//   cluster barrier (release/acquire orders the global-memory column updates).
-// The diagonal betas are kept in shared memory (column j is still being read by the other CTAs
-// while it is reflected) and CTA 0 assembles R_s at the end: each row negated where its diagonal is
-// negative, padded with the identity; a diagonal that is 0, subnormal or not finite sets
-// SINGULAR_SKETCH.  W: s x n column-major (ld lds), overwritten.
-constexpr int kClusterQr = 16;
-constexpr int kClusterQrThreads = 256;
-
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ unsigned cluster_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ unsigned cluster_size() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(r));
-    return r;
-}
-
-// The factorisation itself, by the calling CTA as CTA `rank` of `csize` (CLUSTER: the CTAs of a thread-block
-// cluster, joined by the hardware cluster barrier; otherwise csize = 1 and a CTA barrier).  The arithmetic
-// of every column step depends on the CTA size (kClusterQrThreads threads) but not on csize, so one CTA
-// alone gives the cluster's bits.  qsm: (s + n + 34) doubles of shared memory.
-template <bool CLUSTER>
-__device__ __forceinline__ void hh_factor(double* __restrict__ W, int64_t lds, int s, int n, int np,
-                                          double* __restrict__ Rs, double* __restrict__ Rs_user, int32_t* info,
-                                          unsigned rank, unsigned csize, double* qsm) {
-    double* v = qsm;                 // s
-    double* betas = qsm + s;         // n
-    double* red = betas + n;         // 32 warp partials, then tau and 1 / (alpha - beta)
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
-
-    for (int j = 0; j < n; ++j) {
-        const double* colj = W + static_cast<int64_t>(j) * lds;
-        double part = 0.0;
-        for (int i = j + 1 + tid; i < s; i += blockDim.x) part += colj[i] * colj[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) red[warp] = part;
-        __syncthreads();
-        // the reflector's scalars in one thread (FP64 square root and divisions are long sequences on
-        // the FP64 units; formed once instead of by every thread), then shared
-        if (tid == 0) {
-            double sigma = 0.0;
-            for (int w = 0; w < nwarps; ++w) sigma += red[w];
-            const double alpha = colj[j];
-            double beta, tau, inv;
-            if (sigma == 0.0) {
-                beta = alpha; tau = 0.0; inv = 0.0;
-            } else {
-                const double nrm = sqrt(alpha * alpha + sigma);
-                beta = alpha >= 0.0 ? -nrm : nrm;
-                tau = (beta - alpha) / beta;
-                inv = 1.0 / (alpha - beta);
-            }
-            betas[j] = beta;
-            red[32] = tau;
-            red[33] = inv;
-        }
-        __syncthreads();
-        const double tau = red[32], inv = red[33];
-        for (int i = j + tid; i < s; i += blockDim.x) v[i] = (i == j) ? 1.0 : colj[i] * inv;
-        __syncthreads();
-        if (tau != 0.0) {
-            // this CTA's columns k > j: k = rank (mod csize); one warp per column
-            const int k0 = j + 1 + static_cast<int>((rank + csize - static_cast<unsigned>((j + 1) % csize)) % csize);
-            for (int k = k0 + warp * static_cast<int>(csize); k < n; k += nwarps * static_cast<int>(csize)) {
-                double* colk = W + static_cast<int64_t>(k) * lds;
-                // four independent partial sums keep four column loads in flight per lane
-                double w0 = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
-                int i = j + lane;
-                for (; i + 96 < s; i += 128) {
-                    w0 += v[i] * colk[i];
-                    w1 += v[i + 32] * colk[i + 32];
-                    w2 += v[i + 64] * colk[i + 64];
-                    w3 += v[i + 96] * colk[i + 96];
-                }
-                for (; i < s; i += 32) w0 += v[i] * colk[i];
-                double w = (w0 + w1) + (w2 + w3);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-                const double tw = tau * w;
-#pragma unroll 4
-                for (int i2 = j + lane; i2 < s; i2 += 32) colk[i2] -= v[i2] * tw;
-            }
-        }
-        __syncthreads();
-        if constexpr (CLUSTER) cluster_sync_all();
-    }
-
-    if (rank != 0) return;
-    bool singular = false;
-    for (int e = tid; e < np * np; e += blockDim.x) {
-        const int r = e / np, c = e - r * np;
-        double val;
-        if (r < n && c < n) {
-            const double d = betas[r];
-            const double sg = d < 0.0 ? -1.0 : 1.0;
-            val = c > r ? sg * W[static_cast<int64_t>(c) * lds + r] : (c == r ? fabs(d) : 0.0);
-            if (c == r && (!isfinite(d) || fabs(d) < DBL_MIN)) singular = true;
-            if (Rs_user) Rs_user[r * n + c] = val;
-        } else {
-            val = (r == c) ? 1.0 : 0.0;
-        }
-        Rs[e] = val;
-    }
-    if (__syncthreads_or(singular) && tid == 0) set_status(info, RPCHOLQR_ERR_SINGULAR_SKETCH);
-}
 
 // Upper Cholesky G = R^T R, row by row:
 //   t_l = G[j][l] - sum_{k<j} R[k][j] R[k][l]  (l >= j),  R[j][j] = sqrt(t_j),  R[j][l] = t_l / R[j][j].
