@@ -35,12 +35,12 @@ void launch_prep_tri(const double* T, int64_t ldt, int n, int np, double* frag, 
                      const int32_t* info, cudaStream_t st);
 cudaError_t launch_rowpass(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                            int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                           int32_t* info, int grid, cudaStream_t st);
+                           int32_t* info, int sms, cudaStream_t st);
 void launch_gram_reduce(const double* gpart, int nparts, int np, int n, double* G, int64_t ldg,
                         const int32_t* info, cudaStream_t st);
 cudaError_t launch_rowpass_ex(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                               int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                              int32_t* info, int grid, cudaStream_t st, bool check_finite, int32_t* rowexp,
+                              int32_t* info, int sms, cudaStream_t st, bool check_finite, int32_t* rowexp,
                               int rowexp_mode, int32_t* colexp);
 void launch_fill_noexp(int32_t* p, int n, cudaStream_t st);
 // probe.cu
@@ -422,12 +422,6 @@ void select_tuning(rpcholqr_plan_s* p, int64_t m, int n) {
 int split_sub(const rpcholqr_plan_s* p) {
     const int v = p->cur_tune.split_sub;
     return v == 16 || v == 32 ? v : (p->cur_np > kMaxNP ? kSplitSubWide : kSplitSub);
-}
-
-// CTAs of a row pass over m rows: one per 128-row panel, at most one per SM.
-int row_grid(const rpcholqr_plan_s* p, int64_t m) {
-    const int64_t panels = (m + 127) / 128;
-    return static_cast<int>(panels < p->grid ? panels : p->grid);
 }
 
 // The smoothed sample of the plan's kind into p->As (column-major, ld s, np columns).
@@ -954,7 +948,7 @@ static rpcholqr_status solve_split_right(rpcholqr_plan_s* p, const double* X, in
                                          int64_t ldt, int64_t m, int n, double* Y, int64_t ldy, const double* frag,
                                          const double* diag, int32_t* info, cudaStream_t st, const PhaseMarks* pm,
                                          int64_t row0 = 0) {
-    const int grid = row_grid(p, m);
+    const int grid = p->grid;
     const int blk = kSplitBlk, sub = split_sub(p);
     bool first_update = true;
     auto update = [&](int c0, int K, int c1, int N, const double* B, int64_t ldb) -> rpcholqr_status {
@@ -1019,7 +1013,7 @@ static rpcholqr_status solve_split_wide(rpcholqr_plan_s* p, const double* X, int
     bool marked = false;
     for (int64_t r0 = 0; r0 < m; r0 += p->img_rows) {
         const int64_t rows = m - r0 < p->img_rows ? m - r0 : p->img_rows;
-        const int grid = row_grid(p, rows);
+        const int grid = p->grid;
         const double* Xc = X + r0 * ldx;
         double* Yc = Y + r0 * ldy;
         for (int J = 0; J * kBlk < n; ++J) {
@@ -1091,7 +1085,7 @@ static rpcholqr_status solve_blocked(rpcholqr_plan_s* p, const double* X, int64_
                               int64_t m, int n, double* Y, int64_t ldy, const double* frag, const double* diag,
                               bool split, bool check_finite, int32_t* info, cudaStream_t st,
                               const PhaseMarks* pm, bool pass1_marks) {
-    const int grid = row_grid(p, m);
+    const int grid = p->grid;
     for (int J = 0; J * kBlk < n; ++J) {
         const int c0 = J * kBlk;
         const int nj = n - c0 < kBlk ? n - c0 : kBlk;
@@ -1223,11 +1217,10 @@ static rpcholqr_status precondition_internal(rpcholqr_plan p, const double* A, i
     launch_prep_tri(Rs, ldrs, n, np, p->frag_s, p->diag_s, info, st);
     ++p->launches;
     if (check_launch() != RPCHOLQR_OK) return RPCHOLQR_ERR_CUDA;
-    const int grid = row_grid(p, m);
     if (pm) pm->mark(RPCHOLQR_PHASE_PASS1);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, 2.0 * m * n * n);
-        if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, p->frag_s, p->diag_s, p->gpart, info, grid, st) !=
+        if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, p->frag_s, p->diag_s, p->gpart, info, p->grid, st) !=
             cudaSuccess)
             return RPCHOLQR_ERR_CUDA;
     }
@@ -1237,7 +1230,7 @@ static rpcholqr_status precondition_internal(rpcholqr_plan p, const double* A, i
         pm->mark(RPCHOLQR_PHASE_PASS1_SOLVE2);
         pm->mark(RPCHOLQR_PHASE_GRAM_REDUCE);
     }
-    launch_gram_reduce(p->gpart, grid, np, n, G, ldg, info, st);
+    launch_gram_reduce(p->gpart, rowpass_parts(np, m, p->grid), np, n, G, ldg, info, st);
     ++p->launches;
     return check_launch();
 }
@@ -1256,11 +1249,10 @@ static rpcholqr_status solve_internal(rpcholqr_plan p, const double* X, int64_t 
     launch_prep_tri(T, ldt, n, np, p->frag_1, p->diag_1, info, st);
     ++p->launches;
     if (check_launch() != RPCHOLQR_OK) return RPCHOLQR_ERR_CUDA;
-    const int grid = row_grid(p, m);
     if (pm) pm->mark(RPCHOLQR_PHASE_PASS2);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(m) * n * n);
-        if (launch_rowpass(false, np, X, ldx, Y, ldy, m, n, p->frag_1, p->diag_1, nullptr, info, grid, st) !=
+        if (launch_rowpass(false, np, X, ldx, Y, ldy, m, n, p->frag_1, p->diag_1, nullptr, info, p->grid, st) !=
             cudaSuccess)
             return RPCHOLQR_ERR_CUDA;
     }
@@ -1914,12 +1906,10 @@ static rpcholqr_status cholqr_step(rpcholqr_plan p, const double* X, int64_t m, 
         return solve_internal(p, X, m, n, ldx, R_out, np, Q, ldq, info, st, nullptr);
     }
     launch_prep_tri(nullptr, 0, 0, np, p->frag_s, p->diag_s, info, st);   // identity preconditioner
-    const int64_t panels = (m + 127) / 128;
-    const int grid = static_cast<int>(panels < p->grid ? panels : p->grid);
-    if (launch_rowpass(true, np, X, ldx, Q, ldq, m, n, p->frag_s, p->diag_s, p->gpart, info, grid, st) !=
+    if (launch_rowpass(true, np, X, ldx, Q, ldq, m, n, p->frag_s, p->diag_s, p->gpart, info, p->grid, st) !=
         cudaSuccess)
         return RPCHOLQR_ERR_CUDA;
-    launch_gram_reduce(p->gpart, grid, np, n, p->G, np, info, st);
+    launch_gram_reduce(p->gpart, rowpass_parts(np, m, p->grid), np, n, p->G, np, info, st);
     if (shifted) {
         launch_scholqr3_shift(p->G, np, n, m, info, st);
         ++p->launches;

@@ -17,18 +17,33 @@ __host__ __device__ constexpr int pad16(int n) { return (n + kPad - 1) / kPad * 
 __host__ __device__ constexpr int pad_np(int n) { return n <= kMaxNP ? pad16(n) : (n + 63) / 64 * 64; }
 
 // ---- launch shape of the FP64 row passes (rowpass.cu) ----------------------------------------------
-// Warps per CTA: 8 when the 256-row panel fits shared memory (NP <= 64), else 4 (128-row panel).
-__host__ __device__ constexpr int rowpass_warps(int np) { return np <= 64 ? 8 : 4; }
-// Rows of one panel (32 per warp).
-__host__ __device__ constexpr int rowpass_rows(int np) { return 32 * rowpass_warps(np); }
+// A panel is 256 rows (8 warps x 32) up to 64 columns, 128 rows (8 warps x 16) above: two warps on each of the
+// SM's four schedulers, so that one warp's dependent chains and shared-memory loads run under the other's FP64
+// work (four warps x 32 rows at 128 columns kept the FP64 pipe 74-83 % busy).  Matrices too short to give every
+// SM such a panel take one panel of 64 to 128 rows (4 to 8 warps x 16) per SM.
+constexpr int kRowpassWarps = 8, kRowpassMinWarps = 4;
+__host__ __device__ constexpr int rowpass_rows_per_warp(int np) { return np <= 64 ? 32 : 16; }
+__host__ __device__ constexpr int rowpass_big_rows(int np) { return kRowpassWarps * rowpass_rows_per_warp(np); }
+// Warps of the short shape for m rows on sms SMs, 0: the big panels.
+__host__ __device__ constexpr int rowpass_short_warps(int np, int64_t m, int sms) {
+    const int64_t w = (m + 16 * static_cast<int64_t>(sms) - 1) / (16 * static_cast<int64_t>(sms));
+    return w * 16 >= rowpass_big_rows(np) || w > kRowpassWarps ? 0
+           : w < kRowpassMinWarps                              ? kRowpassMinWarps
+                                                               : static_cast<int>(w);
+}
+__host__ __device__ constexpr int rowpass_rows(int np, int64_t m, int sms) {
+    const int w = rowpass_short_warps(np, m, sms);
+    return w ? 16 * w : rowpass_big_rows(np);
+}
+// CTAs of the fused Gram pass, each leaving one partial: one per panel, at most one per SM.
+__host__ __device__ constexpr int rowpass_parts(int np, int64_t m, int sms) {
+    const int64_t rows = rowpass_rows(np, m, sms), panels = (m + rows - 1) / rows;
+    return static_cast<int>(panels < sms ? panels : sms);
+}
 // The plain solve up to 48 columns runs two CTAs per SM (128 registers a thread, two panels fit the
 // shared memory): one CTA's panel load overlaps the other's FP64 work and each scheduler has four
-// warps' dependent chains to interleave.  The fused Gram keeps one CTA per SM: the caller sizes its
-// per-CTA partials for the grid it passes, which the launcher then uses unchanged.
+// warps' dependent chains to interleave.  The fused Gram keeps one CTA per SM (one partial each).
 __host__ __device__ constexpr int rowpass_ctas_per_sm(int np, bool syrk) { return !syrk && np <= 48 ? 2 : 1; }
-static_assert(rowpass_ctas_per_sm(16, true) == 1 && rowpass_ctas_per_sm(64, true) == 1 &&
-                  rowpass_ctas_per_sm(128, true) == 1,
-              "the fused Gram pass writes one partial per CTA of the grid its caller passes");
 
 // ---- power-of-two bounds used by the split-precision products ------------------------------------
 // exp_bound(v): |v| < 2^e for a normal v (e = unbiased exponent + 1); kNoExp for 0 or subnormal.

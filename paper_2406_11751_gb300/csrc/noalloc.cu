@@ -26,7 +26,7 @@ void launch_prep_tri(const double* T, int64_t ldt, int n, int np, double* frag, 
                      const int32_t* info, cudaStream_t st);
 cudaError_t launch_rowpass(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                            int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                           int32_t* info, int grid, cudaStream_t st);
+                           int32_t* info, int sms, cudaStream_t st);
 void launch_gram_reduce(const double* gpart, int nparts, int np, int n, double* G, int64_t ldg,
                         const int32_t* info, cudaStream_t st);
 
@@ -39,8 +39,6 @@ constexpr size_t kPartDoubles = static_cast<size_t>(kNoAllocMaxCtas) * kNoAllocM
 // fragment table | diagonal blocks | per-CTA Gram partials (each slice 256-byte aligned)
 constexpr size_t kScratchDoubles = kFragDoubles + kDiagDoubles + kPartDoubles;
 static_assert(kFragDoubles % 32 == 0 && kDiagDoubles % 32 == 0, "slices must stay 256-byte aligned");
-static_assert(rowpass_ctas_per_sm(kNoAllocMaxN, true) == 1,
-              "the partial slice holds one Gram partial per CTA of the grid this file launches");
 
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
@@ -99,13 +97,10 @@ extern "C" rpcholqr_status rpcholqr_precondition_gram_noalloc(const double* A, i
     double* gpart = scratch + kFragDoubles + kDiagDoubles;
     launch_prep_tri(Rs, n, n, np, frag, diag, info, st);
     if (cudaGetLastError() != cudaSuccess) return RPCHOLQR_ERR_CUDA;
-    // one CTA per panel of the fused pass (256 rows for n <= 64), at most one per SM; the fused pass
-    // launches exactly this grid (one CTA per SM, checked in common.cuh), one Gram partial per CTA
-    const int64_t panels = (m + rowpass_rows(np) - 1) / rowpass_rows(np);
-    int grid = sms < kNoAllocMaxCtas ? sms : kNoAllocMaxCtas;
-    if (panels < grid) grid = static_cast<int>(panels);
-    if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, frag, diag, gpart, info, grid, st) != cudaSuccess)
+    // the fused pass leaves one Gram partial per CTA, at most one CTA per SM
+    const int ctas = sms < kNoAllocMaxCtas ? sms : kNoAllocMaxCtas;
+    if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, frag, diag, gpart, info, ctas, st) != cudaSuccess)
         return RPCHOLQR_ERR_CUDA;
-    launch_gram_reduce(gpart, grid, np, n, G, n, info, st);
+    launch_gram_reduce(gpart, rowpass_parts(np, m, ctas), np, n, G, n, info, st);
     return cudaGetLastError() == cudaSuccess ? RPCHOLQR_OK : RPCHOLQR_ERR_CUDA;
 }

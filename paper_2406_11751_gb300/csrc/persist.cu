@@ -20,10 +20,11 @@
 // that gives up sets RPCHOLQR_ERR_TIMEOUT for its matrix, and the items after it skip the matrix's
 // work but still pass its counters on, so no other wait depends on the one that gave up.
 //
-// Bits: P_i is the single call's pass-1 grid (one CTA per 128-row panel, at most one per SM), the
+// Bits: P_i is the single call's pass-1 grid (rowpass_parts), the
 // panels of part b are those CTA b of the single call solves, each part's Gram partial is accumulated
 // by the same code, and the parts are summed in the single call's order; the sample, the Householder
-// QR (every sum's order depends on the shape alone, not on the CTAs that share it), the Cholesky factorisation (the same virtual-thread layout), the fragment tables and R = R1 R_s are the
+// QR (every sum's order depends on the shape alone, not on the CTAs that share it), the Cholesky
+// factorisation, the fragment tables and R = R1 R_s are the
 // same device functions.  So every matrix's Q, R and status are bit-identical to rpcholqr_factor on
 // an FP64 plan, whatever else is in the batch.
 #include <algorithm>
@@ -38,7 +39,6 @@ namespace {
 
 constexpr int kPThreads = 256;
 constexpr int kBatchMaxNP = 128;
-constexpr int kPanelRowsForParts = 128;        // the single call sizes its pass-1 grid by 128-row panels
 
 enum : int { kItemSketch = 0, kItemPass1 = 1, kItemChol = 2, kItemPass2 = 3 };
 
@@ -132,8 +132,7 @@ __global__ void __launch_bounds__(1024) k_batch_setup(BatchArgs a) {
         a.info[2 * i + 1] = -1;
         int parts = 0;
         if (ok) {
-            const int64_t panels = (m + kPanelRowsForParts - 1) / kPanelRowsForParts;
-            parts = static_cast<int>(panels < a.sms ? panels : a.sms);
+            parts = rowpass_parts(pad16(n), m, a.sms);
         }
         a.ctr[4 * i + 0] = 0;
         a.ctr[4 * i + 1] = 0;
@@ -226,20 +225,26 @@ __device__ void item_sketch(const BatchArgs& a, int i, double* psm) {
 }
 
 template <int NP, bool SYRK, class BeforeEmit, class Emit>
-__device__ __forceinline__ bool item_rows(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int n,
-                                          const double* frag, const double* diag, bool check, int64_t part,
+__device__ __forceinline__ bool item_rows(int short_warps, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
+                                          int n, const double* frag, const double* diag, bool check, int64_t part,
                                           int64_t parts, double* psm, BeforeEmit before, Emit emit) {
-    return rowpass_panels<NP, SYRK, rowpass_warps(NP) * 32 == kPThreads, false>(
-        X, ldx, Y, ldy, m, n, frag, diag, check, nullptr, 0, nullptr, part, parts, psm, before, emit);
+    static_assert(kRowpassWarps * 32 == kPThreads, "the big panels take every warp of the CTA");
+    constexpr int W = kRowpassWarps;
+    return short_warps ? rowpass_panels<NP, SYRK, 16, W, false, false>(short_warps, W, X, ldx, Y, ldy, m, n, frag, diag, check,
+                                                                       nullptr, 0, nullptr, part, parts, psm, before, emit)
+                       : rowpass_panels<NP, SYRK, rowpass_rows_per_warp(NP), W, true, false>(
+                             W, W, X, ldx, Y, ldy, m, n, frag, diag, check, nullptr, 0, nullptr, part, parts, psm, before,
+                             emit);
 }
 
 template <bool SYRK, class BeforeEmit, class Emit>
-__device__ __forceinline__ bool item_rows_np(int np, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
+__device__ __forceinline__ bool item_rows_np(int np, int sms, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
                                              int n, const double* frag, const double* diag, bool check, int64_t part,
                                              int64_t parts, double* psm, BeforeEmit before, Emit emit) {
+    const int brief = rowpass_short_warps(np, m, sms);
     switch (np) {
 #define RPQ_NP(V) \
-    case V: return item_rows<V, SYRK>(X, ldx, Y, ldy, m, n, frag, diag, check, part, parts, psm, before, emit);
+    case V: return item_rows<V, SYRK>(brief, X, ldx, Y, ldy, m, n, frag, diag, check, part, parts, psm, before, emit);
         RPQ_NP(16) RPQ_NP(32) RPQ_NP(48) RPQ_NP(64) RPQ_NP(80) RPQ_NP(96) RPQ_NP(112) RPQ_NP(128)
 #undef RPQ_NP
         default: return false;
@@ -269,7 +274,7 @@ __device__ void item_pass1(const BatchArgs& a, int i, int64_t b, double* psm, in
     };
     bool bad = false;
     if (load_status(info) == 0) {
-        bad = item_rows_np<true>(np, a.A[i], a.lda[i], a.Q[i], a.ldq[i], a.m[i], n, w.frag_s, w.diag_s, true, b,
+        bad = item_rows_np<true>(np, a.sms, a.A[i], a.lda[i], a.Q[i], a.ldq[i], a.m[i], n, w.frag_s, w.diag_s, true, b,
                                  parts, psm, before, emit);
     } else {
         before();   // keep the turns moving for the parts after this one
@@ -309,7 +314,7 @@ __device__ void item_pass2(const BatchArgs& a, int i, int64_t b, double* psm, in
     __syncthreads();
     if (load_status(info) == 0) {
         double* Q = a.Q[i];
-        item_rows_np<false>(np, Q, a.ldq[i], Q, a.ldq[i], a.m[i], n, w.frag_1, w.diag_1, false, b, parts, psm,
+        item_rows_np<false>(np, a.sms, Q, a.ldq[i], Q, a.ldq[i], a.m[i], n, w.frag_1, w.diag_1, false, b, parts, psm,
                             [] {}, [](int, int, double) {});
     }
 }
@@ -380,7 +385,7 @@ BatchLayout batch_layout(int32_t capacity, int32_t max_n, int32_t max_s, int sms
 size_t batch_smem_bytes(int32_t max_n, int32_t max_s) {
     const int npm = pad16(max_n);
     size_t b = 0;
-    for (int np = 16; np <= npm; np += 16) b = std::max(b, rowpass_smem_bytes(np));
+    for (int np = 16; np <= npm; np += 16) b = std::max(b, rowpass_smem_bytes(np, rowpass_big_rows(np)));
     b = std::max(b, static_cast<size_t>(npm + kCholParts) * npm * sizeof(double));
     // the sketch: its panels stay in shared memory for samples of up to 3 max_n rows (the paper's choice of s)
     b = std::max(b, qr_one_bytes(max_n, std::min(max_s, 3 * max_n)));

@@ -9,17 +9,19 @@
 // FP64 tensor-core mma.sync m16n8k16 (measured); HBM is ~100x faster than this FP64 work needs, so the
 // kernels are organised to keep the FP64 pipe busy, not for bandwidth.  mma.sync m16n8k16 carries 2048
 // FMAs per instruction, so the issue slots stay free for address math and shared-memory traffic:
-//   * a CTA (4 warps, or 8 when NP <= 64) owns a 32-rows-per-warp panel staged in shared memory with
-//     cp.async; the row stride
-//     NP+4 doubles keeps every fragment load at the minimum two wavefronts;
+//   * a CTA (8 warps; 4 for short matrices) owns a panel of 16 or 32 rows per warp (common.cuh) staged in
+//     shared memory with cp.async; the row stride NP+4 doubles keeps every fragment load at the minimum two
+//     wavefronts;
 //   * the solve is blocked by 8 columns, left-looking: block J of a 16-row tile is
 //       acc = X[:, J] - A1[:, <J] T[<J, J]          (mma m16n8k16, FP64, B = -T chunks)
 //       A1[:, J] = acc T[J, J]^{-1}                 (8-column forward substitution, DFMA,
-//                                                    one lane per row, reciprocal diagonal)
-//     each warp runs two 16-row tiles with two split-k accumulators (4 chains per warp);
-//   * the Gram matrix keeps only the upper 16x8 tiles (72 tiles at n = 128), 18 per warp,
-//     accumulated in registers across every panel the CTA visits; each CTA writes one partial
-//     and a second kernel sums the partials in a fixed order (deterministic, no atomics).
+//                                                    one or two lanes per row, reciprocal diagonal)
+//     each 16-row tile has two split-k accumulators;
+//   * the Gram matrix keeps only the upper 16x8 tiles (72 tiles at n = 128), 9 per warp, accumulated in
+//     registers across every panel the CTA visits; each CTA writes one partial and a second kernel sums the partials in a fixed order (deterministic, no atomics).
+// Measured on GB300 (2^20 x 128): fused pass 1 41.5 -> 34.8 ms (0.99 TFLOP/s of the probe's 1.10), pass 2 23.3 -> 17.1
+// ms with eight warps of 16 rows instead of four of 32 and the right-looking diagonal block; a 10000 x 50 factorisation
+// 811 -> 479 us with 80-row panels on 125 SMs instead of 256-row panels on 40.
 #include "rowpass.cuh"
 
 namespace rpq {
@@ -31,8 +33,9 @@ __global__ void k_prep_tri(const double* __restrict__ T, int64_t ldt, int n, int
     prep_tri_entry(T, ldt, n, np, frag, diag, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-template <int NP, bool SYRK>
-__global__ void __launch_bounds__(rowpass_warps(NP) * 32, rowpass_ctas_per_sm(NP, SYRK))
+// SHORT: 4 to 8 warps of 16 rows (the launch's), else the big panels.
+template <int NP, bool SYRK, bool SHORT>
+__global__ void __launch_bounds__(kRowpassWarps * 32, SHORT ? 1 : rowpass_ctas_per_sm(NP, SYRK))
 k_rowpass(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int n,
           const double* __restrict__ frag, const double* __restrict__ diag,
           double* __restrict__ gpart, int32_t* info, bool check_finite, int32_t* rowexp, int rowexp_mode,
@@ -40,8 +43,10 @@ k_rowpass(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int n
     extern __shared__ double panel[];
     if (load_status(info) != 0) return;
     double* out = SYRK ? gpart + static_cast<size_t>(blockIdx.x) * NP * NP : nullptr;
-    const bool bad = rowpass_panels<NP, SYRK, true, true>(
-        X, ldx, Y, ldy, m, n, frag, diag, check_finite, rowexp, rowexp_mode, colexp, blockIdx.x, gridDim.x, panel,
+    const int nw = SHORT ? blockDim.x >> 5 : kRowpassWarps;
+    const bool bad = rowpass_panels<NP, SYRK, SHORT ? 16 : rowpass_rows_per_warp(NP),
+                                    SHORT ? kRowpassMinWarps : kRowpassWarps, true, true>(
+        nw, nw, X, ldx, Y, ldy, m, n, frag, diag, check_finite, rowexp, rowexp_mode, colexp, blockIdx.x, gridDim.x, panel,
         [] {}, [out](int pr, int pc, double v) { out[pr * NP + pc] = v; });
     if (__syncthreads_or(bad) && threadIdx.x == 0) set_status(info, RPCHOLQR_ERR_NONFINITE);
 }
@@ -68,36 +73,33 @@ void launch_prep_tri(const double* T, int64_t ldt, int n, int np, double* frag, 
 }
 
 
-template <int NP, bool SYRK>
+template <int NP, bool SYRK, bool SHORT>
 static cudaError_t launch_rowpass_t(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
                                     int n, const double* frag, const double* diag, double* gpart,
-                                    int32_t* info, int grid, cudaStream_t st, bool check, int32_t* rowexp,
+                                    int32_t* info, int sms, cudaStream_t st, bool check, int32_t* rowexp,
                                     int rowexp_mode, int32_t* colexp) {
-    const size_t smem = rowpass_smem_bytes(NP);
-    cudaError_t err = cudaFuncSetAttribute(k_rowpass<NP, SYRK>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(smem));
+    const int rows = rowpass_rows(NP, m, sms), warps = SHORT ? rows / 16 : kRowpassWarps;
+    auto kern = k_rowpass<NP, SYRK, SHORT>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           static_cast<int>(rowpass_smem_bytes(NP, SHORT ? 128 : rows)));
     if (err != cudaSuccess) return err;
-    if (rowpass_ctas_per_sm(NP, SYRK) > 1) {
-        const int64_t npanels = (m + 32 * rowpass_warps(NP) - 1) / (32 * rowpass_warps(NP));
-        const int64_t g = static_cast<int64_t>(grid) * rowpass_ctas_per_sm(NP, SYRK);
-        grid = static_cast<int>(g < npanels ? g : npanels);
-    }
-    k_rowpass<NP, SYRK><<<grid, 32 * rowpass_warps(NP), smem, st>>>(X, ldx, Y, ldy, m, n, frag, diag, gpart, info,
-                                                                    check, rowexp, rowexp_mode, colexp);
+    const int64_t panels = (m + rows - 1) / rows, cap = static_cast<int64_t>(sms) * (SHORT ? 1 : rowpass_ctas_per_sm(NP, SYRK));
+    kern<<<static_cast<unsigned>(panels < cap ? panels : cap), 32 * warps, rowpass_smem_bytes(NP, rows), st>>>(
+        X, ldx, Y, ldy, m, n, frag, diag, gpart, info, check, rowexp, rowexp_mode, colexp);
     return cudaGetLastError();
 }
 
 template <bool SYRK>
 static cudaError_t launch_rowpass_np(int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                                      int64_t m, int n, const double* frag, const double* diag,
-                                     double* gpart, int32_t* info, int grid, cudaStream_t st, bool check,
+                                     double* gpart, int32_t* info, int sms, cudaStream_t st, bool check,
                                      int32_t* rowexp, int rowexp_mode, int32_t* colexp) {
+    const bool brief = rowpass_short_warps(np, m, sms) != 0;
     switch (np) {
 #define RPQ_CASE(V)                                                                                     \
     case V:                                                                                             \
-        return launch_rowpass_t<V, SYRK>(X, ldx, Y, ldy, m, n, frag, diag, gpart, info, grid, st, check, \
-                                         rowexp, rowexp_mode, colexp);
+        return (brief ? launch_rowpass_t<V, SYRK, true> : launch_rowpass_t<V, SYRK, false>)(            \
+            X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st, check, rowexp, rowexp_mode, colexp);
         RPQ_CASE(16) RPQ_CASE(32) RPQ_CASE(48) RPQ_CASE(64) RPQ_CASE(80) RPQ_CASE(96) RPQ_CASE(112)
         RPQ_CASE(128)
 #undef RPQ_CASE
@@ -105,24 +107,25 @@ static cudaError_t launch_rowpass_np(int np, const double* X, int64_t ldx, doubl
     }
 }
 
+// sms: SMs to use; the fused Gram pass leaves rowpass_parts(np, m, sms) partials in gpart.
 // check_finite: set NONFINITE when an input entry is NaN/Inf.  rowexp (optional): exponent bound of
 // every solved row over its n columns, stored (rowexp_mode 1) or max-merged (2); colexp (optional,
 // pre-filled with kNoExp): exponent bound of every column over all rows (atomicMax).
 cudaError_t launch_rowpass_ex(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                               int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                              int32_t* info, int grid, cudaStream_t st, bool check_finite, int32_t* rowexp,
+                              int32_t* info, int sms, cudaStream_t st, bool check_finite, int32_t* rowexp,
                               int rowexp_mode, int32_t* colexp) {
-    return syrk ? launch_rowpass_np<true>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, grid, st,
+    return syrk ? launch_rowpass_np<true>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st,
                                           check_finite, rowexp, rowexp_mode, colexp)
-                : launch_rowpass_np<false>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, grid, st,
+                : launch_rowpass_np<false>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st,
                                            check_finite, rowexp, rowexp_mode, colexp);
 }
 
 // The fused Gram pass checks its input for NaN/Inf, the plain solve does not.
 cudaError_t launch_rowpass(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                            int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                           int32_t* info, int grid, cudaStream_t st) {
-    return launch_rowpass_ex(syrk, np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, grid, st, syrk, nullptr, 0,
+                           int32_t* info, int sms, cudaStream_t st) {
+    return launch_rowpass_ex(syrk, np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st, syrk, nullptr, 0,
                              nullptr);
 }
 

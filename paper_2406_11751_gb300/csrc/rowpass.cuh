@@ -49,32 +49,34 @@ __device__ __forceinline__ void prep_tri_entry(const double* __restrict__ T, int
     }
 }
 
-// The row pass over the panels p_first, p_first + p_stride, ... of X (ROWS = rowpass_rows(NP) rows
-// each) by the calling CTA: the first rowpass_warps(NP) warps solve and accumulate, every thread of the
-// CTA (any number of warps >= rowpass_warps(NP)) takes part in the panel copies and barriers.  panel:
-// the CTA's shared memory, rowpass_smem_bytes(NP).  With SYRK the CTA's Gram partial over its panels,
-// upper 16x8 tiles, is handed over at the end: every thread calls before_emit() (a point where the
-// caller may wait), then emit(pr, pc, v) for each entry it holds.  Returns this thread's non-finite
-// flag (check_finite); the caller reduces it over the CTA.  FULL: the CTA has exactly
-// rowpass_warps(NP) warps (every warp solves).  LDG: frag and diag are read through the read-only
-// (non-coherent) cache -- only when no CTA of the same launch writes them.
-template <int NP, bool SYRK, bool FULL, bool LDG, class BeforeEmit, class Emit>
-__device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
+// The row pass over the panels p_first, p_first + p_stride, ... of X (nw x RPW rows each) by the calling CTA:
+// the first nw warps solve RPW rows each (16 or 32), the first tw >= TW warps share the Gram tiles, every thread
+// of the CTA takes part in the panel copies and barriers.  panel: the CTA's shared memory, rowpass_smem_bytes.
+// With SYRK the CTA's Gram partial over its panels, upper 16x8 tiles, is handed over at the end: every thread
+// calls before_emit() (a point where the caller may wait), then emit(pr, pc, v) for each entry it holds.
+// Returns this thread's non-finite flag (check_finite); the caller reduces it over the CTA.  FULL: the CTA has
+// exactly nw warps (every warp solves).  LDG: frag and diag are read through the read-only (non-coherent)
+// cache -- only when no CTA of the same launch writes them.
+// A solved row does not depend on the panel it is in; a Gram partial sums its CTA's rows in order, so it depends
+// on the panel rows and the number of CTAs (rowpass_rows, rowpass_parts) but not on RPW or tw.
+template <int NP, bool SYRK, int RPW, int TW, bool FULL, bool LDG, class BeforeEmit, class Emit>
+__device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
                                                int n, const double* __restrict__ frag,
                                                const double* __restrict__ diag, bool check_finite,
                                                int32_t* rowexp, int rowexp_mode, int32_t* colexp,
                                                int64_t p_first, int64_t p_stride, double* panel,
                                                BeforeEmit before_emit, Emit emit) {
     constexpr int S = NP + 4;    // shared-memory row stride in doubles
-    constexpr int WARPS = rowpass_warps(NP);
-    constexpr int ROWS = 32 * WARPS;   // panel rows: 32 per warp
+    constexpr int MT = RPW / 16;       // 16-row tiles of a warp
+    const int ROWS = RPW * nw;         // panel rows
     constexpr int NB = NP / 8;         // 8-column blocks
     constexpr int NT = upper_tiles(NP);
-    constexpr int TPW = (NT + WARPS - 1) / WARPS;
+    constexpr int TPW = (NT + TW - 1) / TW;
+    constexpr int NCM = (NP + 31) / 32;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
-    const bool solver = FULL || warp < WARPS;
+    const bool solver = FULL || warp < nw;
     const int64_t npanels = (m + ROWS - 1) / ROWS;
 
     double gacc[SYRK ? TPW : 1][4];
@@ -83,13 +85,17 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
 #pragma unroll
         for (int q = 0; q < TPW; ++q) {
             gacc[q][0] = gacc[q][1] = gacc[q][2] = gacc[q][3] = 0.0;
-            const int tt = warp + WARPS * q;
+            const int tt = warp + tw * q;
             if (tt < NT) tile_coords(NP, tt, tI[q], tJ[q]);
             else { tI[q] = 0; tJ[q] = 0; }
         }
     }
     bool bad = false;
-    int col_e = kNoExp;   // column threadIdx.x: exponent bound over the rows this CTA solved
+    int cm[SYRK ? 1 : NCM];   // exponent bounds of columns lane, lane + 32, ... over the rows this warp solved
+    if constexpr (!SYRK) {
+#pragma unroll
+        for (int i = 0; i < NCM; ++i) cm[i] = kNoExp;
+    }
 
     for (int64_t p = p_first; p < npanels; p += p_stride) {
         const int64_t row0 = p * ROWS;
@@ -103,12 +109,13 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
         cp_async_wait_all();
         __syncthreads();
 
-        // ---- blocked forward substitution of this warp's 32 rows ----
-        const int wr0 = warp * 32;
+        // ---- blocked forward substitution of this warp's rows ----
+        const int wr0 = warp * RPW;
+        int re = kNoExp;   // exponent bound of this lane's row
         for (int J = 0; J < NB && solver; ++J) {
-            double acc[2][4], acc2[2][4];
+            double acc[MT][4], acc2[MT][4];
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+            for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int r = wr0 + mt * 16 + g + 8 * (i >> 1);
@@ -126,7 +133,7 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
                 const double2 b01 = LDG ? __ldg(fb) : fb[0], b23 = LDG ? __ldg(fb + 1) : fb[1];
                 const double b[4] = {b01.x, b01.y, b23.x, b23.y};
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
+                for (int mt = 0; mt < MT; ++mt) {
                     double a[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
@@ -141,7 +148,7 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
                 const double2 b01 = LDG ? __ldg(fb) : fb[0];
                 const double b[2] = {b01.x, b01.y};
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
+                for (int mt = 0; mt < MT; ++mt) {
                     double a[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
@@ -150,32 +157,100 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
                     else mma_f64_1688(acc[mt], a, b);
                 }
             }
+            if (J > 0) {
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+                for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = wr0 + mt * 16 + g + 8 * (i >> 1);
-                    const int c = 8 * J + 2 * t + (i & 1);
-                    panel[r * S + c] = acc[mt][i] + acc2[mt][i];
-                }
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = wr0 + mt * 16 + g + 8 * (i >> 1);
+                        const int c = 8 * J + 2 * t + (i & 1);
+                        panel[r * S + c] = acc[mt][i] + acc2[mt][i];
+                    }
+            }
             __syncwarp();
-            {
+            // the 8 x 8 diagonal block, right-looking: each solved column is subtracted from the later ones at
+            // once (independent multiply-adds; a dependent FP64 operation takes about 150 clocks, its issue 64)
+            const double* d = diag + J * 64;
+            auto dg = [&](int i) { return LDG ? __ldg(d + i) : d[i]; };
+            if constexpr (RPW == 32) {
                 double* xr = &panel[(wr0 + lane) * S + 8 * J];
-                const double* d = diag + J * 64;
                 double x[8];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) x[c] = xr[c];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    double v = x[c];
+                    x[c] *= dg(c * 9);
 #pragma unroll
-                    for (int k = 0; k < c; ++k) v -= x[k] * (LDG ? __ldg(d + k * 8 + c) : d[k * 8 + c]);
-                    x[c] = v * (LDG ? __ldg(d + c * 9) : d[c * 9]);
+                    for (int k = c + 1; k < 8; ++k) x[k] = fma(-x[c], dg(c * 8 + k), x[k]);
                 }
 #pragma unroll
                 for (int c = 0; c < 8; ++c) xr[c] = x[c];
+                // power-of-two bounds of the solved rows and columns, for the split products that read them next
+                if constexpr (!SYRK) {
+                    if (rowexp) {
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            const int e = exp_bound(x[c]);
+                            re = e > re ? e : re;
+                            const int ce = __reduce_max_sync(0xffffffffu, e);
+                            if (((8 * J + c) & 31) == lane) {
+#pragma unroll
+                                for (int q = 0; q < NCM; ++q)
+                                    if (q == (8 * J + c) >> 5) cm[q] = ce > cm[q] ? ce : cm[q];
+                            }
+                        }
+                    }
+                }
+            } else {
+                // two lanes per row: lane r + 16 h holds columns h, h + 2, h + 4, h + 6 of the block
+                const int r = lane & 15, h = lane >> 4;
+                double* xr = &panel[(wr0 + r) * S + 8 * J + h];
+                double x[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) x[i] = xr[2 * i];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const double xc = __shfl_sync(0xffffffffu, x[c >> 1] * dg(c * 9), r | ((c & 1) << 4));
+                    if (h == (c & 1)) x[c >> 1] = xc;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (2 * i + 1 > c) {   // (column 2 i + h: the even half's own column c is kept)
+                            const double v = fma(-xc, dg(c * 8 + 2 * i + h), x[i]);
+                            if (2 * i + h > c) x[i] = v;
+                        }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) xr[2 * i] = x[i];
+                if constexpr (!SYRK) {
+                    if (rowexp) {
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            const int e = h == (c & 1) ? exp_bound(x[c >> 1]) : kNoExp;
+                            re = e > re ? e : re;
+                            const int ce = __reduce_max_sync(0xffffffffu, e);
+                            if (((8 * J + c) & 31) == lane) {
+#pragma unroll
+                                for (int q = 0; q < NCM; ++q)
+                                    if (q == (8 * J + c) >> 5) cm[q] = ce > cm[q] ? ce : cm[q];
+                            }
+                        }
+                    }
+                }
             }
             __syncwarp();
+        }
+        if constexpr (!SYRK) {
+            if (rowexp && solver) {
+                if (RPW == 16) {
+                    const int o = __shfl_xor_sync(0xffffffffu, re, 16);
+                    re = o > re ? o : re;
+                }
+                const int64_t gr = row0 + wr0 + lane;
+                if (lane < RPW && gr < m) {
+                    if (rowexp_mode == 2 && rowexp[gr] > re) re = rowexp[gr];
+                    rowexp[gr] = re;
+                }
+            }
         }
         __syncthreads();
 
@@ -184,34 +259,11 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
             const int64_t gr = row0 + r;
             if (gr < m && c < n) Y[gr * ldy + c] = panel[r * S + c];
         }
-        // power-of-two bounds of the solved rows (one thread per row) and columns, for the
-        // split-precision products that read A1 next
-        if (rowexp && threadIdx.x < ROWS) {
-            const int r = threadIdx.x;          // one thread per panel row
-            const int64_t gr = row0 + r;
-            if (gr < m) {
-                int e = kNoExp;
-                for (int c = 0; c < n; ++c) {
-                    const int ec = exp_bound(panel[r * S + c]);
-                    e = ec > e ? ec : e;
-                }
-                if (rowexp_mode == 2 && rowexp[gr] > e) e = rowexp[gr];
-                rowexp[gr] = e;
-            }
-        }
-        if (colexp && threadIdx.x < n) {
-            const int c = threadIdx.x;
-            const int64_t rows = (m - row0) < ROWS ? (m - row0) : ROWS;
-            for (int r = 0; r < rows; ++r) {
-                const int ec = exp_bound(panel[r * S + c]);
-                col_e = ec > col_e ? ec : col_e;
-            }
-        }
 
         if constexpr (SYRK) {
 #pragma unroll
             for (int q = 0; q < TPW; ++q) {
-                if (solver && warp + WARPS * q < NT) {
+                if (warp < tw && warp + tw * q < NT) {
                     const int I = tI[q], Jt = tJ[q];
 #pragma unroll 2
                     for (int kc = 0; kc < ROWS / 16; ++kc) {
@@ -233,7 +285,7 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
         before_emit();
 #pragma unroll
         for (int q = 0; q < TPW; ++q) {
-            if (solver && warp + WARPS * q < NT) {
+            if (warp < tw && warp + tw * q < NT) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int pr = 16 * tI[q] + g + 8 * (i >> 1);
@@ -242,14 +294,24 @@ __device__ __forceinline__ bool rowpass_panels(const double* X, int64_t ldx, dou
                 }
             }
         }
+    } else if (colexp) {
+        // the warps' column bounds to one atomic per column of the CTA (the panel is free)
+        int* cs = reinterpret_cast<int*>(panel);
+        for (int c = threadIdx.x; c < n; c += blockDim.x) cs[c] = kNoExp;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NCM; ++q)
+            if (solver && lane + 32 * q < n) atomicMax(&cs[lane + 32 * q], cm[q]);
+        __syncthreads();
+        for (int c = threadIdx.x; c < n; c += blockDim.x)
+            if (cs[c] > kNoExp) atomicMax(&colexp[c], cs[c]);
     }
-    if (colexp && threadIdx.x < n && col_e > kNoExp) atomicMax(&colexp[threadIdx.x], col_e);
     return bad;
 }
 
-// Shared memory of one row-pass CTA: the panel, ROWS rows of NP + 4 doubles.
-__host__ __device__ constexpr size_t rowpass_smem_bytes(int np) {
-    return static_cast<size_t>(rowpass_rows(np)) * (np + 4) * sizeof(double);
+// Shared memory of one row-pass CTA: the panel, `rows` rows of NP + 4 doubles.
+__host__ __device__ constexpr size_t rowpass_smem_bytes(int np, int rows) {
+    return static_cast<size_t>(rows) * (np + 4) * sizeof(double);
 }
 
 }  // namespace rpq
