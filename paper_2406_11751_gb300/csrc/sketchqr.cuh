@@ -147,8 +147,9 @@ __device__ __forceinline__ void qr_scalars(double alpha, double x, double& nrm, 
         const unsigned long long S = (1ull << 60) + static_cast<unsigned long long>(F + ((fh * fh) >> 20));
         const unsigned long long G = __umul64hi(S << 3, R);                                       // Q63, in [1/8, 1]
         const int lz = __clzll(static_cast<long long>(G));
-        g = __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(1022 - lz - k) << 52) +
-                                                        (((G << lz) + 1024) >> 11)));
+        const unsigned long long M = G << lz;   // rounded below without leaving 64 bits: M may be 2^64 - 1
+        g = __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(1022 - lz - k) << 52) + (M >> 11) +
+                                                        ((M >> 10) & 1)));
     } else {
         nrm = sqrt(x);
         g = 1.0 / (nrm * (nrm + fabs(alpha)));

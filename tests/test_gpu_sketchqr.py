@@ -33,6 +33,21 @@ def test_sketch_r_is_the_triangular_factor(lib, s, n, kappa):
     assert np.max(np.abs(R.T @ R - A.T @ A) / np.outer(c, c)) <= 2 * (s + n) * U
 
 
+@pytest.mark.parametrize("shift", [1, 7, 35])   # coprime to the row count: distinct rows
+def test_powers_of_two_are_exact(lib, shift):
+    # columns +-2^e e_i, permuted: every norm, square root and reciprocal is a power of two (the ends of the fixed-point
+    # ranges), so R is exactly the diagonal of the column scales, to the last bit
+    s, n = 96, 40
+    scale = 2.0 ** ((np.arange(n) * 7) % 23 - 11)
+    A = np.zeros((s, n))
+    A[(np.arange(n) * shift + 5) % s, np.arange(n)] = np.where(np.arange(n) % 3, scale, -scale)
+    plan = lib.rpcholqr_plan_create(0, s, n, s)
+    Rs, info = lib.rpcholqr_sketch_r_from_sample(plan, torch.from_numpy(A).cuda())
+    assert info.cpu().tolist() == [0, -1]
+    assert np.array_equal(Rs.cpu().numpy(), np.diag(scale))
+    plan.close()
+
+
 @pytest.mark.parametrize("m,n,s", [(2000, 40, 120), (2000, 40, 2000), (3000, 33, 33), (700, 128, 640)])
 def test_one_cta_gives_the_cluster_bits(lib, m, n, s):
     A = torch.from_numpy(_sample(m, n, 1e6, m + n)).cuda()
