@@ -73,8 +73,9 @@ k_gemm_sub_fp64(const double* __restrict__ X, int64_t ldx, const double* __restr
 
 // Partials of G = X^T X: block (tile, range) accumulates the 64 x 64 tile (I, J), I <= J, of the rows
 // [range*rows_per, ...) and writes gpart[range][p][q] (ld np) for its tile.  Rows staged 32 at a time.
-// Two-level sums: the mma accumulators take 8192 rows, then are added into a running total and
-// cleared, so a range of R rows accumulates rounding over ~8192 + R/8192 terms instead of R.
+// Two-level sums: the mma accumulators take 512 rows, then are added into a running total and cleared, so a range
+// of R rows accumulates rounding over 512 / 16 + R / 512 additions instead of R / 16 (sixteen additions a thread for
+// every 128 mma; the Gram matrix's error enters ||Q^T Q - I|| times kappa(A_1)^2).
 __global__ void __launch_bounds__(256, 2)
 k_syrk_fp64(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np, int64_t rows_per,
             double* __restrict__ gpart, const int32_t* info) {
@@ -98,8 +99,8 @@ k_syrk_fp64(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np,
         for (int i = 0; i < 4; ++i) acc[j][i] = tot[j][i] = 0.0;
     int chunk = 0;
     for (int64_t k0 = rb; k0 < re; k0 += 32) {
-        if (++chunk == 256) {
-            chunk = 0;
+        if (++chunk > 16) {
+            chunk = 1;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
