@@ -26,13 +26,16 @@ size_t householder_smem_bytes(int s, int n);
 int householder_launches(int n);
 size_t householder_ws_bytes(int np);
 // smallfactor.cu
-cudaError_t launch_cholesky(const double* G, int64_t ldg, int n, int np, double* R, double* R_user,
+cudaError_t launch_cholesky(const double* G, int64_t ldg, int n, int np, double* R, double* W, double* D, double* R_user,
                             int32_t* info, cudaStream_t st);
+int cholesky_launches(int n);
 void launch_triu_mul(const double* R1, int64_t ld1, const double* Rs, int64_t lds, int n, double* R,
                      int64_t ldr, const int32_t* info, cudaStream_t st);
 // rowpass.cu
 void launch_prep_tri(const double* T, int64_t ldt, int n, int np, double* frag, double* diag,
                      const int32_t* info, cudaStream_t st);
+void launch_prep_blocks(const double* T, int64_t ldt, int n, int blk, double* frag, double* diag, const int32_t* info,
+                        cudaStream_t st);
 cudaError_t launch_rowpass(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                            int64_t m, int n, const double* frag, const double* diag, double* gpart,
                            int32_t* info, int sms, cudaStream_t st);
@@ -45,10 +48,6 @@ cudaError_t launch_rowpass_ex(bool syrk, int np, const double* X, int64_t ldx, d
 void launch_fill_noexp(int32_t* p, int n, cudaStream_t st);
 // probe.cu
 cudaError_t run_fp64_mma_probe(int iters, double* flops_per_s);
-// smallfactor.cu
-void launch_fill_identity(double* W, int np, const int32_t* info, cudaStream_t st);
-void launch_triu_inv(const double* T, int64_t ldt, int n, int np, double* W, const int32_t* info,
-                     cudaStream_t st);
 // ozaki.cu
 size_t ozaki_yblocks_bytes(int K, int N);
 int32_t ozaki_no_exp();
@@ -112,7 +111,7 @@ cudaError_t launch_dct_sample(const double* A, int64_t m, int n, int64_t lda, in
 cudaError_t launch_dct_sample_f32(const float* A, int64_t m, int n, int64_t lda, int s, uint64_t seed, void* T,
                                   int8_t* sgn, int64_t* idx, double* As, int64_t lds, int np, int32_t* info,
                                   cudaStream_t st, bool scale_sample);
-void launch_pass2_gate(const double* R1, const double* W, int n, int np, double tau, const int32_t* info,
+void launch_pass2_gate(const double* R1, const double* W, int n, int np, double tau, double* part, const int32_t* info,
                        int32_t* gates, cudaStream_t st);
 void launch_gate_merge(int32_t* info, const int32_t* gates, cudaStream_t st);
 void launch_scholqr3_shift(double* G, int64_t ldg, int n, int64_t m, const int32_t* info, cudaStream_t st);
@@ -152,7 +151,6 @@ struct TuneEntry {
 };
 constexpr int64_t kMaxBatchCount = 1 << 16;   // matrices one rpcholqr_factor_batched call may take
 constexpr int32_t kMaxNF32 = 512;              // widest FP32 plan (the FP32 row solve stages T in shared memory)
-constexpr int kTriuInvMaxN = 512;              // widest R1^{-1} of the warp-per-column kernel
 
 struct rpcholqr_plan_s {
     int device = 0;
@@ -925,12 +923,8 @@ static rpcholqr_status ozaki_gemm_internal(rpcholqr_plan p, bool sub, const doub
 // one ragged) gets frag + 4096 J and diag + 512 J.
 static void prep_blocks(rpcholqr_plan_s* p, const double* T, int64_t ldt, int n, double* frag, double* diag,
                         const int32_t* info, cudaStream_t st, int blk = kBlk) {
-    for (int J = 0; J * blk < n; ++J) {
-        const int nj = n - J * blk < blk ? n - J * blk : blk;
-        launch_prep_tri(T + static_cast<int64_t>(J) * blk * ldt + J * blk, ldt, nj, pad16(nj),
-                        frag + J * blk * blk, diag + J * (blk / 8) * 64, info, st);
-        ++p->launches;
-    }
+    launch_prep_blocks(T, ldt, n, blk, frag, diag, info, st);
+    ++p->launches;
 }
 
 // Right-looking blocked row solve for the split mode, Y = X T^{-1}, two-level: over kSplitBlk-column
@@ -1159,22 +1153,6 @@ static rpcholqr_status solve_blocked(rpcholqr_plan_s* p, const double* X, int64_
     return check_launch();
 }
 
-// W = R1^{-1} (np x np, identity-padded) for the split second pass: the warp-per-column back
-// substitution up to kTriuInvMaxN columns; wider, the FP64 blocked row solve of the identity's first n
-// rows by R1 (row i of W solves w_i^T R1 = e_i^T), with R1's diagonal-block tables in frag_1 / diag_1.
-static rpcholqr_status inverse_r1(rpcholqr_plan_s* p, int n, int np, int32_t* info, cudaStream_t st) {
-    if (n <= kTriuInvMaxN) {
-        launch_triu_inv(p->R1, np, n, np, p->W, info, st);
-        ++p->launches;
-        return check_launch();
-    }
-    launch_fill_identity(p->W, np, info, st);
-    ++p->launches;
-    prep_blocks(p, p->R1, np, n, p->frag_1, p->diag_1, info, st);
-    return solve_blocked(p, p->W, np, p->R1, np, n, n, p->W, np, p->frag_1, p->diag_1, false, false, info, st,
-                         nullptr, false);
-}
-
 // Row-range partials of G = X^T X in FP64 (n > 128) and their fixed-order sum into G (ld ldg).
 static rpcholqr_status gram_fp64_wide(rpcholqr_plan_s* p, const double* X, int64_t ldx, int64_t m, int n, double* G,
                                int64_t ldg, int32_t* info, cudaStream_t st) {
@@ -1375,12 +1353,12 @@ static rpcholqr_status factor_split(rpcholqr_plan p, const double* A, int64_t m,
     pm.mark(RPCHOLQR_PHASE_CHOLESKY);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_CHOLESKY, static_cast<double>(n) * n * n / 3.0);
-        if (launch_cholesky(p->G, np, n, np, p->R1, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
+        if (launch_cholesky(p->G, np, n, np, p->R1, p->W, p->qws, nullptr, info, st) != cudaSuccess)
+            return RPCHOLQR_ERR_CUDA;
     }
-    ++p->launches;
+    p->launches += cholesky_launches(n) + 1;
     pm.mark(RPCHOLQR_PHASE_PREP_R1);
-    if ((rc = inverse_r1(p, n, np, info, st)) != RPCHOLQR_OK) return rc;
-    launch_pass2_gate(p->R1, p->W, n, np, kSplitPass2Tau, info, p->gates, st);
+    launch_pass2_gate(p->R1, p->W, n, np, kSplitPass2Tau, p->qws, info, p->gates, st);
     ++p->launches;
     pm.mark(RPCHOLQR_PHASE_PASS2);
     // Q = A1 R1^{-1}: the split product with the explicit inverse when A1 is well conditioned, else the
@@ -1440,9 +1418,10 @@ rpcholqr_status rpcholqr_factor(rpcholqr_plan p, const double* A, int64_t m, int
     pm.mark(RPCHOLQR_PHASE_CHOLESKY);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_CHOLESKY, static_cast<double>(n) * n * n / 3.0);
-        if (launch_cholesky(p->G, np, n, np, p->R1, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
+        if (launch_cholesky(p->G, np, n, np, p->R1, nullptr, p->qws, nullptr, info, st) != cudaSuccess)
+            return RPCHOLQR_ERR_CUDA;
     }
-    ++p->launches;
+    p->launches += cholesky_launches(n);
     if ((rc = solve_internal(p, Q, m, n, ldq, p->R1, np, Q, ldq, info, st, &pm)) != RPCHOLQR_OK) return rc;
     pm.mark(RPCHOLQR_PHASE_RECOVER_R);
     launch_triu_mul(p->R1, np, p->Rs, np, n, R, n, info, st);
@@ -1521,9 +1500,10 @@ rpcholqr_status rpcholqr_factor_f32(rpcholqr_plan p, const float* A, int64_t m, 
     pm.mark(RPCHOLQR_PHASE_CHOLESKY);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_CHOLESKY, static_cast<double>(n) * n * n / 3.0);
-        if (launch_cholesky(p->G, np, n, np, p->R1, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
+        if (launch_cholesky(p->G, np, n, np, p->R1, nullptr, p->qws, nullptr, info, st) != cudaSuccess)
+            return RPCHOLQR_ERR_CUDA;
     }
-    ++p->launches;
+    p->launches += cholesky_launches(n);
     pm.mark(RPCHOLQR_PHASE_PREP_R1);
     launch_prep_f32(p->R1, np, n, p->T32, p->rinv32, RPCHOLQR_ERR_NOT_SPD, info, st);
     ++p->launches;
@@ -1702,10 +1682,11 @@ static rpcholqr_status factor_host_split(rpcholqr_plan p, const double* A, int64
     if ((rc = ozaki_gram_internal(p, p->A1, m, n, ld1, p->G, np, info, st, true)) != RPCHOLQR_OK) return rc;
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_CHOLESKY, static_cast<double>(n) * n * n / 3.0);
-        if (launch_cholesky(p->G, np, n, np, p->R1, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
+        if (launch_cholesky(p->G, np, n, np, p->R1, p->W, p->qws, nullptr, info, st) != cudaSuccess)
+            return RPCHOLQR_ERR_CUDA;
     }
-    if ((rc = inverse_r1(p, n, np, info, st)) != RPCHOLQR_OK) return rc;
-    launch_pass2_gate(p->R1, p->W, n, np, kSplitPass2Tau, info, p->gates, st);
+    p->launches += cholesky_launches(n) + 1;
+    launch_pass2_gate(p->R1, p->W, n, np, kSplitPass2Tau, p->qws, info, p->gates, st);
     p->launches += 2;
     // pass 2 block by block; each block of Q goes back while the next is computed
     for (int c = 0; c < nchunks; ++c) {
@@ -1820,8 +1801,8 @@ rpcholqr_status rpcholqr_cholesky(rpcholqr_plan p, const double* G, int32_t n, d
     rpcholqr_status rc = reset_info(info, st);
     if (rc != RPCHOLQR_OK) return rc;
     const int np = pad_np(n);
-    return launch_cholesky(G, n, n, np, p->R1, R1, info, st) == cudaSuccess ? RPCHOLQR_OK
-                                                                             : RPCHOLQR_ERR_CUDA;
+    return launch_cholesky(G, n, n, np, p->R1, nullptr, p->qws, R1, info, st) == cudaSuccess ? RPCHOLQR_OK
+                                                                                               : RPCHOLQR_ERR_CUDA;
 }
 
 rpcholqr_status rpcholqr_solve_rows(rpcholqr_plan p, const double* X, int64_t m, int32_t n, int64_t ldx,
@@ -1901,8 +1882,9 @@ static rpcholqr_status cholqr_step(rpcholqr_plan p, const double* X, int64_t m, 
             launch_scholqr3_shift(p->G, np, n, m, info, st);
             ++p->launches;
         }
-        if (launch_cholesky(p->G, np, n, np, R_out, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
-        ++p->launches;
+        if (launch_cholesky(p->G, np, n, np, R_out, nullptr, p->qws, nullptr, info, st) != cudaSuccess)
+            return RPCHOLQR_ERR_CUDA;
+        p->launches += cholesky_launches(n);
         return solve_internal(p, X, m, n, ldx, R_out, np, Q, ldq, info, st, nullptr);
     }
     launch_prep_tri(nullptr, 0, 0, np, p->frag_s, p->diag_s, info, st);   // identity preconditioner
@@ -1914,8 +1896,9 @@ static rpcholqr_status cholqr_step(rpcholqr_plan p, const double* X, int64_t m, 
         launch_scholqr3_shift(p->G, np, n, m, info, st);
         ++p->launches;
     }
-    if (launch_cholesky(p->G, np, n, np, R_out, nullptr, info, st) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
-    p->launches += 4;
+    if (launch_cholesky(p->G, np, n, np, R_out, nullptr, p->qws, nullptr, info, st) != cudaSuccess)
+        return RPCHOLQR_ERR_CUDA;
+    p->launches += 3 + cholesky_launches(n);
     return solve_internal(p, Q, m, n, ldq, R_out, np, Q, ldq, info, st, nullptr);
 }
 

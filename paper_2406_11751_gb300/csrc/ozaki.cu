@@ -409,12 +409,20 @@ __global__ void __launch_bounds__(256) k_ozaki_slice_cols(const double* __restri
     const int tn = blockIdx.x, kw = blockIdx.y, nkw = gridDim.y;
     const int q = threadIdx.x & 63, c = threadIdx.x >> 6;   // 64 columns x 4 chunks of 8 rows
     const int col = tn * kTileN + q;
+    // the column's bound over all K rows: a quarter of them per chunk group, eight loads in flight
+    __shared__ int red[4][kTileN];
     int E = kNoExp;
-    if (col < N)
-        for (int k = 0; k < K; ++k) {
+    if (col < N) {
+#pragma unroll 8
+        for (int k = c; k < K; k += 4) {
             const int e = exp_bound(Y[static_cast<int64_t>(k) * ldy + col]);
             E = e > E ? e : E;
         }
+    }
+    red[c][q] = E;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) E = red[i][q] > E ? red[i][q] : E;
     if (kw == 0 && c == 0 && col < N) yexp[col] = E;
     double x[8];
 #pragma unroll

@@ -291,7 +291,7 @@ __device__ void item_chol(const BatchArgs& a, int i, double* psm, int* ok_s) {
     if (!cta_wait_geq(&a.ctr[4 * i + 1], parts, a.spin, ok_s, a.queue + 2) && threadIdx.x == 0)
         set_status(info, RPCHOLQR_ERR_TIMEOUT);
     __syncthreads();
-    if (load_status(info) == 0 && cholesky_small<kPThreads>(w.G, np, n, np, w.R1, nullptr, info, psm)) {
+    if (load_status(info) == 0 && cholesky_one_cta<kPThreads>(w.G, np, n, np, w.R1, info, *reinterpret_cast<CholShared*>(psm))) {
         __syncthreads();
         for (int e = threadIdx.x; e < np * np + (np / 8) * 64; e += kPThreads)
             prep_tri_entry(w.R1, np, n, np, w.frag_1, w.diag_1, e);
@@ -386,7 +386,7 @@ size_t batch_smem_bytes(int32_t max_n, int32_t max_s) {
     const int npm = pad16(max_n);
     size_t b = 0;
     for (int np = 16; np <= npm; np += 16) b = std::max(b, rowpass_smem_bytes(np, rowpass_big_rows(np)));
-    b = std::max(b, static_cast<size_t>(npm + kCholParts) * npm * sizeof(double));
+    b = std::max(b, sizeof(CholShared));
     // the sketch: its panels stay in shared memory for samples of up to 3 max_n rows (the paper's choice of s)
     b = std::max(b, qr_one_bytes(max_n, std::min(max_s, 3 * max_n)));
     b = std::max(b, static_cast<size_t>(max_s) * sizeof(int64_t));

@@ -59,8 +59,17 @@ __global__ void k_gram_reduce(const double* __restrict__ gpart, int nparts, int 
     if (e >= n * n) return;
     const int p = e / n, q = e - p * n;
     if (q < p) return;
+    const double* gp = gpart + static_cast<int64_t>(p) * np + q;
     double sum = 0.0;
-    for (int b = 0; b < nparts; ++b) sum += gpart[static_cast<size_t>(b) * np * np + p * np + q];
+    int b = 0;
+    for (; b + 15 < nparts; b += 16) {   // sixteen loads in flight, summed in order
+        double v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = gp[static_cast<size_t>(b + u) * np * np];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) sum += v[u];
+    }
+    for (; b < nparts; ++b) sum += gp[static_cast<size_t>(b) * np * np];
     G[static_cast<int64_t>(p) * ldg + q] = sum;
     G[static_cast<int64_t>(q) * ldg + p] = sum;
 }
@@ -72,6 +81,21 @@ void launch_prep_tri(const double* T, int64_t ldt, int n, int np, double* frag, 
     k_prep_tri<<<(total + 255) / 256, 256, 0, st>>>(T, ldt, n, np, frag, diag, info);
 }
 
+
+// The tables of every blk x blk diagonal block of T (n x n) at once: block J's at frag + J blk^2 and diag + J 8 blk, of
+// the block padded to a multiple of 16 (the last one may be narrower).
+__global__ void k_prep_blocks(const double* __restrict__ T, int64_t ldt, int n, int blk, double* __restrict__ frag,
+                              double* __restrict__ diag, const int32_t* info) {
+    if (info && load_status(info) != 0) return;
+    const int J = blockIdx.y, nj = n - J * blk < blk ? n - J * blk : blk;
+    prep_tri_entry(T + static_cast<int64_t>(J) * blk * ldt + J * blk, ldt, nj, pad16(nj), frag + static_cast<size_t>(J) * blk * blk,
+                   diag + static_cast<size_t>(J) * blk * 8, blockIdx.x * blockDim.x + threadIdx.x);
+}
+void launch_prep_blocks(const double* T, int64_t ldt, int n, int blk, double* frag, double* diag, const int32_t* info,
+                        cudaStream_t st) {
+    k_prep_blocks<<<dim3((blk * blk + 8 * blk + 255) / 256, (n + blk - 1) / blk), 256, 0, st>>>(T, ldt, n, blk, frag, diag,
+                                                                                             info);
+}
 
 template <int NP, bool SYRK, bool SHORT>
 static cudaError_t launch_rowpass_t(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
