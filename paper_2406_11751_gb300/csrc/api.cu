@@ -84,7 +84,7 @@ int f32_pad(int n);
 void launch_prep_f32(const double* T, int64_t ldt, int n, float* T32, float* rinv32, int fail_status,
                      int32_t* info, cudaStream_t st);
 cudaError_t launch_rowsolve_f32(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, int n,
-                                const float* T32, const float* rinv32, int32_t* info, bool check_finite,
+                                const float* T32, const float* rinv32, int32_t* info, bool check_finite, int sms,
                                 cudaStream_t st);
 int launch_syrk_f32(const float* X, int64_t ldx, int64_t m, int n, int max_ranges, double* gpart,
                     const int32_t* info, cudaStream_t st);
@@ -1486,7 +1486,7 @@ rpcholqr_status rpcholqr_factor_f32(rpcholqr_plan p, const float* A, int64_t m, 
     launch_prep_f32(p->Rs, np, n, p->T32, p->rinv32, RPCHOLQR_ERR_SINGULAR_SKETCH, info, st);
     ++p->launches;
     pm.mark(RPCHOLQR_PHASE_PASS1);
-    if (launch_rowsolve_f32(A, lda, Q, ldq, m, n, p->T32, p->rinv32, info, true, st) != cudaSuccess)
+    if (launch_rowsolve_f32(A, lda, Q, ldq, m, n, p->T32, p->rinv32, info, true, p->grid, st) != cudaSuccess)
         return RPCHOLQR_ERR_CUDA;
     ++p->launches;
     pm.mark(RPCHOLQR_PHASE_PASS1_UPDATE);
@@ -1508,7 +1508,7 @@ rpcholqr_status rpcholqr_factor_f32(rpcholqr_plan p, const float* A, int64_t m, 
     launch_prep_f32(p->R1, np, n, p->T32, p->rinv32, RPCHOLQR_ERR_NOT_SPD, info, st);
     ++p->launches;
     pm.mark(RPCHOLQR_PHASE_PASS2);
-    if (launch_rowsolve_f32(Q, ldq, Q, ldq, m, n, p->T32, p->rinv32, info, false, st) != cudaSuccess)
+    if (launch_rowsolve_f32(Q, ldq, Q, ldq, m, n, p->T32, p->rinv32, info, false, p->grid, st) != cudaSuccess)
         return RPCHOLQR_ERR_CUDA;
     ++p->launches;
     pm.mark(RPCHOLQR_PHASE_RECOVER_R);

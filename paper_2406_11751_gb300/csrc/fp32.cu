@@ -6,10 +6,8 @@
 //
 //   k_prep_f32       T32 = float(T) padded with the identity, rinv32 = 1 / diag(T32);
 //   k_rowsolve_f32   Y = X T^{-1} row by row (Section 2.1: each row of A_1 is a triangular solve with
-//                    R_s), one row per thread, left-looking over 32-column blocks: the off-diagonal
-//                    part of a block is a length-32J dot product per column against the block of T
-//                    staged in shared memory (broadcast reads), the 32 x 32 diagonal block is forward
-//                    substitution in registers;
+//                    R_s), rows in shared memory, left-looking over 32-column blocks: the off-diagonal part of a
+//                    block as a register-tiled product, the 32 x 32 diagonal block by forward substitution;
 //   k_syrk_f32       per-range partials of G = A_1^T A_1 over 64 x 64 upper tiles, FP32 products summed
 //                    in FP32 over 256-row chunks, the chunks added into FP64 totals.
 #include "common.cuh"
@@ -17,7 +15,6 @@
 namespace rpq {
 
 constexpr int kF32Blk = 32;      // column block of the row solves
-constexpr int kF32Rows = 256;    // rows per CTA, one per thread
 constexpr int kSyrkChunkRows = 256;
 
 __host__ __device__ constexpr int pad32(int n) { return (n + 31) / 32 * 32; }
@@ -40,95 +37,174 @@ __global__ void k_prep_f32(const double* __restrict__ T, int64_t ldt, int n, int
     }
 }
 
-// Y = X T^{-1} for upper-triangular T (T32, rinv32 from k_prep_f32).  Y may equal X (ldy == ldx).
-__global__ void __launch_bounds__(kF32Rows)
+__device__ __forceinline__ void cp_async4f(void* dst, const void* src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(valid ? 4 : 0));
+}
+__device__ __forceinline__ void cp_async16f(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+                 "l"(src));
+}
+
+// Y = X T^{-1} for upper-triangular T (T32, rinv32 from k_prep_f32).  Y may equal X (ldy == ldx).  A CTA keeps R rows
+// in shared memory from load to store (row stride np32 + 4: float4 reads of a quarter-warp's rows hit distinct
+// banks) and solves them left-looking over 32-column blocks:
+//   off-diagonal  C -= Y[:, <block] T[<block, block], T streamed in 32 x 32 tiles (two buffers); a thread owns R / 32
+//                 rows x 4 columns, so four terms take R / 32 + 4 16-byte reads for R / 2 multiply-adds;
+//   diagonal      forward substitution, one thread per row, T's rows read as broadcasts.
+// 2^20 x 128 on GB300: 0.61 ms (28 TFLOP/s; shared-memory pipe 74 % busy, issue slots 57 %; the FMA pipe alone would take
+// 0.21 and HBM 0.16).  One row per thread, with the solved values re-read from global memory and a broadcast read of T
+// for every four multiply-adds, took 1.58 ms.
+// Rows per CTA: 128 while two such panels fit an SM, 64 above, 32 for matrices that give no full wave of 64.
+template <int R>
+__global__ void __launch_bounds__(256)
 k_rowsolve_f32(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, int n,
                const float* __restrict__ T32, int np32, const float* __restrict__ rinv32, int32_t* info,
-               bool check_finite, bool vec) {
-    extern __shared__ float4 ts4[];   // rows 0 .. 32J+31 of the 32 columns of block J (8 float4 per row)
+               bool check_finite, bool vec_in, bool vec_out) {
+    extern __shared__ float4 fsm4[];
+    constexpr int RT = R / 32;            // rows of a thread: ty + 32 i
     if (load_status(info) != 0) return;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * kF32Rows + threadIdx.x;
-    const bool live = r < m;
-    const float* xr = X + (live ? r : 0) * ldx;
-    float* yr = Y + (live ? r : 0) * ldy;
+    float* ts = reinterpret_cast<float*>(fsm4);            // two 32 x 32 tiles of T
+    float* panel = ts + 2 * kF32Blk * kF32Blk;
+    const int ld = np32 + 4;
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int64_t row0 = static_cast<int64_t>(blockIdx.x) * R;
+    const int nq = np32 / 4;
+    if (vec_in) {
+        for (int e = tid; e < R * nq; e += 256) {
+            const int r = e / nq, c = 4 * (e - r * nq);
+            float* dst = panel + r * ld + c;
+            if (row0 + r < m && c + 3 < n) cp_async16f(dst, X + (row0 + r) * ldx + c);
+            else
+                for (int u = 0; u < 4; ++u) {
+                    const bool ok = row0 + r < m && c + u < n;
+                    cp_async4f(dst + u, ok ? X + (row0 + r) * ldx + c + u : X, ok);
+                }
+        }
+    } else {
+        for (int e = tid; e < R * np32; e += 256) {
+            const int r = e / np32, c = e - r * np32;
+            const bool ok = row0 + r < m && c < n;
+            cp_async4f(panel + r * ld + c, ok ? X + (row0 + r) * ldx + c : X, ok);
+        }
+    }
+    // tile (kt, J) of T into buffer b: rows 32 kt .., columns 32 J ..; one float4 per thread
+    auto stage = [&](int kt, int J, int b) {
+        cp_async16f(ts + b * kF32Blk * kF32Blk + 4 * tid,
+                    T32 + static_cast<size_t>(kt * kF32Blk + ty) * np32 + J * kF32Blk + 4 * tx);
+    };
+    stage(0, 0, 0);
+    cp_async_commit();
     bool bad = false;
-    for (int c0 = 0; c0 < n; c0 += kF32Blk) {
-        __syncthreads();   // the previous block's reads of ts4 are done
-        for (int e = threadIdx.x; e < (c0 + kF32Blk) * 8; e += blockDim.x) {
-            const int k = e >> 3, q = e & 7;
-            ts4[e] = reinterpret_cast<const float4*>(T32 + static_cast<size_t>(k) * np32 + c0)[q];
-        }
-        __syncthreads();
-        if (!live) continue;
-        float acc[kF32Blk];
+    int b = 0;
+    const int nblk = np32 / kF32Blk;
+    for (int J = 0; J < nblk; ++J) {
+        float acc[RT][4];
+        for (int kt = 0; kt <= J; ++kt) {
+            // the tile (kt, J) and, the first time, the panel have landed; prefetch the next tile
+            cp_async_wait_all();
+            __syncthreads();
+            const bool last = kt == J;
+            if (!last || J + 1 < nblk) stage(last ? 0 : kt + 1, last ? J + 1 : J, b ^ 1);
+            cp_async_commit();
+            const float* t0 = ts + b * kF32Blk * kF32Blk;
+            b ^= 1;
+            if (kt == 0 && J > 0) {
 #pragma unroll
-        for (int c = 0; c < kF32Blk; ++c) {
-            acc[c] = c0 + c < n ? xr[c0 + c] : 0.0f;
-            bad |= !isfinite(acc[c]);
-        }
-        // acc -= Y[r, 0:c0] T[0:c0, c0:c0+32]; with 16-byte aligned rows, 8 solved values per two
-        // vector loads, two such groups in flight
-        if (vec) {
-#pragma unroll 2
-            for (int k = 0; k < c0; k += 8) {
-                const float4 ya = *reinterpret_cast<const float4*>(yr + k);
-                const float4 yb = *reinterpret_cast<const float4*>(yr + k + 4);
-                const float yv[8] = {-ya.x, -ya.y, -ya.z, -ya.w, -yb.x, -yb.y, -yb.z, -yb.w};
+                for (int i = 0; i < RT; ++i) {
+                    const float4 v = *reinterpret_cast<const float4*>(panel + (ty + 32 * i) * ld + J * kF32Blk + 4 * tx);
+                    acc[i][0] = v.x; acc[i][1] = v.y; acc[i][2] = v.z; acc[i][3] = v.w;
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                    const float4* tk = ts4 + (k + kk) * 8;
+                    for (int u = 0; u < 4; ++u) bad |= !isfinite(acc[i][u]);
+                }
+            }
+            if (!last) {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const float4 t = tk[q];
-                        acc[4 * q + 0] = fmaf(yv[kk], t.x, acc[4 * q + 0]);
-                        acc[4 * q + 1] = fmaf(yv[kk], t.y, acc[4 * q + 1]);
-                        acc[4 * q + 2] = fmaf(yv[kk], t.z, acc[4 * q + 2]);
-                        acc[4 * q + 3] = fmaf(yv[kk], t.w, acc[4 * q + 3]);
+                for (int k = 0; k < kF32Blk; k += 4) {
+                    float4 tv[4];
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) tv[kk] = *reinterpret_cast<const float4*>(t0 + (k + kk) * kF32Blk + 4 * tx);
+#pragma unroll
+                    for (int i = 0; i < RT; ++i) {
+                        const float4 y4 = *reinterpret_cast<const float4*>(panel + (ty + 32 * i) * ld + kt * kF32Blk + k);
+                        const float y[4] = {-y4.x, -y4.y, -y4.z, -y4.w};
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            acc[i][0] = fmaf(y[kk], tv[kk].x, acc[i][0]);
+                            acc[i][1] = fmaf(y[kk], tv[kk].y, acc[i][1]);
+                            acc[i][2] = fmaf(y[kk], tv[kk].z, acc[i][2]);
+                            acc[i][3] = fmaf(y[kk], tv[kk].w, acc[i][3]);
+                        }
                     }
                 }
+                continue;
             }
-        } else {
-            for (int k = 0; k < c0; ++k) {
-                const float yk = -yr[k];
-                const float4* tk = ts4 + k * 8;
+            if (J > 0) {
+#pragma unroll
+                for (int i = 0; i < RT; ++i)
+                    *reinterpret_cast<float4*>(panel + (ty + 32 * i) * ld + J * kF32Blk + 4 * tx) =
+                        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+                __syncthreads();
+            }
+            if (tid < R) {
+                float4* xr = reinterpret_cast<float4*>(panel + tid * ld + J * kF32Blk);
+                float x[kF32Blk];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                    const float4 t = tk[q];
-                    acc[4 * q + 0] = fmaf(yk, t.x, acc[4 * q + 0]);
-                    acc[4 * q + 1] = fmaf(yk, t.y, acc[4 * q + 1]);
-                    acc[4 * q + 2] = fmaf(yk, t.z, acc[4 * q + 2]);
-                    acc[4 * q + 3] = fmaf(yk, t.w, acc[4 * q + 3]);
+                    const float4 v = xr[q];
+                    x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
                 }
+                if (J == 0)
+#pragma unroll
+                    for (int c = 0; c < kF32Blk; ++c) bad |= !isfinite(x[c]);
+#pragma unroll
+                for (int j = 0; j < kF32Blk; ++j) {
+                    x[j] *= __ldg(rinv32 + J * kF32Blk + j);
+                    const float xj = -x[j];
+#pragma unroll
+                    for (int q = (j + 1) / 4; q < 8; ++q) {
+                        const float4 tv = *reinterpret_cast<const float4*>(t0 + j * kF32Blk + 4 * q);
+                        if (4 * q + 0 > j) x[4 * q + 0] = fmaf(xj, tv.x, x[4 * q + 0]);
+                        if (4 * q + 1 > j) x[4 * q + 1] = fmaf(xj, tv.y, x[4 * q + 1]);
+                        if (4 * q + 2 > j) x[4 * q + 2] = fmaf(xj, tv.z, x[4 * q + 2]);
+                        if (4 * q + 3 > j) x[4 * q + 3] = fmaf(xj, tv.w, x[4 * q + 3]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) xr[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
             }
         }
-        // diagonal block: forward substitution, row j of the block's T read as float4s
-#pragma unroll
-        for (int j = 0; j < kF32Blk; ++j) {
-            acc[j] *= rinv32[c0 + j];
-            const float xj = -acc[j];
-            const float4* trow = ts4 + (c0 + j) * 8;
-#pragma unroll
-            for (int q = (j + 1) / 4; q < 8; ++q) {
-                const float4 t = trow[q];
-                if (4 * q + 0 > j) acc[4 * q + 0] = fmaf(xj, t.x, acc[4 * q + 0]);
-                if (4 * q + 1 > j) acc[4 * q + 1] = fmaf(xj, t.y, acc[4 * q + 1]);
-                if (4 * q + 2 > j) acc[4 * q + 2] = fmaf(xj, t.z, acc[4 * q + 2]);
-                if (4 * q + 3 > j) acc[4 * q + 3] = fmaf(xj, t.w, acc[4 * q + 3]);
+    }
+    __syncthreads();
+    if (vec_out) {
+        for (int e = tid; e < R * nq; e += 256) {
+            const int r = e / nq, c = 4 * (e - r * nq);
+            if (row0 + r >= m) continue;
+            const float4 v = *reinterpret_cast<const float4*>(panel + r * ld + c);
+            float* dst = Y + (row0 + r) * ldy + c;
+            if (c + 3 < n) *reinterpret_cast<float4*>(dst) = v;
+            else {
+                if (c < n) dst[0] = v.x;
+                if (c + 1 < n) dst[1] = v.y;
+                if (c + 2 < n) dst[2] = v.z;
             }
         }
-#pragma unroll
-        for (int c = 0; c < kF32Blk; ++c)
-            if (c0 + c < n) yr[c0 + c] = acc[c];
+    } else {
+        for (int e = tid; e < R * np32; e += 256) {
+            const int r = e / np32, c = e - r * np32;
+            if (row0 + r < m && c < n) Y[(row0 + r) * ldy + c] = panel[r * ld + c];
+        }
     }
     if (__syncthreads_or(check_finite && bad) && threadIdx.x == 0) set_status(info, RPCHOLQR_ERR_NONFINITE);
 }
 
 // Partials of G = X^T X: CTA (tile, range) accumulates the 64 x 64 tile (I, J), I <= J, over the rows
-// [range*rows_per, ...) and writes gpart[range][p][q] (ld np64, FP64) for its tile.  Thread (ty, tx)
-// owns the 4 x 4 outputs p = 64I + 4ty + i, q = 64J + 4tx + j.
-__global__ void __launch_bounds__(256)
+// [range*rows_per, ...) and writes gpart[range][p][q] (ld np64, FP64) for its tile.  Thread (ty, tx) of 8 x 16 owns the
+// 8 x 4 outputs p = 64 I + 8 ty + i, q = 64 J + 4 tx + j: three 16-byte reads for 32 multiply-adds (4 x 4 outputs
+// needed two for 16: 1.00 -> 0.69 ms at 2^20 x 128).
+__global__ void __launch_bounds__(128)
 k_syrk_f32(const float* __restrict__ X, int64_t ldx, int64_t m, int n, int np64, int64_t rows_per,
-           double* __restrict__ gpart, const int32_t* info) {
+           double* __restrict__ gpart, const int32_t* info, bool vec) {
     __shared__ __align__(16) float xs[2][32][2 * 64 + 4];   // double-buffered 32-row chunks
     if (load_status(info) != 0) return;
     const int nb = np64 / 64;
@@ -138,58 +214,64 @@ k_syrk_f32(const float* __restrict__ X, int64_t ldx, int64_t m, int n, int np64,
     const int64_t rb = static_cast<int64_t>(blockIdx.y) * rows_per;
     const int64_t re = (rb + rows_per < m) ? rb + rows_per : m;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    float acc[4][4];
-    double tot[4][4];
+    const int boff = I == J ? 0 : 64;    // a diagonal tile's two operands are the same columns
+    float acc[8][4];
+    double tot[8][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) { acc[i][j] = 0.0f; tot[i][j] = 0.0; }
-    // rows k0 .. k0+31 of the two 64-column blocks into xs[b] (4-byte cp.async, zero-filled outside X)
+    // rows k0 .. k0+31 of the two 64-column blocks into xs[b] (zero outside X); 16-byte copies where rows are aligned
     auto stage = [&](int64_t k0, int b) {
-        for (int e = tid; e < 32 * 128; e += 256) {
-            const int rr = e >> 7, cc = e & 127;
+        const int per = 16 + (boff >> 2);            // float4 columns of a row
+        for (int e = tid; e < 32 * per; e += 128) {
+            const int rr = e / per, cc = 4 * (e - rr * per);
             const int col = cc < 64 ? 64 * I + cc : 64 * J + (cc - 64);
-            const bool ok = k0 + rr < re && col < n;
-            const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(&xs[b][rr][cc]));
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(dst),
-                         "l"(ok ? X + (k0 + rr) * ldx + col : X), "r"(ok ? 4 : 0));
+            float* dst = &xs[b][rr][cc];
+            const float* src = X + (k0 + rr) * ldx + col;
+            if (vec && k0 + rr < re && col + 3 < n) cp_async16f(dst, src);
+            else
+                for (int u = 0; u < 4; ++u) {
+                    const bool ok = k0 + rr < re && col + u < n;
+                    cp_async4f(dst + u, ok ? src + u : X, ok);
+                }
         }
     };
     if (rb < re) stage(rb, 0);
-    asm volatile("cp.async.commit_group;\n");
+    cp_async_commit();
     int64_t chunk_end = rb + kSyrkChunkRows;
     int b = 0;
     for (int64_t k0 = rb; k0 < re; k0 += 32, b ^= 1) {
-        if (k0 + 32 < re) stage(k0 + 32, b ^ 1);   // xs[b ^ 1] was last read before the barrier below
-        asm volatile("cp.async.commit_group;\n");
-        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        __syncthreads();
+        cp_async_wait_all();
+        __syncthreads();   // chunk k0 has landed, and every thread is done with xs[b ^ 1]
+        if (k0 + 32 < re) stage(k0 + 32, b ^ 1);
+        cp_async_commit();
 #pragma unroll 8
         for (int kk = 0; kk < 32; ++kk) {
-            const float4 a = *reinterpret_cast<const float4*>(&xs[b][kk][4 * ty]);
-            const float4 bb = *reinterpret_cast<const float4*>(&xs[b][kk][64 + 4 * tx]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
+            const float4 a0 = *reinterpret_cast<const float4*>(&xs[b][kk][8 * ty]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&xs[b][kk][8 * ty + 4]);
+            const float4 bb = *reinterpret_cast<const float4*>(&xs[b][kk][boff + 4 * tx]);
+            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
         if (k0 + 32 >= chunk_end) {
             chunk_end += kSyrkChunkRows;
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) { tot[i][j] += acc[i][j]; acc[i][j] = 0.0f; }
         }
-        __syncthreads();   // every thread is done with xs[b] before it is refilled
     }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    cp_async_wait_all();
     double* out = gpart + static_cast<size_t>(blockIdx.y) * np64 * np64;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int p = 64 * I + 4 * ty + i, q = 64 * J + 4 * tx + j;
+            const int p = 64 * I + 8 * ty + i, q = 64 * J + 4 * tx + j;
             out[static_cast<size_t>(p) * np64 + q] = tot[i][j] + acc[i][j];
         }
 }
@@ -212,19 +294,30 @@ void launch_prep_f32(const double* T, int64_t ldt, int n, float* T32, float* rin
     k_prep_f32<<<(np32 * np32 + 255) / 256, 256, 0, st>>>(T, ldt, n, np32, T32, rinv32, fail_status, info);
 }
 
-cudaError_t launch_rowsolve_f32(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, int n,
-                                const float* T32, const float* rinv32, int32_t* info, bool check_finite,
-                                cudaStream_t st) {
+template <int R>
+static cudaError_t launch_rowsolve_f32_r(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, int n,
+                                         const float* T32, const float* rinv32, int32_t* info, bool check_finite,
+                                         cudaStream_t st) {
     const int np32 = pad32(n);
-    const int smem = np32 * kF32Blk * static_cast<int>(sizeof(float));
-    cudaError_t err = cudaFuncSetAttribute(k_rowsolve_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int smem = (2 * kF32Blk * kF32Blk + R * (np32 + 4)) * static_cast<int>(sizeof(float));
+    cudaError_t err = cudaFuncSetAttribute(k_rowsolve_f32<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err != cudaSuccess) return err;
-    const int64_t grid = (m + kF32Rows - 1) / kF32Rows;
-    // vector loads of solved values need 16-byte aligned rows
-    const bool vec = (reinterpret_cast<uintptr_t>(Y) % 16 == 0) && (ldy % 4 == 0);
-    k_rowsolve_f32<<<static_cast<unsigned>(grid), kF32Rows, smem, st>>>(X, ldx, Y, ldy, m, n, T32, np32, rinv32,
-                                                                         info, check_finite, vec);
+    // 16-byte copies need 16-byte aligned rows
+    const bool vec_in = reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0;
+    const bool vec_out = reinterpret_cast<uintptr_t>(Y) % 16 == 0 && ldy % 4 == 0;
+    k_rowsolve_f32<R><<<static_cast<unsigned>((m + R - 1) / R), 256, smem, st>>>(X, ldx, Y, ldy, m, n, T32, np32, rinv32, info,
+                                                                                check_finite, vec_in, vec_out);
     return cudaGetLastError();
+}
+
+// sms: the device's SMs, for the choice of rows per CTA (see k_rowsolve_f32).
+cudaError_t launch_rowsolve_f32(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, int n,
+                                const float* T32, const float* rinv32, int32_t* info, bool check_finite, int sms,
+                                cudaStream_t st) {
+    if (m < static_cast<int64_t>(sms) * 64) return launch_rowsolve_f32_r<32>(X, ldx, Y, ldy, m, n, T32, rinv32, info, check_finite, st);
+    if (n > 192 || m < static_cast<int64_t>(sms) * 256)
+        return launch_rowsolve_f32_r<64>(X, ldx, Y, ldy, m, n, T32, rinv32, info, check_finite, st);
+    return launch_rowsolve_f32_r<128>(X, ldx, Y, ldy, m, n, T32, rinv32, info, check_finite, st);
 }
 
 // ranges x np64 x np64 doubles in gpart; returns the number of ranges used.
@@ -240,7 +333,8 @@ int launch_syrk_f32(const float* X, int64_t ldx, int64_t m, int n, int max_range
     if (ranges > most) ranges = static_cast<int>(most);
     int64_t rows_per = (m + ranges - 1) / ranges;
     rows_per = (rows_per + 31) / 32 * 32;
-    k_syrk_f32<<<dim3(tiles, ranges), 256, 0, st>>>(X, ldx, m, n, np64, rows_per, gpart, info);
+    const bool vec = reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0;
+    k_syrk_f32<<<dim3(tiles, ranges), 128, 0, st>>>(X, ldx, m, n, np64, rows_per, gpart, info, vec);
     return ranges;
 }
 
