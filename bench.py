@@ -429,9 +429,9 @@ def kernels_per_step(ph, calls):
             for k, (ms, nl, fl) in ph.get("kernels", {}).items() if nl > 0}
 
 
-# Each FP64-accurate split product runs 36 BF16 slice products (eight 7-bit slices per operand, the pairs
-# with a + b <= 9); the tensor roofline of a split kernel counts those BF16 flops.
-SLICE_PRODUCTS = 36
+# Each FP64-accurate split product runs 28 FP16 slice products (seven 8-bit digits per operand, the pairs
+# with a + b <= 8); the tensor roofline of a split kernel counts those flops.
+SLICE_PRODUCTS = 28
 SPLIT_CLASSES = ("split_update", "split_gemm_sub", "split_gemm", "split_gram")
 KERNEL_NAMES = {
     "rowpass": "k_rowpass (FP64 row solves: mma.sync m16n8k16 + DFMA)",
@@ -484,7 +484,7 @@ def measured_peaks():
 def kernel_rooflines(phases, calls, fp64_peak_tflops):
     """Roofline entry per kernel class from the per-launch CUDA events of the timed steps: FP64 classes
     against the FP64 pipe (in-run probe), split classes against the BF16 tensor pipe (sustained cuBLAS
-    figure of MEASURED_PEAKS.json: these kernels run inside a seconds-long step) counting the 36 slice
+    figure of MEASURED_PEAKS.json: these kernels run inside a seconds-long step) counting the 28 slice
     products of each FP64-accurate product."""
     peaks = measured_peaks()
     bf16 = peaks.get("bf16_tflops_sustained") or peaks.get("bf16_tflops")
@@ -498,7 +498,7 @@ def kernel_rooflines(phases, calls, fp64_peak_tflops):
             e = {"kernel": KERNEL_NAMES[k], "bound": "tensor", "achieved": achieved, "peak": bf16,
                  "unit": "TFLOP/s", "frac": achieved / bf16 if bf16 else None, "fp64_equivalent_tflops": fp64_tf,
                  "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured); achieved counts "
-                                "36 BF16 slice products per FP64 product"}
+                                "28 FP16 slice products per FP64 product"}
         else:
             e = {"kernel": KERNEL_NAMES[k], "bound": "alu", "achieved": fp64_tf, "peak": fp64_peak_tflops,
                  "unit": "TFLOP/s", "frac": fp64_tf / fp64_peak_tflops,

@@ -65,7 +65,7 @@ typedef enum {
     RPCHOLQR_SPLIT64 = 1, /* FP64-accurate split precision: sketch QR, Cholesky and the diagonal
                             blocks of the row solves in FP64; the Gram matrix, the off-diagonal
                             block update of the row solve (n > 64) and Q = A1 R1^{-1} (explicit
-                            inverse of the well-conditioned R1) as Ozaki-split BF16 tensor-core
+                            inverse of the well-conditioned R1) as Ozaki-split FP16 tensor-core
                             (tcgen05) products with exact FP32 group sums and int64 combination.
                             Q = A1 R1^{-1} takes that path only while ||R1||_F ||R1^{-1}||_F / n <= 2
                             (A1 well conditioned, as for incoherent or smoothed A); otherwise an FP64
@@ -138,7 +138,7 @@ typedef enum {
                                        np = max_n rounded up to 16, plus its work list; 0 frees it.
                                        Default 0: the first batched call allocates for its count. */
     RPCHOLQR_OPT_IMAGE_ROWS = 4     /* SPLIT64 plans above 128 columns: rows of the stage images (the
-                                       BF16 slices the wide passes stream, 16 bytes a value) kept at a
+                                       FP16 slices the wide passes stream, 14 bytes a value) kept at a
                                        time; the first pass and the Gram run chunk by chunk of that
                                        many rows, the second pass by chunks of at most 8 GiB of images.
                                        0 (default): every row when their images take at most a quarter
@@ -263,7 +263,7 @@ rpcholqr_status rpcholqr_solve_rows(rpcholqr_plan plan, const double* X, int64_t
 rpcholqr_status rpcholqr_triu_mul(const double* R1, const double* Rs, int32_t n, double* R,
                                   void* stream);
 
-/* Split-precision FP64 product C = X Y on the BF16 tensor cores (the kernel SPLIT64 uses):
+/* Split-precision FP64 product C = X Y on the FP16 tensor cores (the kernel SPLIT64 uses):
  * X device m x K (ldx), Y device K x N (ldy), C device m x N (ldc; must not overlap X), K, N <= plan
  * max_n; each entry carries an absolute error below ~2^-53 * 2^(Ex+Ey) (Ex, Ey: power-of-two bounds
  * of row i of X and column j of Y).  The plan must be a SPLIT64 plan.  info as above (RPCHOLQR_ERR_TIMEOUT if a bounded

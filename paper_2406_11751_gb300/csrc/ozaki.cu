@@ -1,4 +1,4 @@
-// Split-precision (Ozaki-style) FP64 products on the GB300 BF16 tensor cores (tcgen05).
+// Split-precision (Ozaki-style) FP64 products on the GB300 FP16 tensor cores (tcgen05).
 //
 // Used by the SPLIT64 mode for the well-conditioned products of Algorithm alg_2 (Section 4):
 //   Gram          G_1 = A_1^T A_1               (k_ozaki_gram; above 128 columns k_ozaki_gram_db)
@@ -14,19 +14,20 @@
 //
 // Splitting (Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix multiplication by using
 // fast routines of matrix multiplication and its applications", Numer. Algorithms 2012, restated): every
-// FP64 value x of a row (or column) with the shared power-of-two bound 2^E > max|x| is cut into eight
-// 7-bit signed integer slices, x = 2^E sum_{a=1..8} s_a 2^{-7a} + O(2^{E-56}), |s_a| <= 127 (exact in
-// BF16).  A product of two such operands is sum_{a,b} 2^{-7(a+b)} S_a S_b; the 36 slice pairs with
-// a + b <= 9 are kept (the dropped ones are below 2^-53 of the scale).  Pairs with the same d = a + b
-// share one FP32 accumulator in tensor memory: with K <= 128 every partial sum is an integer below
-// 8 * 127^2 * 128 < 2^24, so the FP32 accumulation is exact.  The eight accumulators (d = 2..9) are
-// combined exactly in int64, I = sum_{d<=6} M_d 2^{7(6-d)} + rint(sum_{d>6} M_d 2^{7(6-d)}), and the
-// result is 2^{E_x + E_y - 42} I.
+// FP64 value x of a row (or column) with the shared power-of-two bound 2^E > max|x| is rounded to 56 bits,
+// F = rint(x 2^{55-E}), and cut into seven signed 8-bit digits, F = sum_{a=1..7} s_a 256^{7-a}, |s_a| <= 128
+// (exact in FP16), so x = 2^E (sum s_a 2^{1-8a} + e), |e| <= 2^-56.  A product of two such operands is
+// sum_{a,b} 2^{2-8(a+b)} S_a S_b; the 28 pairs with a + b <= 8 are kept (the six dropped ones with a + b = 9 are below
+// 6 2^-56 of the scale a term, 2^-56 in the mean square).  Pairs with the same d = a + b share one FP32 accumulator in
+// tensor memory: with K <= 128 every partial sum is an integer below 7 128^2 128 < 2^24, so the FP32 accumulation is
+// exact.  The seven accumulators (d = 2..8) are combined exactly in int64 and rounded once to units of 2^-53 of the
+// scale.  (Eight 7-bit digits in BF16 needed 36 pairs, 16 instead of 14 bytes a value and about twice the
+// instructions per value and per output.)
 //
-// Tiles: M = 128 output rows (TMEM lanes) x N = 64 output columns, 8 groups x 64 columns = the 512 TMEM
-// columns of the SM (k_ozaki_update: N = 32, two tiles in TMEM).  K is staged 32 at a time in shared
+// Tiles: M = 128 output rows (TMEM lanes) x N = 64 output columns, 7 groups x 64 columns of the SM's 512 TMEM
+// columns (k_ozaki_update: N = 32, two tiles in TMEM).  K is staged 32 at a time in shared
 // memory (core-matrix K-major layout, no swizzle), two stages in flight: while the tensor core works on
-// one stage the CTA slices the next.  One thread issues the 72 tcgen05.mma of a stage and commits them
+// one stage the CTA slices the next.  One thread issues the tcgen05.mma of a stage and commits them
 // to the stage's mbarrier.  Every mbarrier wait is bounded: the pipeline waits by the caller's spin limit
 // (a plan option), the final wait for the kernel's own MMAs by kSpinLimit; on timeout the kernel records
 // RPCHOLQR_ERR_TIMEOUT, waits (bounded) for its own MMAs, frees its tensor memory and returns.
@@ -37,8 +38,8 @@
 namespace rpq {
 namespace oz {
 
-constexpr int kSlices = 8;
-constexpr int kGroups = 8;                 // d = 2..9
+constexpr int kSlices = 7;
+constexpr int kGroups = 7;                 // d = 2..8
 constexpr int kTileM = 128;
 constexpr int kTileN = 64;
 constexpr int kKW = 32;                    // K per stage
@@ -56,8 +57,8 @@ constexpr int kSBO = (kKW * 2 / 16) * 128; // 512 B between 8-row core-matrix gr
 constexpr int kLBO = 128;                  // 128 B between K-adjacent core matrices
 constexpr int kASlice = kTileM * kKW * 2;  // 8 KB
 constexpr int kBSlice = kTileN * kKW * 2;  // 4 KB
-constexpr int kAStage = kSlices * kASlice; // 64 KB
-constexpr int kBStage = kSlices * kBSlice; // 32 KB
+constexpr int kAStage = kSlices * kASlice; // 56 KB
+constexpr int kBStage = kSlices * kBSlice; // 28 KB
 // k_ozaki_gemm_ws shared memory: two stages (A slices, then B slices: 96 KB each), then the raw FP64 X
 // rows of the next stage (row stride kRawLd doubles: 16-byte reads of one row per thread are
 // conflict-free).  At a tile end the drained stage's 96 KB stage the 128 x 64 output tile (row stride
@@ -71,10 +72,6 @@ static_assert(kTileM * kEpiLd * 8 <= kStageBytes, "output tile must fit in one s
 static_assert(kGemmSmem + 1024 <= 232448, "k_ozaki_gemm_ws exceeds the 227 KB shared-memory limit");
 constexpr int kTmemCols = 512;
 constexpr long kSpinLimit = 1L << 24;
-// BF16 x BF16 -> FP32, A and B K-major, M = 128, N = 64
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTileN >> 3) << 17) |
-                            ((uint32_t)(kTileM >> 4) << 24);
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -87,18 +84,11 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
     return static_cast<uint64_t>((addr >> 4) & 0x3FFF) | (static_cast<uint64_t>(kLBO >> 4) << 16) |
            (static_cast<uint64_t>(kSBO >> 4) << 32) | (1ull << 46);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-        "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
+// Instruction descriptor: FP16 x FP16 -> FP32, A and B K-major, M = 128, N = n (a multiple of 16, <= 256)
+__host__ __device__ constexpr uint32_t idesc_f16(int n) {
+    return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(kTileM >> 4) << 24);
 }
-// Instruction descriptor: BF16 x BF16 -> FP32, A and B K-major, M = 128, N = n (a multiple of 16, <= 256)
-__host__ __device__ constexpr uint32_t idesc_bf16(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) |
-           (static_cast<uint32_t>(kTileM >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16_n(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_f16_n(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
@@ -149,7 +139,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 // Pre-sliced stages arrive by bulk copies (the TMA engine, no tensor map): the issuing thread arms the
 // stage's load barrier with the byte count, and each copy completes its share of the transaction on it.
-// Sizes are multiples of 16 bytes and both addresses 16-byte aligned (64 KB / 4 KB / 32 KB images at
+// Sizes are multiples of 16 bytes and both addresses 16-byte aligned (56 KB / 2 KB / 4 KB images at
 // 1 KB-aligned stage buffers).
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -167,7 +157,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
 }
-// Stages prefetched into L2 ahead of the stage being copied (64 KB each: 152 SMs x 4 x 64 KB = 39 MB of L2).
+// Stages prefetched into L2 ahead of the stage being copied (56 KB each: 152 SMs x 4 x 56 KB = 34 MB of L2).
 constexpr int kPrefetchAhead = 4;
 
 // Before a kernel that issued bulk copies returns (also after a timeout): the last copy issued into each
@@ -219,92 +209,77 @@ __device__ __forceinline__ void tmem_ld4(uint32_t addr, float (&v)[4]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
 
-// 56-bit fixed-point magnitude F = floor(|x| 2^{56-E}) of x relative to the bound 2^E > |x|, split in
-// two 28-bit halves (hi: slices 1..4, lo: slices 5..8).  0 for zero, subnormal, non-finite or unknown E.
-// Branch-free: F = (mantissa 2^3) >> (3 - sh) with sh = ex - 1019 - E <= 3 for a valid bound (a larger
-// sh, |x| >= 2^E, saturates).
-__device__ __forceinline__ void fixed56(double x, int E, uint32_t& fhi, uint32_t& flo) {
+// G = F + 0x80808080808080, F = rint(x 2^{55-E}) for |x| < 2^E: the bytes of G are the seven digits plus 128
+// (digit 7 the lowest byte).  F = 0 for zero, subnormal, non-finite or unknown E.  Branch-free: 2 |F| before the last
+// rounding is (mantissa 2^3) >> r with r = E + 1022 - ex >= 0 for a valid bound (|x| >= 2^E saturates).
+__device__ __forceinline__ void digits56(double x, int E, uint32_t& hi, uint32_t& lo) {
     const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
     const int ex = static_cast<int>((bits >> 52) & 0x7FF);
     const unsigned long long mant8 = ((bits & ((1ull << 52) - 1)) | (1ull << 52)) << 3;   // < 2^56
     const int r = E + 1022 - ex;
-    unsigned long long F = mant8 >> (r < 63 ? (r > 0 ? r : 0) : 63);
-    F = r < 0 ? (1ull << 56) - 1 : F;
+    unsigned long long F = ((mant8 >> (r < 63 ? (r > 0 ? r : 0) : 63)) + 1) >> 1;
+    F = r < 0 ? (1ull << 55) - 1 : F;
     F = (ex != 0 && ex != 0x7FF && E > kNoExp) ? F : 0ull;
-    fhi = static_cast<uint32_t>(F >> 28);
-    flo = static_cast<uint32_t>(F) & 0x0FFFFFFFu;
+    const unsigned long long neg = static_cast<unsigned long long>(static_cast<long long>(bits) >> 63);   // 0 or ~0
+    const unsigned long long G = (F ^ neg) + (0x80808080808080ull - neg);
+    hi = static_cast<uint32_t>(G >> 32);
+    lo = static_cast<uint32_t>(G);
 }
 
-// Two 7-bit fields (bits pos..pos+6 of u0 and u1) as a packed BF16 pair (u0 in the low half), signed:
-// the pair of BF16 numbers 128 + v (exponent 7, mantissa v) goes through one packed BF16 FMA,
-// (128 + v) s - 128 s = s v, exact.  sgn2: the BF16 pair (s0, s1), s = +-1; off2: (-128 s0, -128 s1).
-__device__ __forceinline__ uint32_t bf16x2_field(uint32_t u0, uint32_t u1, int pos, uint32_t sgn2, uint32_t off2) {
-    const uint32_t t = ((u0 >> pos) & 0x7Fu) | (((u1 >> pos) & 0x7Fu) << 16) | 0x43004300u;
+// Digit from byte `b` of w0 and w1 as a packed FP16 pair (w0's in the low half): 1024 + byte is the bit pattern
+// 0x6400 + byte, and 1152 is subtracted exactly.  b = 2 is the first digit, which may be 128 (x just below 2^E): all
+// the upper bits of G.
+__device__ __forceinline__ uint32_t f16x2_digit(uint32_t w0, uint32_t w1, int b, bool first = false) {
+    const uint32_t t = first ? __byte_perm(w0, w1, 0x7632) | 0x64006400u
+                             : (__byte_perm(w0, w1, b | ((4 + b) << 8)) & 0x00FF00FFu) | 0x64006400u;
     uint32_t r;
-    asm("fma.rn.bf16x2 %0, %1, %2, %3;\n" : "=r"(r) : "r"(t), "r"(sgn2), "r"(off2));
+    asm("add.rn.f16x2 %0, %1, %2;\n" : "=r"(r) : "r"(t), "r"(0xE480E480u));
     return r;
 }
 
 // Slice the 8 values x[0..7] (consecutive K) and store slice a of all eight as one 16-byte core-matrix
-// row at dst + a * slice_bytes (x[i] in BF16 lane i).  Every slice carries the sign of its value.
-__device__ __forceinline__ void slice_store8(const double (&x)[8], int E, uint8_t* dst, int slice_bytes) {
-    uint32_t fh[8], fl[8], sgn2[4], off2[4];
+// row at dst + a * slice_bytes (x[i] in FP16 lane i), and at dst2 + a * slice_bytes2 too unless dst2 is null.
+__device__ __forceinline__ void slice_store8(const double (&x)[8], int E, uint8_t* dst, int slice_bytes,
+                                             uint8_t* dst2 = nullptr, int slice_bytes2 = 0) {
+    uint32_t hi[8], lo[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) fixed56(x[i], E, fh[i], fl[i]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const bool n0 = __double_as_longlong(x[2 * j]) < 0, n1 = __double_as_longlong(x[2 * j + 1]) < 0;
-        sgn2[j] = (n0 ? 0xBF80u : 0x3F80u) | ((n1 ? 0xBF80u : 0x3F80u) << 16);    // -1 / +1
-        off2[j] = (n0 ? 0x4300u : 0xC300u) | ((n1 ? 0x4300u : 0xC300u) << 16);    // +128 / -128
-    }
+    for (int i = 0; i < 8; ++i) digits56(x[i], E, hi[i], lo[i]);
 #pragma unroll
     for (int a = 0; a < kSlices; ++a) {
-        const int pos = 21 - 7 * (a & 3);
         uint32_t w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            w[j] = a < 4 ? bf16x2_field(fh[2 * j], fh[2 * j + 1], pos, sgn2[j], off2[j])
-                         : bf16x2_field(fl[2 * j], fl[2 * j + 1], pos, sgn2[j], off2[j]);
-        *reinterpret_cast<uint4*>(dst + a * slice_bytes) = make_uint4(w[0], w[1], w[2], w[3]);
+            w[j] = a < 3 ? f16x2_digit(hi[2 * j], hi[2 * j + 1], 2 - a, a == 0) : f16x2_digit(lo[2 * j], lo[2 * j + 1], 6 - a);
+        const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(dst + a * slice_bytes) = v;
+        if (dst2) *reinterpret_cast<uint4*>(dst2 + a * slice_bytes2) = v;
     }
 }
 
-// Exact combination of the eight group sums M_d (d = 2..9) of one output element:
-//   I = sum_{d=2..6} M_d 2^{7(6-d)}  (units of 2^-42 of the operand scale, |I| < 2^50),
-//   L = sum_{d=7..9} M_d 2^{7(9-d)}  (units of 2^-63, |L| < 2^39).
-__device__ __forceinline__ void combine_groups(const float (&m)[kGroups], long long& I, long long& L) {
-    I = (static_cast<long long>(__float2int_rn(m[0])) << 28) +
-        (static_cast<long long>(__float2int_rn(m[1])) << 21) +
-        (static_cast<long long>(__float2int_rn(m[2])) << 14) +
-        (static_cast<long long>(__float2int_rn(m[3])) << 7) + static_cast<long long>(__float2int_rn(m[4]));
-    L = (static_cast<long long>(__float2int_rn(m[5])) << 14) +
-        (static_cast<long long>(__float2int_rn(m[6])) << 7) + static_cast<long long>(__float2int_rn(m[7]));
+// One output element from its seven group sums M_d (d = 2..8), sum_d M_d 2^{2-8d}, in units of 2^-UNITS (53 or 49),
+// exact up to one rounding.  |M_d| <= (d - 1) 2^21 with K <= 128, so M_4 2^8 + M_5 and M_6 2^7 fit int32.
+template <int UNITS>
+__device__ __forceinline__ long long combine_ints(const int (&v)[kGroups]) {
+    constexpr int S = 53 - UNITS;   // 0 or 4
+    const long long L = static_cast<long long>(v[5]) * 256 + static_cast<long long>(v[6] + (256 << S));   // 2^-62
+    const int low = v[4] * (128 >> S) + static_cast<int>(L >> (9 + S));
+    return ((static_cast<long long>(v[0]) << 39) >> S) + static_cast<long long>(v[1] * 2) * (1 << (30 - S)) +
+           static_cast<long long>(v[2] * 256 + v[3]) * (1 << (15 - S)) + static_cast<long long>(low);
 }
-// For K <= 32 every group sum is below 8 * 127^2 * 32 < 2^22 in magnitude, so M + 1.5 2^23 holds M
-// exactly in its low mantissa bits: the integer is read from the bit pattern (no conversion
-// instruction), and pairs of neighbouring groups fit one int32 (M_d 2^7 + M_{d+1} < 2^30), leaving
-// three 32 x 32 -> 64-bit multiply-adds for the int64 part.
+template <int UNITS>
+__device__ __forceinline__ long long combine_units(const float (&m)[kGroups]) {
+    int v[kGroups];
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) v[g] = __float2int_rn(m[g]);
+    return combine_ints<UNITS>(v);
+}
+// For K <= 32 every group sum is below 7 128^2 32 < 2^22 in magnitude, so M + 1.5 2^23 holds M exactly in its low
+// mantissa bits: the integer is read from the bit pattern, no conversion instruction.
 __device__ __forceinline__ long long combine_units53_k32(const float (&m)[kGroups]) {
     int v[kGroups];
 #pragma unroll
     for (int g = 0; g < kGroups; ++g) v[g] = __float_as_int(m[g] + 12582912.0f) - 0x4B400000;
-    const int u = v[1] * 128 + v[2], t = v[3] * 128 + v[4], w = v[6] * 128 + v[7];
-    const long long I = static_cast<long long>(v[0]) * (1ll << 28) +
-                        (static_cast<long long>(u) * (1ll << 14) + static_cast<long long>(t));
-    const long long L = static_cast<long long>(v[5]) * (1ll << 14) + static_cast<long long>(w);
-    return I * 2048 + ((L + 512) >> 10);
-}
-// the value in units of 2^-53 (rounded), for a single-window product: |result| < 2^61
-__device__ __forceinline__ long long combine_units53(const float (&m)[kGroups]) {
-    long long I, L;
-    combine_groups(m, I, L);
-    return (I << 11) + ((L + 512) >> 10);
-}
-// the value in units of 2^-49 (rounded), accumulated across windows
-__device__ __forceinline__ long long combine_units49(const float (&m)[kGroups]) {
-    long long I, L;
-    combine_groups(m, I, L);
-    return (I << 7) + ((L + (1ll << 13)) >> 14);
+    return combine_ints<53>(v);
 }
 
 // I * 2^e: I converted to FP64 (rounded to nearest above 2^53), exponent added in the bit pattern
@@ -318,7 +293,19 @@ __device__ __forceinline__ double scale_pow2(long long I, int e) {
     return ldexp(v, e);
 }
 
-// Add the eight TMEM group sums of this thread's row and its NC columns (col0.. of the 64-column tile,
+// The same without FP64 instructions (rounded to nearest, ties away), for the update, whose FP64 units carry the
+// subtraction already.
+__device__ __forceinline__ double scale_pow2_int(long long I, int e) {
+    const unsigned long long neg = static_cast<unsigned long long>(I >> 63), a = (static_cast<unsigned long long>(I) ^ neg) - neg;
+    const int lz = __clzll(static_cast<long long>(a)), field = 1085 - lz + e;
+    const unsigned long long M = a << (lz & 63);
+    const unsigned long long b = (static_cast<unsigned long long>(field) << 52) + (M >> 11) + ((M >> 10) & 1);
+    if (a == 0) return 0.0;
+    if (field <= 0 || field >= 0x7FD) return ldexp(static_cast<double>(I), e);
+    return __longlong_as_double(static_cast<long long>(b | (neg << 63)));
+}
+
+// Add the TMEM group sums of this thread's row and its NC columns (col0.. of the 64-column tile,
 // read CW at a time) to int64 accumulators in units of 2^-53 (U53) or 2^-49 of the operand scale.
 // The sliced operands are below 0.51 of their power-of-two bounds, so a K-term sum stays below
 // 0.26 K scale: units of 2^-53 hold K < 2^10 / 0.26 (about 3900) terms -- the products take K <= 2048,
@@ -338,68 +325,39 @@ __device__ __forceinline__ void drain_acc(uint32_t tmem, int warp, int col0, lon
             float grp[kGroups];
 #pragma unroll
             for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][j];
-            acc[c0 + j] += U53 ? combine_units53(grp) : combine_units49(grp);
+            acc[c0 + j] += combine_units<U53 ? 53 : 49>(grp);
         }
     }
 }
 
-// Issue the 72 MMAs of one stage: all pairs (a, b), a + b <= 9, for the two K=16 steps, one N = 64 MMA
-// per pair (any slice stride of B: used when B's slices are not stored back to back).
-// first_window: the stage starts an exactness window (the first MMA into each accumulator clears it).
-// The descriptors of the stage's two base addresses are formed once; every MMA adds its (constant)
-// offset to the 14-bit start field, which cannot carry (shared memory < 256 KB).
-__device__ __forceinline__ void issue_stage_pairs(uint32_t tmem, uint32_t a_base, uint32_t b_base,
-                                                  uint32_t b_slice_bytes, bool first_window) {
-    const uint64_t a0 = sdesc(a_base), b0 = sdesc(b_base);
-    const uint32_t bstep = b_slice_bytes >> 4;
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-#pragma unroll
-        for (int d = 2; d <= 9; ++d) {
-            const int alo = d - 8 > 1 ? d - 8 : 1, ahi = d - 1 < 8 ? d - 1 : 8;
-#pragma unroll
-            for (int a = alo; a <= ahi; ++a) {
-                const int b = d - a;
-                const uint64_t ad = a0 + static_cast<uint32_t>(((a - 1) * kASlice + kk * 256) >> 4);
-                const uint64_t bd = b0 + (static_cast<uint32_t>(b - 1) * bstep + static_cast<uint32_t>(kk * 16));
-                const uint32_t acc = (first_window && kk == 0 && a == alo) ? 0u : 1u;
-                mma_bf16(tmem + (d - 2) * kTileN, ad, bd, acc);
-            }
-        }
-    }
-}
-
-// The same 36 pairs per K = 16 step in 12 MMAs, for B slices stored back to back (kBSlice apart: the
-// eight 64-row slices form one 512-row operand in the same core-matrix layout).  For slice a of X the
-// pairs (a, b), b = 1 .. 9 - a, go to the groups d = a + b, whose accumulators are adjacent 64-column
-// ranges of tensor memory: one MMA with N = 64 nb multiplies slice a by nb consecutive B slices at once
-// (N <= 256, so slices 1-4 and 5-8 are two MMAs).  Same products, same exact integer sums.
+// The 28 slice pairs of one 32-wide K stage in 10 MMAs per K = 16 step: B's seven 64-row slices are stored back to back
+// (kBSlice apart), so they form one 448-row operand in the same core-matrix layout.  For slice a of X the pairs (a, b),
+// b = 1 .. 8 - a, go to the groups d = a + b, whose accumulators are adjacent 64-column ranges of tensor memory: one
+// MMA with N = 64 nb multiplies slice a by nb consecutive B slices at once (N <= 256, so slices 1-4 and 5-7 are two
+// MMAs).  first_window: the stage starts an exactness window (slice 1's MMAs clear all seven accumulators).  The
+// descriptors of the stage's two base addresses are formed once; every MMA adds its (constant) offset to the 14-bit
+// start field, which cannot carry (shared memory < 256 KB).
 __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t a_base, uint32_t b_base, bool first_window) {
     const uint64_t a0 = sdesc(a_base), b0 = sdesc(b_base);
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
-        for (int a = 1; a <= 8; ++a) {
-            const int nb = 9 - a;
+        for (int a = 1; a <= kSlices; ++a) {
+            const int nb = kSlices + 1 - a;
             const int n1 = nb < 4 ? nb : 4;
             const uint64_t ad = a0 + static_cast<uint32_t>(((a - 1) * kASlice + kk * 256) >> 4);
             const uint32_t acc = (first_window && kk == 0 && a == 1) ? 0u : 1u;
-            mma_bf16_n(tmem + (a - 1) * kTileN, ad, b0 + static_cast<uint32_t>(kk * 16), idesc_bf16(kTileN * n1),
-                       acc);
+            mma_f16_n(tmem + (a - 1) * kTileN, ad, b0 + static_cast<uint32_t>(kk * 16), idesc_f16(kTileN * n1), acc);
             if (nb > 4)
-                mma_bf16_n(tmem + (a + 3) * kTileN, ad,
-                           b0 + static_cast<uint32_t>((4 * kBSlice) >> 4) + static_cast<uint32_t>(kk * 16),
-                           idesc_bf16(kTileN * (nb - 4)), acc);
+                mma_f16_n(tmem + (a + 3) * kTileN, ad,
+                          b0 + static_cast<uint32_t>((4 * kBSlice) >> 4) + static_cast<uint32_t>(kk * 16),
+                          idesc_f16(kTileN * (nb - 4)), acc);
         }
     }
 }
 
-struct TmemState {
-    uint32_t base;
-};
-
 // ---- column slices of a small K x N matrix Y (the B operand of k_ozaki_gemm_ws and k_ozaki_update) --
-// yexp[q] = exponent bound of column q over its K rows; blocks[(tn*nkw + kw)*8 + b] (4 KB each) hold
+// yexp[q] = exponent bound of column q over its K rows; blocks[(tn*nkw + kw)*7 + b] (4 KB each) hold
 // slice b of columns 64tn..64tn+63 and rows 32kw..32kw+31 in the core-matrix K-major layout.
 // Y rows >= K and columns >= N read as 0.  One CTA per (tn, kw), 256 threads: (column, 8-row chunk).
 __global__ void __launch_bounds__(256) k_ozaki_slice_cols(const double* __restrict__ Y, int64_t ldy, int K,
@@ -435,7 +393,7 @@ __global__ void __launch_bounds__(256) k_ozaki_slice_cols(const double* __restri
 }
 
 // ---- stage images of X's row slices ------------------------------------------------------------------
-// img[(tm * nkw + kw) * kAStage ..] = the eight 8 KB slices of rows 128 tm .. 128 tm + 127, K values
+// img[(tm * nkw + kw) * kAStage ..] = the seven 8 KB slices of rows 128 tm .. 128 tm + 127, K values
 // 32 kw .. 32 kw + 31 of X, in the core-matrix layout of a k_ozaki_gemm_ws stage buffer, against the row
 // bounds xexp: exactly what that kernel's producers would slice for the stage (zeros outside X).  One
 // CTA per (row tile, K stage), one thread per (row, 8-value chunk).  Skipped when *info != 0.
@@ -459,7 +417,7 @@ __global__ void __launch_bounds__(512) k_slice_images(const double* __restrict__
 }
 
 // ---- stage images of X's column slices (the split Gram's operands) -------------------------------------
-// img[(blk * nst + st) * kAStage ..] = the eight 8 KB slices of columns 128 blk .. 128 blk + 127 (the
+// img[(blk * nst + st) * kAStage ..] = the seven 8 KB slices of columns 128 blk .. 128 blk + 127 (the
 // tile's M dimension) over rows 32 st .. 32 st + 31 (K) of X, against the column bounds colexp, in the
 // layout k_ozaki_gram's producers would slice them (zeros outside X); nst = ceil(m / 32).
 __global__ void __launch_bounds__(512) k_slice_col_images(const double* __restrict__ X, int64_t ldx, int64_t m,
@@ -594,7 +552,7 @@ __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid
 #pragma unroll
                 for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][j];
                 if (col < N) {
-                    const long long I = combine_units53(grp);
+                    const long long I = combine_units<53>(grp);
                     const int ey = yexp[col];
                     const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2(I, E + ey - 53) : 0.0;
                     wr[c0 + j] = v;
@@ -870,26 +828,27 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
 // ---- C = X Y / C = B - X Y from stage images, with the accumulators double-buffered ------------------------
 // The product over pre-sliced X (k_slice_images) for the wide passes: pass 2 (Q = A_1 R_1^{-1}, Y upper
 // triangular) and the left-looking block updates of the first pass (C = B - X Y, K up to 2048).  Output
-// tiles of 128 rows x 32 columns, so that one exactness window's eight group accumulators take 256 TMEM
+// tiles of 128 rows x 32 columns, so that one exactness window's seven group accumulators take 224 TMEM
 // columns and two sets fit: consecutive windows of a CTA (within a tile and across its tiles) alternate
-// between the sets, so a window's drain (the eight FP32 group sums into int64, or the tile's result out
+// between the sets, so a window's drain (the FP32 group sums into int64, or the tile's result out
 // to C) runs while the tensor core fills the other set.  Warp roles: warps 0-7 drain (two threads per
 // tile row, 16 columns each: warp w reads TMEM lanes 32 (w % 4)..), warp 8 lane 0 streams the stages
-// (one 64 KB bulk copy of X's stage image, eight 2 KB copies of Y's slices, on the stage's load barrier),
-// warp 9 lane 0 issues the MMAs (8 per K = 16 step: Y's eight 32-column slices are stacked, N = 32 (9 - a)
+// (one 56 KB bulk copy of X's stage image, seven 2 KB copies of Y's slices, on the stage's load barrier),
+// warp 9 lane 0 issues the MMAs (7 per K = 16 step: Y's seven 32-column slices are stacked, N = 32 (8 - a)
 // for slice a of X).  Barriers: load[s] (bytes landed) and empty[s] (MMAs of the stage done) per stage
 // buffer; acc_full[b] (the window's MMAs done) and acc_empty[b] (the set read out) per accumulator set.
 // The arithmetic is that of k_ozaki_gemm_ws: the same slices, exact group sums per window of 128, the
 // same int64 combination in units of 2^-53, so the results are the same bits.
 constexpr int kDbN = 32;
 constexpr int kDbBSlice = kDbN * kKW * 2;            // 2 KB: one slice of a 32-column tile's stage
-constexpr int kDbBStage = kSlices * kDbBSlice;       // 16 KB
-constexpr int kDbStage = kAStage + kDbBStage;        // 80 KB
+constexpr int kDbBStage = kSlices * kDbBSlice;       // 14 KB
+constexpr int kDbStage = kAStage + kDbBStage;        // 70 KB
 constexpr int kDbEpiWarps = 8;
 constexpr int kDbEpi = 32 * kDbEpiWarps;             // 256 drain threads
 constexpr int kDbThreads = kDbEpi + 64;              // + the copy warp and the MMA warp
 constexpr int kDbCols = kDbN / (kDbEpi / kTileM);    // 16 columns per drain thread
 constexpr int kDbEpiLd = kDbN + 1;
+constexpr int kDbSetCols = 256;                       // TMEM columns between the two accumulator sets (7 x 32 used)
 constexpr int kDbSmem = 2 * kDbStage + kTileM * kDbEpiLd * 8;
 static_assert(kDbSmem + 1024 <= 232448, "k_ozaki_gemm_db exceeds the 227 KB shared-memory limit");
 
@@ -900,17 +859,18 @@ __device__ __forceinline__ int db_tile_stages(int tn, int nkw, bool tri) {
     return last < nkw ? last : nkw;
 }
 
-// The 36 slice pairs of one 32-wide K stage into accumulator set `tset` (group d at columns (d - 2) 32):
-// 8 MMAs per K = 16 step; `first`: the stage opens a window (the a = 1 MMA clears all eight groups).
-__device__ __forceinline__ void issue_stage_n32(uint32_t tset, uint32_t a_base, uint32_t b_base, bool first) {
+// The 28 slice pairs of nkk (1 or 2) K = 16 steps of a stage into accumulator set `tset` (group d at columns (d - 2) 32):
+// 7 MMAs per step, B's seven 32-column slices back to back; `first`: the a = 1 MMA clears all seven groups.
+__device__ __forceinline__ void issue_stage_n32(uint32_t tset, uint32_t a_base, uint32_t b_base, bool first, int nkk = 2) {
     const uint64_t a0 = sdesc(a_base), b0 = sdesc(b_base);
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
+        if (kk >= nkk) break;
 #pragma unroll
-        for (int a = 1; a <= 8; ++a) {
+        for (int a = 1; a <= kSlices; ++a) {
             const uint64_t ad = a0 + static_cast<uint32_t>(((a - 1) * kASlice + kk * 256) >> 4);
-            mma_bf16_n(tset + (a - 1) * kDbN, ad, b0 + static_cast<uint32_t>(kk * 16), idesc_bf16(kDbN * (9 - a)),
-                       (first && kk == 0 && a == 1) ? 0u : 1u);
+            mma_f16_n(tset + (a - 1) * kDbN, ad, b0 + static_cast<uint32_t>(kk * 16), idesc_f16(kDbN * (kSlices + 1 - a)),
+                      (first && kk == 0 && a == 1) ? 0u : 1u);
         }
     }
 }
@@ -922,7 +882,7 @@ __device__ __forceinline__ long long shift_round(long long I, int sh) {
     return (I + (1ll << (sh - 1))) >> sh;
 }
 
-// Add one window's eight group sums of this thread's row (TMEM address taddr: set + lane quarter) and
+// Add one window's group sums of this thread's row (TMEM address taddr: set + lane quarter) and
 // columns col0 .. col0 + NC - 1 of the 32-column tile to int64 accumulators in units of 2^-53 (U49: 2^-49)
 // of the window's scale, shifted down by sh bits (a window sliced against a row bound 2^sh below the
 // tile's).
@@ -939,7 +899,7 @@ __device__ __forceinline__ void drain_set32(uint32_t taddr, int col0, int sh, lo
             float grp[kGroups];
 #pragma unroll
             for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][j];
-            acc[c0 + j] += shift_round(U49 ? combine_units49(grp) : combine_units53(grp), sh);
+            acc[c0 + j] += shift_round(combine_units<U49 ? 49 : 53>(grp), sh);
         }
     }
 }
@@ -1078,7 +1038,7 @@ k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xe
                         break;
                     }
                     tc_after_sync();
-                    issue_stage_n32(tmem + static_cast<uint32_t>(set) * (kGroups * kDbN), smem_u32(stA[s]),
+                    issue_stage_n32(tmem + static_cast<uint32_t>(set) * kDbSetCols, smem_u32(stA[s]),
                                     smem_u32(stB[s]), first);
                     mma_commit(&empty_bar[s]);
                     if (kw % wlen == wlen - 1 || kw == nk - 1) {
@@ -1129,7 +1089,7 @@ k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xe
                     const int ew = bexp[w * ld_bexp + row];
                     sh = ew > kNoExp ? E - ew : 63;
                 }
-                drain_set32<kDbCols>(tmem + lane_off + static_cast<uint32_t>(set) * (kGroups * kDbN), kDbCols * h, sh,
+                drain_set32<kDbCols>(tmem + lane_off + static_cast<uint32_t>(set) * kDbSetCols, kDbCols * h, sh,
                                      acc);
                 tc_before_sync();
                 __syncwarp();
@@ -1182,7 +1142,7 @@ k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xe
 }
 
 // ---- C = B - X Y for K <= 32 (the right-looking updates of the split first pass) -------------------------
-// Tiles of 128 rows x 32 output columns, so that one tile's eight group accumulators take 256 TMEM
+// Tiles of 128 rows x 32 output columns, so that one tile's seven group accumulators take 224 TMEM
 // columns and two tiles are in flight: the tensor core fills one buffer while the other is drained.
 // The X slices of a 128-row block (one K stage) are produced once and used by all N/32 column tiles of
 // the block; the Y slices (at most 128 columns) stay in shared memory for the whole launch.  The X rows
@@ -1202,25 +1162,7 @@ constexpr int kUpdRawOff = 2 * kAStage + (kUpdMaxN / kTileN) * kBStage;  // afte
 constexpr int kUpdSmem = kUpdRawOff + kTileM * kUpdRawLd * 8;            // 225 KB
 static_assert(kUpdSmem + 1024 <= 232448, "k_ozaki_update exceeds the 227 KB shared-memory limit");
 constexpr int kUpdBSlice = kUpdTileN * kKW * 2;                          // 2 KB: one slice of a 32-column tile
-constexpr int kUpdBTile = kSlices * kUpdBSlice;                          // 16 KB: its eight slices
-// The 36 slice pairs of one 32-column tile for nkk K steps of 16 (group d into columns (d - 2) * 32 of
-// the tile's TMEM buffer), 8 MMAs per step: the tile's eight B slices lie back to back (2 KB apart, one
-// 256-row operand), so slice a of X meets slices b = 1 .. 9 - a in one MMA with N = 32 (9 - a) whose
-// accumulators d = a + 1 .. 9 are adjacent.  The first MMA (a = 1, all eight groups) clears them.
-__device__ __forceinline__ void issue_tile_n32(uint32_t tmem, uint32_t a_base, uint32_t b_base, int nkk) {
-    const uint64_t a0 = sdesc(a_base), b0 = sdesc(b_base);
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        if (kk >= nkk) break;
-#pragma unroll
-        for (int a = 1; a <= 8; ++a) {
-            const uint64_t ad = a0 + static_cast<uint32_t>(((a - 1) * kASlice + kk * 256) >> 4);
-            mma_bf16_n(tmem + (a - 1) * kUpdTileN, ad, b0 + static_cast<uint32_t>(kk * 16),
-                       idesc_bf16(kUpdTileN * (9 - a)), (kk == 0 && a == 1) ? 0u : 1u);
-        }
-    }
-}
-
+constexpr int kUpdBTile = kSlices * kUpdBSlice;                          // 14 KB: its seven slices
 __global__ void __launch_bounds__(kUpdThreads, 1)
 k_ozaki_update(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, int K,
                const uint8_t* __restrict__ yblocks, const int32_t* __restrict__ yexp, int N, const double* B,
@@ -1375,7 +1317,7 @@ k_ozaki_update(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, i
                             for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][i];
                             const long long I = combine_units53_k32(grp);
                             const int ey = col < N ? yexp[col] : kNoExp;
-                            const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2(I, E + ey - 53) : 0.0;
+                            const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2_int(I, E + ey - 53) : 0.0;
                             cv[i] = bv[c0 + i] - v;
                         }
 #pragma unroll
@@ -1414,7 +1356,7 @@ k_ozaki_update(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, i
                     }
                     tc_after_sync();
                     const uint32_t bbase = smem_u32(yres) + j * kUpdBTile;
-                    issue_tile_n32(tmem + 256u * b, smem_u32(stA[s]), bbase, nkk);
+                    issue_stage_n32(tmem + 256u * b, smem_u32(stA[s]), bbase, true, nkk);
                     mma_commit(&acc_full[b]);
                 }
                 if (!ok) { abort_s = 1; break; }
@@ -1437,8 +1379,8 @@ k_ozaki_update(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, i
 // ---- Gram partials from column stage images, with the accumulators double-buffered ------------------------
 // Output tiles (P, Qb) of rows p in [128P, 128P+128) (TMEM lanes) x columns q in [32Qb, 32Qb+32), all
 // tiles with Qb >= 4P (every q >= p is covered); grid = ntiles x nranges, CTA (tile, rr) sums the rows
-// [rr*rows_per, ...) of the launch.  A = P's 128-column stage image (64 KB), B = rows 32 (Qb % 4).. of
-// each slice of block Qb / 4's image (eight 2 KB copies); windows of 128 rows alternate between the two
+// [rr*rows_per, ...) of the launch.  A = P's 128-column stage image (56 KB), B = rows 32 (Qb % 4).. of
+// each slice of block Qb / 4's image (seven 2 KB copies); windows of 128 rows alternate between the two
 // TMEM sets as in k_ozaki_gemm_db, each drained into int64 in units of 2^-49 and, every 64 windows and
 // at the end, added into the CTA's FP64 partial (accum: the launch adds into partials of earlier row
 // chunks).  The same slices, sums and flush points as k_ozaki_gram's 64-column tiles: the same bits.
@@ -1495,7 +1437,7 @@ k_ozaki_gram_db(int64_t m, int n, int np, const int32_t* __restrict__ colexp, in
             bool ok = true;
             const uint8_t* abase = gimg + static_cast<size_t>(P) * nsg * kAStage;
             const uint8_t* bbase = gimg + static_cast<size_t>(Qb >> 2) * nsg * kAStage + (Qb & 3) * kDbBSlice;
-            // L2 prefetch of the stage kPrefetchAhead ahead (A stage and B's eight slices)
+            // L2 prefetch of the stage kPrefetchAhead ahead (A stage and B's slices)
             auto prefetch = [&](int64_t pst) {
                 if (pst >= nstages) return;
                 const size_t sg = static_cast<size_t>(r0 / kKW + pst);
@@ -1544,7 +1486,7 @@ k_ozaki_gram_db(int64_t m, int n, int np, const int32_t* __restrict__ colexp, in
                     break;
                 }
                 tc_after_sync();
-                issue_stage_n32(tmem + static_cast<uint32_t>(set) * (kGroups * kDbN), smem_u32(stA[s]), smem_u32(stB[s]),
+                issue_stage_n32(tmem + static_cast<uint32_t>(set) * kDbSetCols, smem_u32(stA[s]), smem_u32(stB[s]),
                                 first);
                 mma_commit(&empty_bar[s]);
                 if ((st & 3) == 3 || st == nstages - 1) {
@@ -1593,7 +1535,7 @@ k_ozaki_gram_db(int64_t m, int n, int np, const int32_t* __restrict__ colexp, in
                 break;
             }
             tc_after_sync();
-            drain_set32<kDbCols, true>(tmem + lane_off + static_cast<uint32_t>(set) * (kGroups * kDbN), kDbCols * h, 0,
+            drain_set32<kDbCols, true>(tmem + lane_off + static_cast<uint32_t>(set) * kDbSetCols, kDbCols * h, 0,
                                        acc);
             tc_before_sync();
             __syncwarp();
@@ -1622,8 +1564,8 @@ k_ozaki_gram_db(int64_t m, int n, int np, const int32_t* __restrict__ colexp, in
 // X: m x n FP64 (ldx), column exponent bounds colexp[n] over all m rows.  Output tiles (P, Qb): rows
 // p in [128P, 128P+128) (TMEM lanes) x columns q in [64Qb, 64Qb+64), all tiles with Qb >= 2P (every
 // q >= p is covered).  Grid = ntiles x nranges CTAs; CTA (tile, rr) accumulates the rows
-// [rr*rows_per, ...) and writes gpart[rr][p][q] (np x np) for its tile.  The B operand reuses the A
-// slices when its 64 columns lie inside the P block, else it is sliced into its own stage.  Exactness
+// [rr*rows_per, ...) and writes gpart[rr][p][q] (np x np) for its tile.  B's 64 columns
+// have a stage of their own, sliced apart from A's where they lie outside the P block.  Exactness
 // windows of 128 rows are drained into int64 accumulators in units of 2^-49 of the scale 2^(Ep+Eq)
 // (one output row per thread, 32 columns); every 64 windows (8192 rows, |sum| < 2^63 even for maximal
 // slices) they are added into the CTA's own FP64 partial and cleared.
@@ -1637,17 +1579,12 @@ __device__ __forceinline__ void gram_tile_coords(int nqb, int tt, int& P, int& Q
 // sliced, one arrival per producer warp; empty[s]: its MMAs done).  A window's drain waits for the
 // MMAs of the stage before and arrives on full of the next stage only after reading TMEM.
 constexpr int kGramNT = kThreads;
-// PRE: the column slices of every (128-column block, 32-row stage) of this launch's rows were made
-// beforehand by k_slice_col_images (gimg): A is one 64 KB copy per stage, B (when it is not part of A)
-// the matching half of another block's image.  accum: add into the partials instead of starting them
-// (the launch is one of several row chunks summed in order).
-template <bool PRE>
 __global__ void __launch_bounds__(kGramNT + 32, 1)
 k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np,
              const int32_t* __restrict__ colexp, int64_t rows_per, int ntiles, double* __restrict__ gpart,
-             int32_t* info, long spin, const uint8_t* __restrict__ gimg, int accum) {
+             int32_t* info, long spin) {
     extern __shared__ __align__(1024) uint8_t sm[];
-    __shared__ uint64_t empty_bar[2], full_bar[2], load_bar[2], done_bar;
+    __shared__ uint64_t empty_bar[2], full_bar[2], done_bar;
     __shared__ uint32_t tslot;
     __shared__ int abort_s;
     if (load_status(info) != 0) return;
@@ -1673,7 +1610,6 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
         for (int i = 0; i < 2; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty_bar[i])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&full_bar[i])), "r"(NT / 32));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&load_bar[i])));
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&done_bar)));
         asm volatile("fence.mbarrier_init.release.cluster;\n");
@@ -1687,22 +1623,16 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
 
     if (warp == NT / 32) {
         if (lane == 0) {
-            uint32_t fphase[2] = {0u, 0u}, lphase[2] = {0u, 0u};
-            const uint32_t boff = b_inside ? static_cast<uint32_t>(((64 * Qb - 128 * P) / 8) * kSBO) : 0u;
+            uint32_t fphase[2] = {0u, 0u};
             for (int64_t st = 0; st < nstages; ++st) {
                 const int s = static_cast<int>(st & 1);
-                if (!mbar_wait_ab(&full_bar[s], fphase[s], &abort_s, spin) ||
-                    (PRE && !mbar_wait_ab(&load_bar[s], lphase[s], &abort_s, spin))) {
+                if (!mbar_wait_ab(&full_bar[s], fphase[s], &abort_s, spin)) {
                     abort_s = 1;
                     break;
                 }
                 fphase[s] ^= 1u;
-                lphase[s] ^= 1u;
                 tc_after_sync();
-                if (!PRE && b_inside)
-                    issue_stage_pairs(tmem, smem_u32(stA[s]), smem_u32(stA[s]) + boff, kASlice, (st & 3) == 0);
-                else
-                    issue_stage(tmem, smem_u32(stA[s]), smem_u32(stB[s]), (st & 3) == 0);
+                issue_stage(tmem, smem_u32(stA[s]), smem_u32(stB[s]), (st & 3) == 0);
                 mma_commit(&empty_bar[s]);
             }
             mma_commit(&done_bar);
@@ -1714,17 +1644,19 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
         const int rq = tid >> 7;                // producer row chunk(s) NCH*rq..; drain columns kCols*rq..
         const int p = 128 * P + lr;
         const int Ep = p < n ? colexp[p] : kNoExp;
+        // where B's columns lie inside the P block the threads that slice them store them into B's stage too (back to back
+        // there, for the stacked MMAs: one N = 64 MMA per pair took 1.3 of the Gram's 1.9 ms at 2^20 x 128)
+        const int b_row = b_inside && p >= 64 * Qb && p < 64 * Qb + 64 ? p - 64 * Qb : -1;
         long long acc[kCols];
 #pragma unroll
         for (int j = 0; j < kCols; ++j) acc[j] = 0;
         uint32_t phase[2] = {0u, 0u};
         bool pending[2] = {false, false};
         bool timed_out = false;
-        int64_t issued[2] = {0, 0};         // bulk copies issued into each stage buffer (PRE, thread 0)
 
         // Drain the window just finished (its MMAs complete) into acc; every 64 windows, and at the end,
         // add acc into the CTA's FP64 partial (the first flush initialises it) and clear it.
-        bool flushed = accum != 0;
+        bool flushed = false;
         auto drain_window = [&](bool flush) {
             tc_after_sync();
             drain_acc<false, kCols, 4>(tmem, warp, kCols * rq, acc);
@@ -1755,24 +1687,6 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
                 pending[s] = false;
             }
             const int64_t k0 = r0 + st * kKW;
-            if constexpr (PRE) {
-                // A: the P block's 64 KB stage image; B (columns 64 Qb .. 64 Qb + 63): half (Qb & 1) of every
-                // slice of block Qb / 2's image (P's own when they lie inside the P block), eight 4 KB pieces
-                // placed back to back for the stacked MMAs.  Bulk copies on the stage's load barrier.
-                if (tid == 0) {
-                    const int64_t sg = k0 / kKW, nsg = (m + kKW - 1) / kKW;
-                    const uint8_t* asrc = gimg + static_cast<size_t>(P * nsg + sg) * kAStage;
-                    const uint8_t* bsrc = gimg + static_cast<size_t>((Qb >> 1) * nsg + sg) * kAStage +
-                                          (Qb & 1) * kBSlice;
-                    mbar_expect_tx(&load_bar[s], kAStage + kBStage);
-                    bulk_g2s(stA[s], asrc, kAStage, &load_bar[s]);
-#pragma unroll
-                    for (int a = 0; a < kSlices; ++a)
-                        bulk_g2s(stB[s] + a * kBSlice, bsrc + static_cast<size_t>(a) * kASlice, kBSlice, &load_bar[s]);
-                    ++issued[s];
-                }
-            }
-            if constexpr (!PRE) {
 #pragma unroll
             for (int cc = 0; cc < NCH; ++cc) {
                 const int c = NCH * rq + cc;
@@ -1782,10 +1696,10 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
                     const int64_t row = k0 + 8 * c + i;
                     x[i] = (row < r1 && p < n) ? X[row * ldx + p] : 0.0;
                 }
-                slice_store8(x, Ep, stA[s] + core_off(lr, 16 * c), kASlice);
+                slice_store8(x, Ep, stA[s] + core_off(lr, 16 * c), kASlice,
+                             b_row >= 0 ? stB[s] + core_off(b_row, 16 * c) : nullptr, kBSlice);
             }
-            }
-            if (!PRE && !b_inside) {
+            if (!b_inside) {
                 for (int e = tid; e < 4 * 64; e += NT) {
                     const int c = e >> 6, col = 64 * Qb + (e & 63);   // 64 columns x 4 chunks of 8 rows
                     const int Ec = col < n ? colexp[col] : kNoExp;
@@ -1824,10 +1738,9 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
                 }
             if (!timed_out) drain_window(true);
         }
-        if (PRE && tid == 0 && !bulk_drain(load_bar, issued)) timed_out = true;
         if (timed_out) {
             abort_s = 1;
-        } else if (nstages == 0 && p < np && !accum) {
+        } else if (nstages == 0 && p < np) {
             double* out = gpart + static_cast<size_t>(rr) * np * np + static_cast<size_t>(p) * np;
             for (int j = 0; j < kCols; ++j) {
                 const int q = 64 * Qb + kCols * rq + j;
@@ -1986,14 +1899,13 @@ cudaError_t launch_ozaki_gram(const double* X, int64_t ldx, int64_t m, int n, in
         return cudaGetLastError();
     }
     const int smem = 2 * (oz::kAStage + oz::kBStage);
-    auto kern = oz::k_ozaki_gram<false>;
+    auto kern = oz::k_ozaki_gram;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err != cudaSuccess) return err;
     const int nt = ozaki_gram_halves(np);
     int64_t rows_per = (m + nranges - 1) / nranges;
     rows_per = (rows_per + oz::kKW - 1) / oz::kKW * oz::kKW;
-    kern<<<nt * nranges, oz::kGramNT + 32, smem, st>>>(X, ldx, m, n, np, colexp, rows_per, nt, gpart, info, spin,
-                                                       gimg, accum ? 1 : 0);
+    kern<<<nt * nranges, oz::kGramNT + 32, smem, st>>>(X, ldx, m, n, np, colexp, rows_per, nt, gpart, info, spin);
     return cudaGetLastError();
 }
 
