@@ -601,13 +601,15 @@ __device__ __forceinline__ int tile_stages(int tn, int nkw, bool tri) {
     return last < nkw ? last : nkw;
 }
 
-// Column tile of tile t (row tile t / ntn).  With a triangular Y the tiles' costs differ (2 (tn + 1)
-// stages), and a grid that is a multiple of ntn would give every CTA one fixed tn: the column tile is
-// rotated by the row tile, so a CTA's tiles t, t + gridDim.x, ... cycle through all tn, while the ntn
-// tiles of one row tile still run side by side (their A stages shared in L2).
+// Column tile of tile t (row tile t / ntn).  With a triangular Y the tiles' costs differ (2 (tn + 1) stages), so a CTA's
+// tiles t, t + gridDim.x, ... must cycle through all tn, while the ntn tiles of one row tile still run side by side
+// (their A stages shared in L2): the column tile is rotated by the CTA's turn where the grid is a multiple of ntn
+// (every tile of a row tile is then in the same turn), else by the row tile.  (Rotating by the row tile alone gave each
+// CTA one fixed tn at ntn = 2 and 152 CTAs: the SMs were busy 79 % of the time.)
 __device__ __forceinline__ int tile_col(int64_t t, int ntn, bool tri) {
     const int j = static_cast<int>(t % ntn);
-    return tri ? static_cast<int>((j + t / ntn) % ntn) : j;
+    if (!tri) return j;
+    return static_cast<int>((j + (gridDim.x % ntn == 0 ? t / gridDim.x : t / ntn)) % ntn);
 }
 
 // Walks the stages of the output tiles one CTA owns (tiles t = blockIdx.x, + gridDim.x, ...; stages
@@ -1589,7 +1591,8 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
     __shared__ int abort_s;
     if (load_status(info) != 0) return;
     constexpr int NT = kGramNT;
-    constexpr int kCols = Share<NT>::kDrainCols, NCH = Share<NT>::kChunks;
+    constexpr int kCols = Share<NT>::kDrainCols;
+    static_assert(Share<NT>::kChunks == 1, "one 8-row chunk per producer thread");
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nqb = (np + kTileN - 1) / kTileN;
     int P, Qb;
@@ -1641,7 +1644,7 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
         __syncwarp();
     } else {
         const int lr = tid & 127;               // TMEM lane: output row p = 128P + lr; producer column of A
-        const int rq = tid >> 7;                // producer row chunk(s) NCH*rq..; drain columns kCols*rq..
+        const int rq = tid >> 7;                // producer row chunk rq; drain columns kCols*rq..
         const int p = 128 * P + lr;
         const int Ep = p < n ? colexp[p] : kNoExp;
         // where B's columns lie inside the P block the threads that slice them store them into B's stage too (back to back
@@ -1676,6 +1679,16 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
             if (flush) flushed = true;
         };
 
+        // this thread's eight values of a stage: column p, rows 8 rq .. of the stage
+        double xv[8];
+        auto load_x = [&](int64_t st) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int64_t row = r0 + st * kKW + 8 * rq + i;
+                xv[i] = (row < r1 && p < n) ? X[row * ldx + p] : 0.0;
+            }
+        };
+        load_x(0);
         // Stage st is sliced into buffer st & 1 while the MMAs of stage st - 1 run; a stage that opens a
         // window first drains the previous window (after being produced, before it is handed over).
         for (int64_t st = 0; st < nstages; ++st) {
@@ -1687,18 +1700,9 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
                 pending[s] = false;
             }
             const int64_t k0 = r0 + st * kKW;
-#pragma unroll
-            for (int cc = 0; cc < NCH; ++cc) {
-                const int c = NCH * rq + cc;
-                double x[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int64_t row = k0 + 8 * c + i;
-                    x[i] = (row < r1 && p < n) ? X[row * ldx + p] : 0.0;
-                }
-                slice_store8(x, Ep, stA[s] + core_off(lr, 16 * c), kASlice,
-                             b_row >= 0 ? stB[s] + core_off(b_row, 16 * c) : nullptr, kBSlice);
-            }
+            slice_store8(xv, Ep, stA[s] + core_off(lr, 16 * rq), kASlice,
+                         b_row >= 0 ? stB[s] + core_off(b_row, 16 * rq) : nullptr, kBSlice);
+            load_x(st + 1);   // in flight until the next stage's slicing
             if (!b_inside) {
                 for (int e = tid; e < 4 * 64; e += NT) {
                     const int c = e >> 6, col = 64 * Qb + (e & 63);   // 64 columns x 4 chunks of 8 rows
