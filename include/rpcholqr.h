@@ -101,9 +101,8 @@ rpcholqr_status rpcholqr_plan_create(rpcholqr_plan* plan, int device, rpcholqr_m
  * (uniform entries; any full-rank matrix serves), times rpcholqr_factor on it -- one warm-up and `reps`
  * timed calls, CUDA events -- for every candidate set of launch parameters, and keeps the fastest in the
  * plan's table under (mode, padded n, ceil(log2 m)):
- *   SPLIT64: the width of the first pass's FP64 diagonal-block solves (16 or 32 columns; the rest of
- *            the solve is split tensor-core updates) x the row ranges (split-K factor) of the Gram
- *            matrix (the built-in rule, one per SM over the output tiles, twice that);
+ *   SPLIT64: the row ranges (split-K factor) of the Gram matrix (the built-in rule, one per SM over the output
+ *            tiles, twice that); "split_sub" records the width of the first pass's FP64 substitutions (16);
  *   FP64, n > 128: the row ranges (split-K factor) of the wide Gram matrix (x1, x4 of one wave).
  * Other shapes are timed with the built-in rules and recorded as such.  out_json (nullable): file the
  * whole table is written to (the format rpcholqr_plan_create reads).  Synchronous; allocates and frees

@@ -63,6 +63,11 @@ void launch_slice_images(const double* X, int64_t ldx, int64_t m, int K, const i
                          const int32_t* info, cudaStream_t st);
 void launch_slice_block_images(const double* X, int64_t ldx, int64_t m, int nc, uint8_t* img, int img_nkw, int kw0,
                                int32_t* bexp, const int32_t* info, cudaStream_t st);
+size_t split_solve_tab_bytes(int n);
+void launch_split_solve_prep(const double* T, int64_t ldt, int n, uint8_t* tab, const int32_t* info, cudaStream_t st);
+cudaError_t launch_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int nc, const uint8_t* tab, int J,
+                               int32_t* rowexp, int rowexp_mode, int32_t* colexp, int32_t* info, int sms, cudaStream_t st,
+                               long spin);
 int ozaki_gram_halves(int np);
 int ozaki_gram_tiles(int np, bool images);
 cudaError_t launch_ozaki_gram(const double* X, int64_t ldx, int64_t m, int n, int np, const int32_t* colexp,
@@ -139,7 +144,7 @@ constexpr int64_t kDefaultSpinLimit = int64_t{1} << 24;
 
 // Launch parameters the autotuner chooses (rpcholqr_autotune); 0 = the built-in rule.
 struct Tuning {
-    int32_t split_sub = 0;      // SPLIT64 first pass: width of the FP64 diagonal-block solves (16 or 32)
+    int32_t split_sub = 0;      // SPLIT64 first pass: width of the FP64 diagonal-block solves (16; recorded only)
     int32_t gram_ranges = 0;    // SPLIT64 Gram: row ranges (split-K factor of G = A1^T A1)
     int32_t syrk_ranges = 0;    // FP64 Gram of wide panels: row ranges
 };
@@ -219,6 +224,7 @@ struct rpcholqr_plan_s {
     int32_t* colexp = nullptr;  // np
     int32_t* yexp = nullptr;    // np
     uint8_t* yblocks = nullptr; // Ozaki column slices (K, N <= np)
+    uint8_t* sstab = nullptr;   // tables of the first pass's diagonal blocks (split_solve_tab_bytes)
     // stage images (np > 128; separate allocation img_ws), img_rows rows at a time: the wide first pass's
     // row slices of finished column blocks, then the Gram's column slices of A1, then pass 2's row slices
     // of A1; when they cover every row each pass is a single launch over all rows
@@ -374,17 +380,9 @@ double ozaki_flops(bool sub, bool y_upper, int64_t m, int K, int N) {
     return per_row * m;
 }
 
-constexpr int kBlk = 64;   // column block of the FP64 blocked solves (n > 128)
-// Blocks of the split mode's first pass: the FP64 row passes solve split_sub-column diagonal blocks
-// (FP64 work per row n * split_sub); the rest of the solve runs as split tensor-core updates, K =
-// kSplitBlk across blocks and K = split_sub inside one (n <= 128; wider, 64-column blocks).  At
-// m = 2^20, n = 128, sub-blocks of 16 measured the same step time as 32 (13.75 vs 13.79 ms: the FP64
-// work halves, the extra K = 16 updates cost as much), so up to 128 columns the blocks are not split; at
-// m = 2^23, n = 512, 16 took the step from 558 to 540 ms (row passes 159 -> 96 ms, updates 32 -> 76 ms),
-// so wider matrices take 16.
-constexpr int kSplitBlk = 32;
-constexpr int kSplitSub = 32;
-constexpr int kSplitSubWide = 16;
+constexpr int kBlk = 64;   // column block of the blocked solves (FP64: n > 128)
+// Width of the FP64 substitutions inside a 64-column block of the split mode's first pass (k_split_solve).
+constexpr int kSplitSub = 16;
 // Split mode: the explicit-inverse second pass is used while ||R1||_F ||R1^{-1}||_F / n <= this
 // (1.1-1.25 for well-sampled incoherent A; the estimate lies in [kappa(A1)/n, kappa(A1)]; at 3.3
 // (kappa(A1) ~ 30) the explicit inverse already costs 10x in residual).
@@ -414,12 +412,6 @@ void select_tuning(rpcholqr_plan_s* p, int64_t m, int n) {
         }
     }
     p->cur_tune = t;
-}
-
-// Width of the SPLIT64 first pass's FP64 diagonal-block solves for the current call.
-int split_sub(const rpcholqr_plan_s* p) {
-    const int v = p->cur_tune.split_sub;
-    return v == 16 || v == 32 ? v : (p->cur_np > kMaxNP ? kSplitSubWide : kSplitSub);
 }
 
 // The smoothed sample of the plan's kind into p->As (column-major, ld s, np columns).
@@ -638,11 +630,12 @@ rpcholqr_status rpcholqr_workspace_size(rpcholqr_plan p, int64_t max_m, int32_t 
     const int32_t ws_n = mode == RPCHOLQR_FP32 ? (max_n + 63) / 64 * 64 : max_n;
     size_t total = ws_layout(ws_n, max_s, gram_parts(mode, max_m, max_n, grid)).total;
     const size_t np = static_cast<size_t>(pad_np(max_n));
-    if (mode == RPCHOLQR_SPLIT64)   // A1, row/column bounds, column slices, R1^{-1}, gate words
+    if (mode == RPCHOLQR_SPLIT64)   // A1, row/column bounds, column slices, R1^{-1}, gate words, diagonal-block tables
         total += align256(sizeof(double) * static_cast<size_t>(max_m) * np) +
                  align256(sizeof(int32_t) * static_cast<size_t>(max_m)) + 2 * align256(sizeof(int32_t) * np) +
                  align256(ozaki_yblocks_bytes(static_cast<int>(np), static_cast<int>(np))) +
-                 align256(sizeof(double) * np * np) + align256(sizeof(int32_t) * 8);
+                 align256(sizeof(double) * np * np) + align256(sizeof(int32_t) * 8) +
+                 align256(split_solve_tab_bytes(static_cast<int>(np)));
     if (mode == RPCHOLQR_SPLIT64 && np > static_cast<size_t>(kMaxNP)) {   // stage images
         int device = 0;
         if (p) device = p->device;
@@ -742,6 +735,7 @@ rpcholqr_status rpcholqr_plan_create(rpcholqr_plan* plan, int device, rpcholqr_m
         const size_t oB = take(ozaki_yblocks_bytes(p->np, p->np));
         const size_t oW = take(sizeof(double) * np * np);
         const size_t oG = take(sizeof(int32_t) * 8);
+        const size_t oS = take(split_solve_tab_bytes(p->np));
         if (cudaMalloc(&p->split_ws, off) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(p->ws);
@@ -756,6 +750,7 @@ rpcholqr_status rpcholqr_plan_create(rpcholqr_plan* plan, int device, rpcholqr_m
         p->yblocks = reinterpret_cast<uint8_t*>(c + oB);
         p->W = reinterpret_cast<double*>(c + oW);
         p->gates = reinterpret_cast<int32_t*>(c + oG);
+        p->sstab = reinterpret_cast<uint8_t*>(c + oS);
         if (cudaMemset(p->gates, 0, sizeof(int32_t) * 8) != cudaSuccess) cudaGetLastError();
         p->ws_bytes += off;
         if (np > static_cast<size_t>(kMaxNP) && alloc_images(p, 0) != RPCHOLQR_OK) {
@@ -927,63 +922,38 @@ static void prep_blocks(rpcholqr_plan_s* p, const double* T, int64_t ldt, int n,
     ++p->launches;
 }
 
-// Right-looking blocked row solve for the split mode, Y = X T^{-1}, two-level: over kSplitBlk-column
-// blocks J, each solved as two kSplitSub-column halves.  A half is solved by the FP64 row pass,
-// Y[:, h] <- (current X[:, h]) T[h, h]^{-1}; after the first half, the second half is updated by one
-// split tensor-core product with K = N = kSplitSub; after the block, every later column is updated at
-// once, Y[:, >J] = (X or Y)[:, >J] - Y[:, J] T[J, >J], by one split product with K = kSplitBlk (one
-// exactness stage) and N = the remaining width.  The FP64 work per row is n * kSplitSub.  The diagonal
-// blocks must have been set up by prep_blocks with blk = kSplitSub.  The row passes store (first half)
-// and max-merge the row bounds of Y into p->xexp (the updates' left operands use the bound over the
-// columns solved so far) and their column bounds into p->colexp.  Marks PASS1 / PASS1_UPDATE /
-// PASS1_SOLVE2 as the first row pass / the first update / the rest when pm is given.  row0: X's first
-// row within the matrix whose row bounds p->xexp holds (a block of rows is solved on its own).
-static rpcholqr_status solve_split_right(rpcholqr_plan_s* p, const double* X, int64_t ldx, const double* T,
-                                         int64_t ldt, int64_t m, int n, double* Y, int64_t ldy, const double* frag,
-                                         const double* diag, int32_t* info, cudaStream_t st, const PhaseMarks* pm,
-                                         int64_t row0 = 0) {
-    const int grid = p->grid;
-    const int blk = kSplitBlk, sub = split_sub(p);
-    bool first_update = true;
-    auto update = [&](int c0, int K, int c1, int N, const double* B, int64_t ldb) -> rpcholqr_status {
-        if (pm && first_update) pm->mark(RPCHOLQR_PHASE_PASS1_UPDATE);
-        rpcholqr_status rc = ozaki_gemm_internal(p, true, Y + c0, m, K, ldy, T + static_cast<int64_t>(c0) * ldt + c1,
-                                                 N, ldt, B, ldb, Y + c1, ldy, info, st, true, row0);
-        if (pm && first_update) pm->mark(RPCHOLQR_PHASE_PASS1_SOLVE2);
-        first_update = false;
-        return rc;
-    };
-    for (int J = 0; J * blk < n; ++J) {
-        const int c0 = J * blk;
-        const int nj = n - c0 < blk ? n - c0 : blk;
-        for (int h = 0; h * sub < nj; ++h) {
-            const int c1 = c0 + h * sub;
-            const int nh = nj - h * sub < sub ? nj - h * sub : sub;
-            // column c1 still holds A only in the very first half; later ones were written by an update
-            const double* src = c1 == 0 ? X : Y;
-            const int64_t lsrc = c1 == 0 ? ldx : ldy;
-            const int js = c1 / sub;
-            {
-                KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(m) * nh * nh);
-                if (launch_rowpass_ex(false, pad16(nh), src + c1, lsrc, Y + c1, ldy, m, nh, frag + js * sub * sub,
-                                      diag + js * (sub / 8) * 64, nullptr, info, grid, st, true, p->xexp + row0,
-                                      c1 == 0 ? 1 : 2, p->colexp + c1) != cudaSuccess)
-                    return RPCHOLQR_ERR_CUDA;
-            }
-            ++p->launches;
-            if (h == 0 && nj > nh) {
-                const rpcholqr_status rc = update(c1, nh, c1 + nh, nj - nh, (J == 0 ? X : Y) + c1 + nh,
-                                                  J == 0 ? ldx : ldy);
-                if (rc != RPCHOLQR_OK) return rc;
-            }
-        }
-        const int rest = n - c0 - nj;
-        if (rest > 0) {
-            const rpcholqr_status rc = update(c0, nj, c0 + nj, rest, (J == 0 ? X : Y) + c0 + nj, J == 0 ? ldx : ldy);
-            if (rc != RPCHOLQR_OK) return rc;
-        }
+// One 64-column diagonal block of the split first pass (block J of T's tables in p->sstab) on `rows` rows.
+static rpcholqr_status solve_split_block(rpcholqr_plan_s* p, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t rows,
+                                         int nc, int J, int64_t row0, int32_t* info, cudaStream_t st) {
+    KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(rows) * nc * kSplitSub);
+    ++p->launches;
+    return launch_split_solve(X, ldx, Y, ldy, rows, nc, p->sstab, J, p->xexp + row0, J == 0 ? 1 : 2, p->colexp + J * kBlk, info,
+                              p->grid, st, static_cast<long>(p->spin_limit)) == cudaSuccess
+               ? RPCHOLQR_OK
+               : RPCHOLQR_ERR_CUDA;
+}
+
+// The SPLIT64 first pass without stage images (up to 128 columns), Y = X T^{-1} (T = R_s upper triangular, tables in
+// p->sstab), left-looking over 64-column blocks: block J is first Y[:, J] = X[:, J] - Y[:, <J] T[<J, J] (split product;
+// the left operand's row bounds are those over the columns solved so far), then solved (solve_split_block).  The
+// block solves store and max-merge the row bounds of Y into p->xexp and its column bounds into p->colexp.  Marks
+// PASS1_UPDATE / PASS1_SOLVE2 around the first product when pm is given.  row0: X's first row within the matrix
+// whose row bounds p->xexp holds (a block of rows is solved on its own).
+static rpcholqr_status solve_split(rpcholqr_plan_s* p, const double* X, int64_t ldx, const double* T, int64_t ldt, int64_t m,
+                                   int n, double* Y, int64_t ldy, int32_t* info, cudaStream_t st, const PhaseMarks* pm,
+                                   int64_t row0 = 0) {
+    for (int J = 0; J * kBlk < n; ++J) {
+        const int c0 = J * kBlk, nj = n - c0 < kBlk ? n - c0 : kBlk;
+        if (pm && J == 1) pm->mark(RPCHOLQR_PHASE_PASS1_UPDATE);
+        rpcholqr_status rc = RPCHOLQR_OK;
+        if (J > 0)
+            rc = ozaki_gemm_internal(p, true, Y, m, c0, ldy, T + c0, nj, ldt, X + c0, ldx, Y + c0, ldy, info, st, true, row0);
+        if (rc != RPCHOLQR_OK) return rc;
+        if (pm && J == 1) pm->mark(RPCHOLQR_PHASE_PASS1_SOLVE2);
+        rc = solve_split_block(p, (J == 0 ? X : Y) + c0, J == 0 ? ldx : ldy, Y + c0, ldy, m, nj, J, row0, info, st);
+        if (rc != RPCHOLQR_OK) return rc;
     }
-    if (pm && first_update) {
+    if (pm && n <= kBlk) {
         pm->mark(RPCHOLQR_PHASE_PASS1_UPDATE);
         pm->mark(RPCHOLQR_PHASE_PASS1_SOLVE2);
     }
@@ -994,20 +964,16 @@ static rpcholqr_status solve_split_right(rpcholqr_plan_s* p, const double* X, in
 // 64-column blocks, one row chunk (p->img_rows rows) at a time so that the chunk's stage image holds the
 // slices of every finished block: block J of a chunk is first Y[:, J] = X[:, J] - Y[:, <J] T[<J, J], one
 // split product over the image of blocks < J (each pair of blocks one exactness window, sliced against
-// the row's bound over that pair alone), then its sub-block FP64 row passes joined by K = sub split
-// updates (as in solve_blocked), and the finished block is sliced into the image (an odd block together
-// with its even partner, which was sliced alone before).  The row passes max-merge
+// the row's bound over that pair alone), then solved (solve_split_block), and the finished block is sliced into the
+// image (an odd block together with its even partner, which was sliced alone before).  The block solves max-merge
 // the bounds of the whole row into p->xexp (pass 2 slices against them) and of each column into
 // p->colexp.  Marks PASS1_UPDATE / PASS1_SOLVE2 around the first chunk's first product.
 static rpcholqr_status solve_split_wide(rpcholqr_plan_s* p, const double* X, int64_t ldx, const double* T,
-                                        int64_t ldt, int64_t m, int n, double* Y, int64_t ldy, const double* frag,
-                                        const double* diag, int32_t* info, cudaStream_t st, const PhaseMarks* pm) {
+                                        int64_t ldt, int64_t m, int n, double* Y, int64_t ldy, int32_t* info, cudaStream_t st, const PhaseMarks* pm) {
     const int img_nkw = (n + 31) / 32;
-    const int sub = split_sub(p);
     bool marked = false;
     for (int64_t r0 = 0; r0 < m; r0 += p->img_rows) {
         const int64_t rows = m - r0 < p->img_rows ? m - r0 : p->img_rows;
-        const int grid = p->grid;
         const double* Xc = X + r0 * ldx;
         double* Yc = Y + r0 * ldy;
         for (int J = 0; J * kBlk < n; ++J) {
@@ -1025,33 +991,9 @@ static rpcholqr_status solve_split_wide(rpcholqr_plan_s* p, const double* X, int
                     marked = true;
                 }
             }
-            for (int h = 0; h * sub < nj; ++h) {
-                const int c1 = c0 + h * sub;
-                const int nh = nj - h * sub < sub ? nj - h * sub : sub;
-                const bool from_input = J == 0 && h == 0;
-                const double* hsrc = (from_input ? Xc : Yc) + c1;
-                const int64_t lh = from_input ? ldx : ldy;
-                const int js = c1 / sub;
-                {
-                    KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(rows) * nh * nh);
-                    if (launch_rowpass_ex(false, pad16(nh), hsrc, lh, Yc + c1, ldy, rows, nh, frag + js * sub * sub,
-                                          diag + js * (sub / 8) * 64, nullptr, info, grid, st, true, p->xexp + r0,
-                                          c1 == 0 ? 1 : 2, p->colexp + c1) != cudaSuccess)
-                        return RPCHOLQR_ERR_CUDA;
-                }
-                ++p->launches;
-                const int rest = c0 + nj - (c1 + nh);
-                if (rest > 0) {
-                    // the block's first sub-block update reads its input columns (X for block 0, else the
-                    // product's output in Y), later ones the updated columns
-                    const double* B = (from_input ? Xc : Yc) + c1 + nh;
-                    const int64_t ldb = from_input ? ldx : ldy;
-                    rpcholqr_status rc = ozaki_gemm_internal(p, true, Yc + c1, rows, nh, ldy,
-                                                             T + static_cast<int64_t>(c1) * ldt + c1 + nh, rest, ldt,
-                                                             B, ldb, Yc + c1 + nh, ldy, info, st, true, r0);
-                    if (rc != RPCHOLQR_OK) return rc;
-                }
-            }
+            const rpcholqr_status rc = solve_split_block(p, (J == 0 ? Xc : Yc) + c0, J == 0 ? ldx : ldy, Yc + c0, ldy, rows, nj,
+                                                         J, r0, info, st);
+            if (rc != RPCHOLQR_OK) return rc;
             if (c0 + nj < n) {
                 // the products' exactness windows are pairs of blocks (K = 128) with their own row bound: an
                 // even block is sliced alone (the last window of block J + 1's update), an odd one re-slices
@@ -1066,18 +1008,13 @@ static rpcholqr_status solve_split_wide(rpcholqr_plan_s* p, const double* X, int
     return check_launch();
 }
 
-// Left-looking blocked row solve Y = X T^{-1} (T upper triangular, n x n, ld ldt) over 64-column
-// blocks J:  Y[:, J] = X[:, J] - Y[:, <J] T[<J, J]  (FP64 mma, or the split tensor-core product when
-// split), then Y[:, J] <- Y[:, J] T[J, J]^{-1} by the row pass (NP = 64; split: two 32-column row
-// passes and a K = 32 split update between them, so the FP64 work per row is n * 32).  Y may equal X
-// (ldy == ldx).  The diagonal blocks must have been set up by prep_blocks (split: with blk =
-// kSplitSub).  split: the row passes store (block 0) and
-// max-merge (later blocks) the row bounds of Y into p->xexp and max-merge its column bounds into
-// p->colexp, both needed by the split products; marks PASS1 / PASS1_UPDATE / PASS1_SOLVE2 when
-// pass1_marks (blocks 2.. fall in PASS1_SOLVE2).
+// Left-looking blocked FP64 row solve Y = X T^{-1} (T upper triangular, n x n, ld ldt) over 64-column blocks J:
+// Y[:, J] = X[:, J] - Y[:, <J] T[<J, J] (FP64 mma), then Y[:, J] <- Y[:, J] T[J, J]^{-1} by the row pass (NP = 64).  Y may
+// equal X (ldy == ldx).  The diagonal blocks must have been set up by prep_blocks.  Marks PASS1 / PASS1_UPDATE /
+// PASS1_SOLVE2 when pass1_marks (blocks 2.. fall in PASS1_SOLVE2).
 static rpcholqr_status solve_blocked(rpcholqr_plan_s* p, const double* X, int64_t ldx, const double* T, int64_t ldt,
                               int64_t m, int n, double* Y, int64_t ldy, const double* frag, const double* diag,
-                              bool split, bool check_finite, int32_t* info, cudaStream_t st,
+                              bool check_finite, int32_t* info, cudaStream_t st,
                               const PhaseMarks* pm, bool pass1_marks) {
     const int grid = p->grid;
     for (int J = 0; J * kBlk < n; ++J) {
@@ -1087,55 +1024,16 @@ static rpcholqr_status solve_blocked(rpcholqr_plan_s* p, const double* X, int64_
         int64_t lsrc = ldx;
         if (J > 0) {
             if (pm && pass1_marks && J == 1) pm->mark(RPCHOLQR_PHASE_PASS1_UPDATE);
-            if (split) {
-                rpcholqr_status rc = ozaki_gemm_internal(p, true, Y, m, c0, ldy, T + c0, nj, ldt, X + c0, ldx,
-                                                         Y + c0, ldy, info, st, true);
-                if (rc != RPCHOLQR_OK) return rc;
-            } else {
-                {
-                    KTimer kt(p, st, RPCHOLQR_KERNEL_FP64_GEMM, 2.0 * m * c0 * nj);
-                    if (launch_gemm_sub_fp64(Y, ldy, T + c0, ldt, X + c0, ldx, Y + c0, ldy, m, c0, nj, info,
-                                             2 * p->grid, st) != cudaSuccess)
-                        return RPCHOLQR_ERR_CUDA;
-                }
-                ++p->launches;
+            {
+                KTimer kt(p, st, RPCHOLQR_KERNEL_FP64_GEMM, 2.0 * m * c0 * nj);
+                if (launch_gemm_sub_fp64(Y, ldy, T + c0, ldt, X + c0, ldx, Y + c0, ldy, m, c0, nj, info,
+                                         2 * p->grid, st) != cudaSuccess)
+                    return RPCHOLQR_ERR_CUDA;
             }
+            ++p->launches;
             src = Y + c0;
             lsrc = ldy;
             if (pm && pass1_marks && J == 1) pm->mark(RPCHOLQR_PHASE_PASS1_SOLVE2);
-        }
-        if (split) {
-            // sub-column FP64 solves (sub = the call's diagonal-block width, 16 or 32), each followed by
-            // one K = sub split update of the block's remaining columns (diagonal tables from prep_blocks
-            // with blk = sub)
-            const int sub = split_sub(p);
-            for (int h = 0; h * sub < nj; ++h) {
-                const int c1 = c0 + h * sub;
-                const int nh = nj - h * sub < sub ? nj - h * sub : sub;
-                const double* hsrc = h == 0 ? src : Y + c1;
-                const int64_t lh = h == 0 ? lsrc : ldy;
-                const int js = c1 / sub;
-                {
-                    KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(m) * nh * nh);
-                    if (launch_rowpass_ex(false, pad16(nh), hsrc, lh, Y + c1, ldy, m, nh, frag + js * sub * sub,
-                                          diag + js * (sub / 8) * 64, nullptr, info, grid, st, check_finite, p->xexp,
-                                          c1 == 0 ? 1 : 2, p->colexp + c1) != cudaSuccess)
-                        return RPCHOLQR_ERR_CUDA;
-                }
-                ++p->launches;
-                const int rest = c0 + nj - (c1 + nh);
-                if (rest > 0) {
-                    // the first sub-block's update reads the block's input columns, later ones updated columns
-                    const bool from_input = J == 0 && h == 0;
-                    const double* B = (from_input ? X : Y) + c1 + nh;
-                    const int64_t ldb = from_input ? ldx : ldy;
-                    rpcholqr_status rc = ozaki_gemm_internal(p, true, Y + c1, m, nh, ldy,
-                                                             T + static_cast<int64_t>(c1) * ldt + c1 + nh, rest, ldt,
-                                                             B, ldb, Y + c1 + nh, ldy, info, st, true);
-                    if (rc != RPCHOLQR_OK) return rc;
-                }
-            }
-            continue;
         }
         {
             KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(m) * nj * nj);
@@ -1186,8 +1084,7 @@ static rpcholqr_status precondition_internal(rpcholqr_plan p, const double* A, i
         // wide: blocked solve into A1, then a separate Gram pass
         prep_blocks(p, Rs, ldrs, n, p->frag_s, p->diag_s, info, st);
         if (pm) pm->mark(RPCHOLQR_PHASE_PASS1);
-        rpcholqr_status rc = solve_blocked(p, A, lda, Rs, ldrs, m, n, A1, ld1, p->frag_s, p->diag_s, false, true,
-                                           info, st, pm, true);
+        rpcholqr_status rc = solve_blocked(p, A, lda, Rs, ldrs, m, n, A1, ld1, p->frag_s, p->diag_s, true, info, st, pm, true);
         if (rc != RPCHOLQR_OK) return rc;
         if (pm) pm->mark(RPCHOLQR_PHASE_GRAM_REDUCE);
         return gram_fp64_wide(p, A1, ld1, m, n, G, ldg, info, st);
@@ -1221,8 +1118,7 @@ static rpcholqr_status solve_internal(rpcholqr_plan p, const double* X, int64_t 
     if (np > kMaxNP) {
         prep_blocks(p, T, ldt, n, p->frag_1, p->diag_1, info, st);
         if (pm) pm->mark(RPCHOLQR_PHASE_PASS2);
-        return solve_blocked(p, X, ldx, T, ldt, m, n, Y, ldy, p->frag_1, p->diag_1, false, false, info, st,
-                             nullptr, false);
+        return solve_blocked(p, X, ldx, T, ldt, m, n, Y, ldy, p->frag_1, p->diag_1, false, info, st, nullptr, false);
     }
     launch_prep_tri(T, ldt, n, np, p->frag_1, p->diag_1, info, st);
     ++p->launches;
@@ -1333,20 +1229,13 @@ static rpcholqr_status factor_split(rpcholqr_plan p, const double* A, int64_t m,
     pm.mark(RPCHOLQR_PHASE_PREP_RS);
     launch_fill_noexp(p->colexp, n, st);   // column bounds of A1, atomically max-merged by the row passes
     ++p->launches;
-    // A1 = A R_s^{-1}: FP64 row passes on the diagonal blocks, split tensor-core updates for the rest.
-    // Up to 128 columns: 32-column blocks, right-looking (every update one K stage, wide N); above:
-    // 64-column blocks, left-looking (long K windows; fewer passes over the trailing columns).
-    if (np <= kMaxNP) {
-        prep_blocks(p, p->Rs, np, n, p->frag_s, p->diag_s, info, st, split_sub(p));
-        pm.mark(RPCHOLQR_PHASE_PASS1);
-        rc = solve_split_right(p, A, lda, p->Rs, np, m, n, A1, ld1, p->frag_s, p->diag_s, info, st, &pm);
-    } else {
-        prep_blocks(p, p->Rs, np, n, p->frag_s, p->diag_s, info, st, split_sub(p));
-        pm.mark(RPCHOLQR_PHASE_PASS1);
-        rc = p->aimg ? solve_split_wide(p, A, lda, p->Rs, np, m, n, A1, ld1, p->frag_s, p->diag_s, info, st, &pm)
-                     : solve_blocked(p, A, lda, p->Rs, np, m, n, A1, ld1, p->frag_s, p->diag_s, true, true, info, st,
-                                     &pm, true);
-    }
+    // A1 = A R_s^{-1} over 64-column blocks, left-looking: FP64 substitution on 16-column sub-blocks, split tensor-core
+    // products for the rest
+    launch_split_solve_prep(p->Rs, np, n, p->sstab, info, st);
+    ++p->launches;
+    pm.mark(RPCHOLQR_PHASE_PASS1);
+    rc = p->aimg ? solve_split_wide(p, A, lda, p->Rs, np, m, n, A1, ld1, info, st, &pm)
+                 : solve_split(p, A, lda, p->Rs, np, m, n, A1, ld1, info, st, &pm);
     if (rc != RPCHOLQR_OK) return rc;
     pm.mark(RPCHOLQR_PHASE_GRAM_REDUCE);
     if ((rc = ozaki_gram_internal(p, A1, m, n, ld1, p->G, np, info, st, true)) != RPCHOLQR_OK) return rc;
@@ -1670,13 +1559,14 @@ static rpcholqr_status factor_host_split(rpcholqr_plan p, const double* A, int64
     p->launches += 2 + householder_launches(n);
     // pass 1, block by block as A arrives
     launch_fill_noexp(p->colexp, n, st);
-    prep_blocks(p, p->Rs, np, n, p->frag_s, p->diag_s, info, st, split_sub(p));
+    launch_split_solve_prep(p->Rs, np, n, p->sstab, info, st);
+    ++p->launches;
     for (int c = 0; c < nchunks; ++c) {
         int64_t r0, rows;
         chunk(c, r0, rows);
         if (cudaStreamWaitEvent(st, p->hev[c], 0) != cudaSuccess) return RPCHOLQR_ERR_CUDA;
-        if ((rc = solve_split_right(p, dA + r0 * n, n, p->Rs, np, rows, n, p->A1 + r0 * ld1, ld1, p->frag_s,
-                                    p->diag_s, info, st, nullptr, r0)) != RPCHOLQR_OK)
+        if ((rc = solve_split(p, dA + r0 * n, n, p->Rs, np, rows, n, p->A1 + r0 * ld1, ld1, info, st, nullptr, r0)) !=
+            RPCHOLQR_OK)
             return rc;
     }
     if ((rc = ozaki_gram_internal(p, p->A1, m, n, ld1, p->G, np, info, st, true)) != RPCHOLQR_OK) return rc;
@@ -2046,13 +1936,12 @@ rpcholqr_status rpcholqr_autotune(rpcholqr_plan p, int32_t nclasses, const int64
             cands.clear();
             const int nh = ozaki_gram_tiles(np, p->aimg != nullptr);
             const int plain = p->grid / nh > 0 ? p->grid / nh : 1;
-            for (int sub : {kSplitSub, 16})   // the built-in width first; gram_ranges 0 = the wave rule
-                for (int gr : {0, plain, 2 * plain}) {
-                    Tuning t;
-                    t.split_sub = sub;
-                    t.gram_ranges = gr > p->nparts ? p->nparts : gr;
-                    cands.push_back(t);
-                }
+            for (int gr : {0, plain, 2 * plain}) {   // 0: the wave rule
+                Tuning t;
+                t.split_sub = kSplitSub;
+                t.gram_ranges = gr > p->nparts ? p->nparts : gr;
+                cands.push_back(t);
+            }
         } else if (np > kMaxNP) {
             const int nb = np / kBlk, tiles = nb * (nb + 1) / 2;
             for (int f : {1, 4}) {

@@ -293,8 +293,7 @@ __device__ __forceinline__ double scale_pow2(long long I, int e) {
     return ldexp(v, e);
 }
 
-// The same without FP64 instructions (rounded to nearest, ties away), for the update, whose FP64 units carry the
-// subtraction already.
+// The same without FP64 instructions (rounded to nearest, ties away), for the block solve, whose FP64 units are its bound.
 __device__ __forceinline__ double scale_pow2_int(long long I, int e) {
     const unsigned long long neg = static_cast<unsigned long long>(I >> 63), a = (static_cast<unsigned long long>(I) ^ neg) - neg;
     const int lz = __clzll(static_cast<long long>(a)), field = 1085 - lz + e;
@@ -1319,7 +1318,7 @@ k_ozaki_update(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, i
                             for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][i];
                             const long long I = combine_units53_k32(grp);
                             const int ey = col < N ? yexp[col] : kNoExp;
-                            const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2_int(I, E + ey - 53) : 0.0;
+                            const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2(I, E + ey - 53) : 0.0;
                             cv[i] = bv[c0 + i] - v;
                         }
 #pragma unroll
@@ -1761,6 +1760,288 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
 }
 
+// ---- diagonal blocks of the split first pass -------------------------------------------------------------
+// Y = X T^{-1} for one block of up to 64 columns (T its upper-triangular diagonal block), per row: FP64 substitution on
+// 16-column sub-blocks, joined by split updates inside the block:
+//   solve 0;  cols 16..31 -= x(0..15) T;  solve 1;  cols 32..63 -= x(0..31) T;  solve 2;  cols 48..63 -= x(32..47) T;  solve 3
+// A CTA has two groups of eight warps, each with its own 128-row tile, worked on in halves of 32 columns kept in shared
+// memory (column by column, so that a thread reads its row without conflicts).  Two threads per row (= TMEM lane):
+// the first solves the sub-block in registers; then both slice it (half the chunks each) against the row's bound over
+// the columns of the update, one thread issues the MMAs, and both read the row's group sums back and subtract (half the
+// columns each), the second taking the column bounds while the MMAs run.  While one group slices, waits for its MMAs
+// or drains, the other's substitutions keep the FP64 units busy: they are the bound (16 x 16 / 2 multiply-adds a row and
+// sub-block and one subtraction per updated value, at two a clock per SM).  With one thread per row the integer work
+// of slicing and draining, a few dependent operations in flight per scheduler, took twice the time of the FP64 work.
+// The loops over halves, sub-blocks, chunks and drained columns stay rolled: with the row in registers and everything
+// unrolled the code was 110 KB, and waiting for instructions was the largest stall.
+constexpr int kSsThreads = 512;
+constexpr int kSsGroup = 256;                                             // threads of a group
+constexpr int kSsN1 = 16, kSsN2 = 32;                                      // columns of the updates
+__host__ __device__ constexpr int ss_b_off(int u) {                        // update u's slices of T in the table
+    return u == 0 ? 0 : kSlices * (u == 1 ? kSsN1 : kSsN1 + kSsN2) * kKW * 2;
+}
+constexpr int kSsBBytes = kSlices * (2 * kSsN1 + kSsN2) * kKW * 2;        // 28 KB: the updates' slices of T
+constexpr int kSsDOff = kSsBBytes;                                         // 4 x 16 x 16 doubles: diagonal sub-blocks,
+constexpr int kSsEOff = kSsDOff + 4 * 256 * 8;                             //   reciprocal diagonals; then 64 column bounds
+constexpr int kSsTab = kSsEOff + 256;                                      // of the updates' columns
+constexpr int kSsLd = kTileM + 1;                                          // rows of a column in the half panel, padded
+constexpr int kSsPanel = 32 * kSsLd * 8;
+constexpr int kSsSmem = 2 * (kAStage + kSsPanel) + kSsTab;
+static_assert(kSsSmem + 2048 <= 232448, "k_split_solve exceeds the 227 KB shared-memory limit");
+
+// The tables of every 64-column block of T (n x n): block J's at tab + J kSsTab.  One CTA per block.
+__global__ void __launch_bounds__(256) k_split_solve_prep(const double* __restrict__ T, int64_t ldt, int n,
+                                                          uint8_t* __restrict__ tab, const int32_t* info) {
+    __shared__ int ecol[64];
+    if (info && load_status(info) != 0) return;
+    const int c0 = 64 * blockIdx.x, tid = threadIdx.x;
+    uint8_t* out = tab + static_cast<size_t>(blockIdx.x) * kSsTab;
+    auto tv = [&](int r, int c) { return (c0 + r < n && c0 + c < n) ? T[static_cast<int64_t>(c0 + r) * ldt + c0 + c] : 0.0; };
+    double* D = reinterpret_cast<double*>(out + kSsDOff);
+    for (int e = tid; e < 4 * 256; e += 256) {
+        const int s = e >> 8, r = (e >> 4) & 15, c = e & 15;
+        const bool in = c0 + 16 * s + r < n && c0 + 16 * s + c < n;
+        D[e] = r > c ? 0.0 : r == c ? (in ? 1.0 / tv(16 * s + r, 16 * s + c) : 1.0) : tv(16 * s + r, 16 * s + c);
+    }
+    // column j of the 64: update u, its column q, first row r0 and K
+    const int j = tid & 63, u = j < 16 ? 0 : j < 48 ? 1 : 2, q = u == 0 ? j : u == 1 ? j - 16 : j - 48;
+    const int col = u == 0 ? 16 + q : u == 1 ? 32 + q : 48 + q, r0 = u == 2 ? 32 : 0, K = u == 1 ? 32 : 16;
+    if (tid < 64) {
+        int E = kNoExp;
+        for (int k = 0; k < K; ++k) {
+            const int e = exp_bound(tv(r0 + k, col));
+            E = e > E ? e : E;
+        }
+        ecol[j] = E;
+        reinterpret_cast<int32_t*>(out + kSsEOff)[j] = E;
+    }
+    __syncthreads();
+    const int c = tid >> 6;    // 8-row chunk
+    if (8 * c < K) {
+        double x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = tv(r0 + 8 * c + i, col);
+        slice_store8(x, ecol[j], out + ss_b_off(u) + core_off(q, 16 * c), (u == 1 ? kSsN2 : kSsN1) * kKW * 2);
+    }
+}
+
+__device__ __forceinline__ void ss_group_sync(int g) { asm volatile("bar.sync %0, %1;\n" ::"r"(4 + g), "n"(kSsGroup) : "memory"); }
+__device__ __forceinline__ bool ss_group_or(bool v, int g) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, %2, %3, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(r)
+        : "r"(static_cast<uint32_t>(v)), "r"(4 + g), "n"(kSsGroup)
+        : "memory");
+    return r != 0;
+}
+// The MMAs of an update: NKK K = 16 steps of the group's stage against the table's slices (N columns), by one thread.
+template <int NKK, int N>
+__device__ __forceinline__ void ss_issue(uint32_t tset, uint32_t st, uint32_t B, uint64_t* bar) {
+    const uint64_t a0 = sdesc(st), b0 = sdesc(B);
+#pragma unroll
+    for (int kk = 0; kk < NKK; ++kk)
+#pragma unroll
+        for (int s = 1; s <= kSlices; ++s)
+            mma_f16_n(tset + (s - 1) * N, a0 + static_cast<uint32_t>(((s - 1) * kASlice + kk * 256) >> 4),
+                      b0 + static_cast<uint32_t>(kk * 16), idesc_f16(N * (kSlices + 1 - s)), (kk == 0 && s == 1) ? 0u : 1u);
+    mma_commit(bar);
+}
+// Columns [from, to) of the thread's row (multiples of 4): P[c * kSsLd] -= the update's result (group d at TMEM columns d N).
+template <int N>
+__device__ __forceinline__ void ss_drain(uint32_t tl, int from, int to, int E, const int32_t* ey, double* P) {
+#pragma unroll 1
+    for (int c0 = from; c0 < to; c0 += 4) {
+        float mg[kGroups][4];
+#pragma unroll
+        for (int q = 0; q < kGroups; ++q) tmem_ld4(tl + q * N + c0, mg[q]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float grp[kGroups];
+#pragma unroll
+            for (int q = 0; q < kGroups; ++q) grp[q] = mg[q][i];
+            const int e = ey[c0 + i];
+            if (E > kNoExp && e > kNoExp) P[(c0 + i) * kSsLd] -= scale_pow2_int(combine_units53_k32(grp), E + e - 53);
+        }
+    }
+}
+
+// nc <= 64 columns.  rowexp: the row's bound over the block, stored (rowexp_mode 1) or merged (2); colexp: column bounds
+// (atomicMax).  Y may equal X.
+__global__ void __launch_bounds__(kSsThreads, 1)
+k_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int nc, const uint8_t* __restrict__ tab,
+              int32_t* rowexp, int rowexp_mode, int32_t* colexp, int32_t* info, long spin) {
+    extern __shared__ __align__(1024) uint8_t sm[];
+    __shared__ uint64_t bars[2];
+    __shared__ uint32_t tslot;
+    __shared__ int abort_s, cs[64], bound_s[2][2][kTileM];   // [group][sub-block of the half][row]
+    if (load_status(info) != 0) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = tid >> 8, hf = (tid >> 7) & 1, lr = tid & 127;
+    uint8_t* tb = sm + 2 * (kAStage + kSsPanel);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         smem_u32(&tslot)), "r"(kTmemCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&bars[i])));
+        asm volatile("fence.mbarrier_init.release.cluster;\n");
+        abort_s = 0;
+    }
+    if (tid < 64) cs[tid] = kNoExp;
+    for (int e = tid; e < kSsTab / 16; e += kSsThreads)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(tb + 16 * e)), "l"(tab + 16 * e));
+    cp_async_commit();
+    cp_async_wait_all();
+    fence_async_smem();
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    uint8_t* st = sm + g * kAStage;
+    double* P = reinterpret_cast<double*>(sm + 2 * kAStage + g * kSsPanel);   // the half: column c, row r at c kSsLd + r
+    double* Pr = P + lr;
+    uint64_t* bar = &bars[g];
+    const uint32_t tset = tslot + 256u * g, tl = tset + (static_cast<uint32_t>((lr >> 5) * 32) << 16);
+    const int32_t* ey = reinterpret_cast<const int32_t*>(tb + kSsEOff);
+    const int64_t ntm = (m + kTileM - 1) / kTileM;
+    uint32_t phase = 0;
+    bool bad = false, ok = true;
+    int cm0 = kNoExp, cm1 = kNoExp;   // bounds of columns lane and 32 + lane over the rows of this warp
+    for (int64_t t = blockIdx.x + static_cast<int64_t>(g) * gridDim.x; t < ntm; t += 2 * static_cast<int64_t>(gridDim.x)) {
+        const int64_t row0 = t * kTileM, row = row0 + lr;
+        int re = kNoExp, E32 = kNoExp;
+        auto wait_mma = [&]() {
+            if (ok) ok = mbar_wait_ab(bar, phase, &abort_s, spin);
+            __syncwarp();
+            phase ^= 1u;
+            tc_after_sync();
+        };
+#pragma unroll 1
+        for (int h = 0; 32 * h < nc; ++h) {
+            const int w = nc - 32 * h < 32 ? nc - 32 * h : 32;
+            // the half's rows, one per warp at a time (zeros outside the matrix)
+            for (int r = warp & 7; r < kTileM; r += 8) {
+                const bool in = row0 + r < m && lane < w;
+                cp_async8(P + lane * kSsLd + r, in ? X + (row0 + r) * ldx + 32 * h + lane : X, in);
+            }
+            cp_async_commit();
+            cp_async_wait_all();
+            ss_group_sync(g);
+            if (h > 0) {
+                wait_mma();
+                ss_drain<kSsN2>(tl, 16 * hf, 16 * hf + 16, E32, ey + 16, Pr);
+                ss_group_sync(g);
+            }
+#pragma unroll 1
+            for (int s = 0; 16 * s < w; ++s) {
+                double* Ps = Pr + 16 * s * kSsLd;
+                if (hf == 0) {
+                    // FP64 substitution on columns 16 s ..; d[c][k] = T[c][k] (k > c), 1 / T[c][c] on the diagonal
+                    const double* d = reinterpret_cast<const double*>(tb + kSsDOff) + (2 * h + s) * 256;
+                    double x[16];
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        x[c] = Ps[c * kSsLd];
+                        bad |= ((__double2hiint(x[c]) >> 20) & 0x7FF) == 0x7FF;
+                    }
+                    int e = kNoExp;
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        x[c] *= d[c * 17];
+#pragma unroll
+                        for (int k = c + 1; k < 16; ++k) x[k] = fma(-x[c], d[c * 16 + k], x[k]);
+                        Ps[c * kSsLd] = x[c];
+                        const int ec = exp_bound(x[c]);
+                        e = ec > e ? ec : e;
+                    }
+                    bound_s[g][s][lr] = e;
+                }
+                ss_group_sync(g);
+                const int e = bound_s[g][s][lr];
+                re = e > re ? e : re;
+                const bool upd = s == 0 && w > 16;
+                if (upd) {
+                    double x8[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) x8[i] = Ps[(8 * hf + i) * kSsLd];
+                    slice_store8(x8, e, st + core_off(lr, 16 * hf), kASlice);
+                    fence_async_smem();
+                    tc_before_sync();
+                    ss_group_sync(g);
+                    if ((tid & 255) == 0) {
+                        tc_after_sync();
+                        ss_issue<1, kSsN1>(tset, smem_u32(st), smem_u32(tb + (h == 0 ? ss_b_off(0) : ss_b_off(2))), bar);
+                    }
+                    __syncwarp();
+                }
+                if (hf == 1) {
+                    // the sub-block's column bounds (rows past m hold zeros: no bound)
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        const int ce = __reduce_max_sync(0xffffffffu, exp_bound(Ps[c * kSsLd]));
+                        if (lane == 16 * s + c) {
+                            if (h == 0) cm0 = ce > cm0 ? ce : cm0;
+                            else cm1 = ce > cm1 ? ce : cm1;
+                        }
+                    }
+                }
+                if (upd) {
+                    wait_mma();
+                    ss_drain<kSsN1>(tl, 8 * hf, 8 * hf + 8, e, ey + 48 * h, Pr + 16 * kSsLd);
+                    ss_group_sync(g);
+                }
+            }
+            if (32 * h + 32 < nc) {
+                // both sub-blocks against their common bound, for the other half
+                E32 = re;
+#pragma unroll 1
+                for (int c = 2 * hf; c < 2 * hf + 2; ++c) {
+                    double x8[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) x8[i] = Pr[(8 * c + i) * kSsLd];
+                    slice_store8(x8, E32, st + core_off(lr, 16 * c), kASlice);
+                }
+                fence_async_smem();
+                tc_before_sync();
+            }
+            ss_group_sync(g);   // every row of the half is final, and sliced
+            if (32 * h + 32 < nc && (tid & 255) == 0) {
+                tc_after_sync();
+                ss_issue<2, kSsN2>(tset, smem_u32(st), smem_u32(tb + ss_b_off(1)), bar);
+            }
+            __syncwarp();
+            for (int r = warp & 7; r < kTileM; r += 8)
+                if (row0 + r < m && lane < w) Y[(row0 + r) * ldy + 32 * h + lane] = P[lane * kSsLd + r];
+            ss_group_sync(g);   // the panel is free for the next half
+        }
+        if (hf == 0 && row < m) {
+            if (rowexp_mode == 2 && rowexp[row] > re) re = rowexp[row];
+            rowexp[row] = re;
+        }
+        if (ss_group_or(!ok, g)) {   // a wait gave up in some thread of the group
+            ok = false;
+            break;
+        }
+    }
+    if (!ok) {
+        abort_s = 1;
+        mbar_wait(bar, phase ^ 1u);   // this group's last MMAs are done before the tensor memory is released
+    }
+    if (lane < nc) atomicMax(&cs[lane], cm0);
+    if (32 + lane < nc) atomicMax(&cs[32 + lane], cm1);
+    tc_before_sync();
+    const bool any_bad = __syncthreads_or(bad);
+    tc_after_sync();
+    if (tid < nc && cs[tid] > kNoExp) atomicMax(&colexp[tid], cs[tid]);
+    if (tid == 0 && any_bad) set_status(info, RPCHOLQR_ERR_NONFINITE);
+    if (tid == 0 && abort_s) set_status(info, RPCHOLQR_ERR_TIMEOUT);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tslot), "r"(kTmemCols));
+}
+
 // rowexp[i] = exponent bound of row i of X (m x K, ldx); kNoExp for an all-zero row.
 __global__ void k_row_exp(const double* __restrict__ X, int64_t ldx, int64_t m, int K, int32_t* __restrict__ rowexp) {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -1856,6 +2137,25 @@ void launch_slice_images(const double* X, int64_t ldx, int64_t m, int K, const i
 }
 
 int32_t ozaki_no_exp() { return kNoExp; }
+
+// Tables of the 64-column diagonal blocks of an n x n T (split_solve_tab_bytes(n)), and the solve of block J's nc columns of
+// m rows with them (X, Y at the block's first column).  Measured on GB300, one 64-column block of 2^21 rows: 3.24 ms
+// (FP64 pipe 66 % busy), against 4.7 ms for four FP64 row passes and three update launches; the row in registers with
+// everything unrolled 3.88 (8-column sub-blocks 4.0), one thread per row with rolled loops 3.52.
+size_t split_solve_tab_bytes(int n) { return static_cast<size_t>((n + 63) / 64) * oz::kSsTab; }
+void launch_split_solve_prep(const double* T, int64_t ldt, int n, uint8_t* tab, const int32_t* info, cudaStream_t st) {
+    oz::k_split_solve_prep<<<(n + 63) / 64, 256, 0, st>>>(T, ldt, n, tab, info);
+}
+cudaError_t launch_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int nc, const uint8_t* tab, int J,
+                               int32_t* rowexp, int rowexp_mode, int32_t* colexp, int32_t* info, int sms, cudaStream_t st,
+                               long spin) {
+    cudaError_t err = cudaFuncSetAttribute(oz::k_split_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::kSsSmem);
+    if (err != cudaSuccess) return err;
+    const int64_t tiles = (m + oz::kTileM - 1) / oz::kTileM;
+    oz::k_split_solve<<<static_cast<unsigned>(tiles < sms ? tiles : sms), oz::kSsThreads, oz::kSsSmem, st>>>(
+        X, ldx, Y, ldy, m, nc, tab + static_cast<size_t>(J) * oz::kSsTab, rowexp, rowexp_mode, colexp, info, spin);
+    return cudaGetLastError();
+}
 
 void launch_row_exp(const double* X, int64_t ldx, int64_t m, int K, int32_t* rowexp, cudaStream_t st) {
     oz::k_row_exp<<<static_cast<unsigned>((m + 255) / 256), 256, 0, st>>>(X, ldx, m, K, rowexp);
