@@ -73,7 +73,7 @@ def parse_args(argv=None):
                     help="draw A with torch on the GPU (fast) or with the numpy recipe on the host")
     ap.add_argument("--no-metrics", action="store_true", help="skip the orthogonality/residual check")
     ap.add_argument("--mode", choices=["fp64", "split", "fp32"], default="split",
-                    help="split (default): FP64-accurate Ozaki-split BF16 tensor-core products for the "
+                    help="split (default): FP64-accurate Ozaki-split FP16 tensor-core products for the "
                          "well-conditioned steps; fp64: every step in FP64; fp32: float data, FP32 "
                          "passes (FP64 sketch QR and Cholesky)")
     ap.add_argument("--workload", choices=["single", "batch"], default="single",
@@ -434,7 +434,7 @@ def kernels_per_step(ph, calls):
 SLICE_PRODUCTS = 28
 SPLIT_CLASSES = ("split_update", "split_gemm_sub", "split_gemm", "split_gram")
 KERNEL_NAMES = {
-    "rowpass": "k_rowpass (FP64 row solves: mma.sync m16n8k16 + DFMA)",
+    "rowpass": "k_rowpass (FP64 row solves: mma.sync m16n8k16 + DFMA); split mode: oz::k_split_solve (diagonal blocks)",
     "split_update": "oz::k_ozaki_update (split C = B - X Y, K <= 32)",
     "split_gemm_sub": "oz::k_ozaki_gemm_db<SUB> (n > 128; k_ozaki_gemm_ws<.,SUB> up to 128) (split C = B - X Y, "
                       "wide pass-1 block updates)",
@@ -442,14 +442,14 @@ KERNEL_NAMES = {
     "split_gram": "oz::k_ozaki_gram (split G1 = A1^T A1)",
     "fp64_gemm": "k_gemm_sub_fp64 (FP64 block updates)",
     "fp64_syrk": "k_syrk_fp64 (FP64 Gram)",
-    "sketch_qr": "k_hh_cluster (Householder QR of the sample)",
-    "cholesky": "k_cholesky (G1 = R1^T R1)",
+    "sketch_qr": "k_qr_panel, k_qr_y, k_qr_z, k_qr_update (Householder QR of the sample)",
+    "cholesky": "k_chol_panel, k_chol_trail (G1 = R1^T R1, with R1^-1)",
 }
 
 
 CLASS_SOURCE = {"rowpass": "rowpass.cuh", "split_update": "ozaki.cu", "split_gemm_sub": "ozaki.cu",
                 "split_gemm": "ozaki.cu", "split_gram": "ozaki.cu", "fp64_gemm": "blocked.cu",
-                "fp64_syrk": "blocked.cu", "sketch_qr": "smallfactor.cuh", "cholesky": "smallfactor.cuh"}
+                "fp64_syrk": "blocked.cu", "sketch_qr": "sketchqr.cuh", "cholesky": "smallfactor.cuh"}
 
 
 def class_bytes(cls, mode, m, n):

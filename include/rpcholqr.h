@@ -445,7 +445,7 @@ enum {
 
 /* Kernel classes of rpcholqr_plan_collect_kernel_timing. */
 enum {
-    RPCHOLQR_KERNEL_ROWPASS = 0,     /* FP64 row passes: fused pass 1, pass 2, diagonal-block solves       */
+    RPCHOLQR_KERNEL_ROWPASS = 0,     /* FP64 row passes: fused pass 1, pass 2; SPLIT64 diagonal-block solves */
     RPCHOLQR_KERNEL_SPLIT_UPDATE,    /* split C = B - X Y with K <= 32 (k_ozaki_update)                    */
     RPCHOLQR_KERNEL_SPLIT_GEMM_SUB,  /* split C = B - X Y, K > 32 (wide pass-1 block updates)              */
     RPCHOLQR_KERNEL_SPLIT_GEMM,      /* split C = X Y (pass 2, Q = A1 R1^{-1})                              */

@@ -502,7 +502,7 @@ def rpcholqr_scholqr3(plan: Plan, A, Q=None, R=None, info=None, stream=None):
 
 
 def rpcholqr_ozaki_gemm(plan: Plan, X, Y, C=None, info=None, stream=None):
-    """C = X Y as a split-precision (FP64-accurate) BF16 tensor-core product (SPLIT64 plan)."""
+    """C = X Y as a split-precision (FP64-accurate) FP16 tensor-core product (SPLIT64 plan)."""
     torch = _torch()
     _mat(X, "X")
     _mat(Y, "Y")
@@ -540,7 +540,7 @@ def rpcholqr_ozaki_update(plan: Plan, X, Y, B, C=None, info=None, stream=None):
 
 
 def rpcholqr_ozaki_gram(plan: Plan, X, G=None, info=None, stream=None):
-    """G = X^T X as a split-precision BF16 tensor-core product (SPLIT64 plan)."""
+    """G = X^T X as a split-precision FP16 tensor-core product (SPLIT64 plan)."""
     torch = _torch()
     _mat(X, "X")
     m, n = X.shape

@@ -6,9 +6,9 @@
 //                                                columns k_ozaki_gemm_db; kappa(R_1) = kappa(A_1) is
 //                                                small, Lemma l_31)
 //   precondition  the off-diagonal block update A[:,J] - A_1[:,<J] R_s[<J,J] of the blocked row solve
-//                                               (k_ozaki_update for K <= 32, else k_ozaki_gemm_ws /
-//                                                k_ozaki_gemm_db, subtract form; the diagonal blocks stay
-//                                                FP64 substitution)
+//                                               (k_ozaki_gemm_ws / k_ozaki_gemm_db, subtract form; k_ozaki_update
+//                                                serves the update entry point up to K = 32), and the diagonal
+//                                                blocks (k_split_solve: FP64 substitution joined by split updates)
 // Above 128 columns the left operand is sliced beforehand into stage images (k_slice_images,
 // k_slice_block_images, k_slice_col_images) that the *_db kernels stream in by TMA bulk copies.
 //
