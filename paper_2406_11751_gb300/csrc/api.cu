@@ -174,7 +174,7 @@ struct rpcholqr_plan_s {
     double* diag_s = nullptr;   // np/8*64
     double* frag_1 = nullptr;
     double* diag_1 = nullptr;
-    double* gpart = nullptr;    // grid x np x np
+    double* gpart = nullptr;    // Gram partials (gpart_doubles)
     double* qws = nullptr;      // the sketch QR's workspace (householder_ws_bytes)
     int32_t* info_ws = nullptr; // 2 ints (for step calls without a caller info)
     // staging for rpcholqr_factor_host
@@ -268,7 +268,15 @@ int gram_parts(rpcholqr_mode mode, int64_t max_m, int32_t max_n, int grid) {
     return parts < 1 ? 1 : static_cast<int>(parts);
 }
 
-WsLayout ws_layout(int32_t max_n, int32_t max_s, int grid) {
+// Doubles of those partials.  A plan above 128 columns also takes narrower calls, whose fused pass writes
+// rowpass_parts partials of its own width: at most rowpass_max_parts of 128 x 128 (19.9 MB at 152 SMs).
+size_t gpart_doubles(int64_t max_m, int32_t max_n, int parts, int grid) {
+    const size_t np = static_cast<size_t>(pad_np(max_n)), own = static_cast<size_t>(parts) * np * np;
+    const size_t narrow = static_cast<size_t>(rowpass_max_parts(max_m, grid)) * kMaxNP * kMaxNP;
+    return np > static_cast<size_t>(kMaxNP) && narrow > own ? narrow : own;
+}
+
+WsLayout ws_layout(int64_t max_m, int32_t max_n, int32_t max_s, int parts, int grid) {
     const size_t np = static_cast<size_t>(pad_np(max_n));
     WsLayout L{};
     size_t off = 0;
@@ -281,7 +289,7 @@ WsLayout ws_layout(int32_t max_n, int32_t max_s, int grid) {
     L.diag_s = take(sizeof(double) * (np / 8) * 64);
     L.frag_1 = take(sizeof(double) * np * np);
     L.diag_1 = take(sizeof(double) * (np / 8) * 64);
-    L.gpart = take(sizeof(double) * static_cast<size_t>(grid) * np * np);
+    L.gpart = take(sizeof(double) * gpart_doubles(max_m, max_n, parts, grid));
     L.qws = take(householder_ws_bytes(static_cast<int>(np)));
     L.info = take(sizeof(int32_t) * 2);
     L.total = off;
@@ -628,7 +636,7 @@ rpcholqr_status rpcholqr_workspace_size(rpcholqr_plan p, int64_t max_m, int32_t 
     const rpcholqr_mode mode = p ? p->mode : RPCHOLQR_FP64;
     const int grid = p ? p->grid : 152;
     const int32_t ws_n = mode == RPCHOLQR_FP32 ? (max_n + 63) / 64 * 64 : max_n;
-    size_t total = ws_layout(ws_n, max_s, gram_parts(mode, max_m, max_n, grid)).total;
+    size_t total = ws_layout(max_m, ws_n, max_s, gram_parts(mode, max_m, max_n, grid), grid).total;
     const size_t np = static_cast<size_t>(pad_np(max_n));
     if (mode == RPCHOLQR_SPLIT64)   // A1, row/column bounds, column slices, R1^{-1}, gate words, diagonal-block tables
         total += align256(sizeof(double) * static_cast<size_t>(max_m) * np) +
@@ -705,7 +713,7 @@ rpcholqr_status rpcholqr_plan_create(rpcholqr_plan* plan, int device, rpcholqr_m
     // the FP32 Gram works on 64 x 64 tiles: size the shared FP64 buffers for max_n rounded up to 64
     const int32_t ws_n = mode == RPCHOLQR_FP32 ? (max_n + 63) / 64 * 64 : max_n;
     p->nparts = gram_parts(mode, max_m, max_n, p->grid);
-    const WsLayout L = ws_layout(ws_n, max_s, p->nparts);
+    const WsLayout L = ws_layout(max_m, ws_n, max_s, p->nparts, p->grid);
     if (cudaMalloc(&p->ws, L.total) != cudaSuccess) {
         cudaGetLastError();
         delete p;

@@ -40,6 +40,11 @@ __host__ __device__ constexpr int rowpass_parts(int np, int64_t m, int sms) {
     const int64_t rows = rowpass_rows(np, m, sms), panels = (m + rows - 1) / rows;
     return static_cast<int>(panels < sms ? panels : sms);
 }
+// The most of those partials any width and any row count up to m leave: short panels have 64 rows or more.
+__host__ __device__ constexpr int rowpass_max_parts(int64_t m, int sms) {
+    const int64_t panels = (m + 16 * kRowpassMinWarps - 1) / (16 * kRowpassMinWarps);
+    return static_cast<int>(panels < sms ? panels : sms);
+}
 // The plain solve up to 48 columns runs two CTAs per SM (128 registers a thread, two panels fit the
 // shared memory): one CTA's panel load overlaps the other's FP64 work and each scheduler has four
 // warps' dependent chains to interleave.  The fused Gram keeps one CTA per SM (one partial each).
