@@ -62,6 +62,11 @@ __device__ __forceinline__ int exp_bound(double v) {
 __device__ __forceinline__ int load_status(const int32_t* info) {
     return *reinterpret_cast<const volatile int32_t*>(info);
 }
+// True for every thread of the CTA when a status is set: one answer for all of them.  A kernel that sets the status
+// itself decides whether to run by this, not by each thread's own read: a CTA that starts late may find another CTA's
+// status appear between the reads of its warps, and the warps that went on would wait for ever at a barrier with a fixed
+// count, or work on tensor memory that the warp that left was to allocate.
+__device__ __forceinline__ bool cta_stopped(const int32_t* info) { return __syncthreads_or(load_status(info) != 0) != 0; }
 // First error wins.
 __device__ __forceinline__ void set_status(int32_t* info, int status, int pivot = -1) {
     if (atomicCAS(info, 0, status) == 0 && pivot >= 0) info[1] = pivot;

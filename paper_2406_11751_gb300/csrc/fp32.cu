@@ -63,7 +63,7 @@ k_rowsolve_f32(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, in
                bool check_finite, bool vec_in, bool vec_out) {
     extern __shared__ float4 fsm4[];
     constexpr int RT = R / 32;            // rows of a thread: ty + 32 i
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     float* ts = reinterpret_cast<float*>(fsm4);            // two 32 x 32 tiles of T
     float* panel = ts + 2 * kF32Blk * kF32Blk;
     const int ld = np32 + 4;

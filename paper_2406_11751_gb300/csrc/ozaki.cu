@@ -641,7 +641,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
     __shared__ uint64_t empty_bar[2], full_bar[2], done_bar;
     __shared__ uint32_t tslot;
     __shared__ int abort_s;
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     constexpr int NT = WIN ? kThreadsWin : kThreads;
     constexpr int NC = Share<NT>::kDrainCols, NCH = Share<NT>::kChunks;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -928,7 +928,7 @@ k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xe
     __shared__ uint64_t load_bar[2], empty_bar[2], acc_full[2], acc_empty[2], done_bar;
     __shared__ uint32_t tslot;
     __shared__ int abort_s;
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint8_t* stA[2] = {sm, sm + kDbStage};
     uint8_t* stB[2] = {sm + kAStage, sm + kDbStage + kAStage};
@@ -1172,7 +1172,7 @@ k_ozaki_update(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, i
     __shared__ uint64_t stage_full[2], stage_empty[2], acc_full[2], acc_empty[2], done_bar;
     __shared__ uint32_t tslot;
     __shared__ int abort_s;
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint8_t* stA[2] = {sm, sm + kAStage};
     uint8_t* yres = sm + 2 * kAStage;                 // Y slices: 32-column tile j at j * kUpdBTile
@@ -1398,7 +1398,7 @@ k_ozaki_gram_db(int64_t m, int n, int np, const int32_t* __restrict__ colexp, in
     __shared__ uint64_t load_bar[2], empty_bar[2], acc_full[2], acc_empty[2], done_bar;
     __shared__ uint32_t tslot;
     __shared__ int abort_s;
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint8_t* stA[2] = {sm, sm + kDbStage};
     uint8_t* stB[2] = {sm + kAStage, sm + kDbStage + kAStage};
@@ -1588,7 +1588,7 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
     __shared__ uint64_t empty_bar[2], full_bar[2], done_bar;
     __shared__ uint32_t tslot;
     __shared__ int abort_s;
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     constexpr int NT = kGramNT;
     constexpr int kCols = Share<NT>::kDrainCols;
     static_assert(Share<NT>::kChunks == 1, "one 8-row chunk per producer thread");
@@ -1877,7 +1877,7 @@ k_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, i
     __shared__ uint64_t bars[2];
     __shared__ uint32_t tslot;
     __shared__ int abort_s, cs[64], bound_s[2][2][kTileM];   // [group][sub-block of the half][row]
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = tid >> 8, hf = (tid >> 7) & 1, lr = tid & 127;
     uint8_t* tb = sm + 2 * (kAStage + kSsPanel);
     if (warp == 0) {

@@ -215,10 +215,8 @@ __device__ void item_sketch(const BatchArgs& a, int i, double* psm) {
         w.As[static_cast<int64_t>(c) * s + j] = v;
     }
     if (__syncthreads_or(bad) && tid == 0) set_status(info, RPCHOLQR_ERR_NONFINITE);
-    __syncthreads();
-    if (load_status(info) == 0) qr_factor_one_cta<kPThreads>(w.As, s, s, n, np, w.Rs, info, psm, a.smem);
-    __syncthreads();
-    if (load_status(info) == 0)
+    if (!cta_stopped(info)) qr_factor_one_cta<kPThreads>(w.As, s, s, n, np, w.Rs, info, psm, a.smem);
+    if (!cta_stopped(info))
         for (int e = tid; e < np * np + (np / 8) * 64; e += kPThreads)
             prep_tri_entry(w.Rs, np, n, np, w.frag_s, w.diag_s, e);
     cta_signal(&a.ctr[4 * i + 0], 1);
@@ -259,7 +257,6 @@ __device__ void item_pass1(const BatchArgs& a, int i, int64_t b, double* psm, in
     const int n = a.n[i], np = pad16(n);
     if (!cta_wait_geq(&a.ctr[4 * i + 0], 1, a.spin, ok_s, a.queue + 2) && threadIdx.x == 0)
         set_status(info, RPCHOLQR_ERR_TIMEOUT);
-    __syncthreads();
     // wait for this part's turn to add its Gram partial (parts are summed in the order b = 0, 1, ...)
     auto before = [&] {
         if (!cta_wait_geq(turn, static_cast<int>(b), a.spin, ok_s, a.queue + 2) && threadIdx.x == 0)
@@ -273,7 +270,7 @@ __device__ void item_pass1(const BatchArgs& a, int i, int64_t b, double* psm, in
         if (*go_s) G[pr * np + pc] += v;
     };
     bool bad = false;
-    if (load_status(info) == 0) {
+    if (!cta_stopped(info)) {
         bad = item_rows_np<true>(np, a.sms, a.A[i], a.lda[i], a.Q[i], a.ldq[i], a.m[i], n, w.frag_s, w.diag_s, true, b,
                                  parts, psm, before, emit);
     } else {
@@ -290,8 +287,7 @@ __device__ void item_chol(const BatchArgs& a, int i, double* psm, int* ok_s) {
     const int n = a.n[i], np = pad16(n);
     if (!cta_wait_geq(&a.ctr[4 * i + 1], parts, a.spin, ok_s, a.queue + 2) && threadIdx.x == 0)
         set_status(info, RPCHOLQR_ERR_TIMEOUT);
-    __syncthreads();
-    if (load_status(info) == 0 && cholesky_one_cta<kPThreads>(w.G, np, n, np, w.R1, info, *reinterpret_cast<CholShared*>(psm))) {
+    if (!cta_stopped(info) && cholesky_one_cta<kPThreads>(w.G, np, n, np, w.R1, info, *reinterpret_cast<CholShared*>(psm))) {
         __syncthreads();
         for (int e = threadIdx.x; e < np * np + (np / 8) * 64; e += kPThreads)
             prep_tri_entry(w.R1, np, n, np, w.frag_1, w.diag_1, e);
@@ -311,8 +307,7 @@ __device__ void item_pass2(const BatchArgs& a, int i, int64_t b, double* psm, in
     const int n = a.n[i], np = pad16(n);
     if (!cta_wait_geq(&a.ctr[4 * i + 2], 1, a.spin, ok_s, a.queue + 2) && threadIdx.x == 0)
         set_status(info, RPCHOLQR_ERR_TIMEOUT);
-    __syncthreads();
-    if (load_status(info) == 0) {
+    if (!cta_stopped(info)) {
         double* Q = a.Q[i];
         item_rows_np<false>(np, a.sms, Q, a.ldq[i], Q, a.ldq[i], a.m[i], n, w.frag_1, w.diag_1, false, b, parts, psm,
                             [] {}, [](int, int, double) {});

@@ -41,7 +41,7 @@ k_rowpass(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int n
           double* __restrict__ gpart, int32_t* info, bool check_finite, int32_t* rowexp, int rowexp_mode,
           int32_t* colexp) {
     extern __shared__ double panel[];
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     double* out = SYRK ? gpart + static_cast<size_t>(blockIdx.x) * NP * NP : nullptr;
     const int nw = SHORT ? blockDim.x >> 5 : kRowpassWarps;
     const bool bad = rowpass_panels<NP, SYRK, SHORT ? 16 : rowpass_rows_per_warp(NP),

@@ -71,7 +71,7 @@ k_qr_update(double* __restrict__ W, int64_t lds, int s, int k0, int nb, int n, c
 __global__ void __launch_bounds__(256)
 k_qr_out(const double* __restrict__ W, int64_t lds, int n, int np, const double* __restrict__ betas, double* __restrict__ Rs,
          double* __restrict__ Rs_user, int32_t* info) {
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     const int64_t e = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
     const bool bad = e < static_cast<int64_t>(np) * np && !qr_out_entry(W, lds, n, np, betas, static_cast<int>(e), Rs, Rs_user);
     if (__syncthreads_or(bad) && threadIdx.x == 0) set_status(info, RPCHOLQR_ERR_SINGULAR_SKETCH);

@@ -26,7 +26,7 @@ __global__ void k_chol_init(const double* __restrict__ G, int64_t ldg, int n, in
 __global__ void __launch_bounds__(128)
 k_chol_panel(double* R, double* W, double* __restrict__ D, int n, int np, int k, int32_t* info) {
     __shared__ CholShared sh;
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     const int tid = threadIdx.x, warp = tid >> 5, nb = (n + kCb - 1) / kCb;
     const int k0 = k * kCb, nk = n - k0 < kCb ? n - k0 : kCb;
     double* Rk = R + static_cast<int64_t>(k0) * np;

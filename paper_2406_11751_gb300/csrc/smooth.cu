@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(256)
 k_dct_pass_a(const TA* __restrict__ A, int64_t m, int n, int64_t lda, int p, int l1, int lg, int cs,
              const int8_t* __restrict__ sgn, Cplx* __restrict__ T, int32_t* info) {
     extern __shared__ Cplx cs_buf[];
-    if (load_status(info) != 0) return;
+    if (cta_stopped(info)) return;
     const int64_t N = int64_t{1} << p;
     const int L = 1 << l1, l2 = p - l1, H = 1 << l2, G = 1 << lg;
     const int U = G * cs;
