@@ -1836,9 +1836,11 @@ __device__ __forceinline__ bool ss_group_or(bool v, int g) {
         : "memory");
     return r != 0;
 }
-// The MMAs of an update: NKK K = 16 steps of the group's stage against the table's slices (N columns), by one thread.
+// The MMAs of an update: NKK K = 16 steps of the group's stage against the table's slices (N columns), by one thread, and
+// their commit (counted in `commits`).
 template <int NKK, int N>
-__device__ __forceinline__ void ss_issue(uint32_t tset, uint32_t st, uint32_t B, uint64_t* bar) {
+__device__ __forceinline__ void ss_issue(uint32_t tset, uint32_t st, uint32_t B, uint64_t* bar, uint32_t& commits) {
+    ++commits;
     const uint64_t a0 = sdesc(st), b0 = sdesc(B);
 #pragma unroll
     for (int kk = 0; kk < NKK; ++kk)
@@ -1907,7 +1909,7 @@ k_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, i
     const uint32_t tset = tslot + 256u * g, tl = tset + (static_cast<uint32_t>((lr >> 5) * 32) << 16);
     const int32_t* ey = reinterpret_cast<const int32_t*>(tb + kSsEOff);
     const int64_t ntm = (m + kTileM - 1) / kTileM;
-    uint32_t phase = 0;
+    uint32_t phase = 0, commits = 0;
     bool bad = false, ok = true;
     int cm0 = kNoExp, cm1 = kNoExp;   // bounds of columns lane and 32 + lane over the rows of this warp
     for (int64_t t = blockIdx.x + static_cast<int64_t>(g) * gridDim.x; t < ntm; t += 2 * static_cast<int64_t>(gridDim.x)) {
@@ -1915,6 +1917,7 @@ k_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, i
         int re = kNoExp, E32 = kNoExp;
         auto wait_mma = [&]() {
             if (ok) ok = mbar_wait_ab(bar, phase, &abort_s, spin);
+            if (!ok) abort_s = 1;
             __syncwarp();
             phase ^= 1u;
             tc_after_sync();
@@ -1971,9 +1974,9 @@ k_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, i
                     fence_async_smem();
                     tc_before_sync();
                     ss_group_sync(g);
-                    if ((tid & 255) == 0) {
+                    if ((tid & 255) == 0 && ok) {   // (see the closing wait)
                         tc_after_sync();
-                        ss_issue<1, kSsN1>(tset, smem_u32(st), smem_u32(tb + (h == 0 ? ss_b_off(0) : ss_b_off(2))), bar);
+                        ss_issue<1, kSsN1>(tset, smem_u32(st), smem_u32(tb + (h == 0 ? ss_b_off(0) : ss_b_off(2))), bar, commits);
                     }
                     __syncwarp();
                 }
@@ -2008,9 +2011,9 @@ k_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, i
                 tc_before_sync();
             }
             ss_group_sync(g);   // every row of the half is final, and sliced
-            if (32 * h + 32 < nc && (tid & 255) == 0) {
+            if (32 * h + 32 < nc && (tid & 255) == 0 && ok) {
                 tc_after_sync();
-                ss_issue<2, kSsN2>(tset, smem_u32(st), smem_u32(tb + ss_b_off(1)), bar);
+                ss_issue<2, kSsN2>(tset, smem_u32(st), smem_u32(tb + ss_b_off(1)), bar, commits);
             }
             __syncwarp();
             for (int r = warp & 7; r < kTileM; r += 8)
@@ -2026,10 +2029,11 @@ k_split_solve(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, i
             break;
         }
     }
-    if (!ok) {
-        abort_s = 1;
-        mbar_wait(bar, phase ^ 1u);   // this group's last MMAs are done before the tensor memory is released
-    }
+    // The group's MMAs are done before the tensor memory is released.  The issuing thread has seen every commit but its
+    // last one complete: it issues nothing once a wait of its own gave up, so one commit at most is open and the parity
+    // of its number names it.
+    if (commits > 0 && !mbar_wait(bar, (commits - 1) & 1u)) abort_s = 1;
+    __syncwarp();
     if (lane < nc) atomicMax(&cs[lane], cm0);
     if (32 + lane < nc) atomicMax(&cs[32 + lane], cm1);
     tc_before_sync();
