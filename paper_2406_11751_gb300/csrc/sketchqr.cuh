@@ -117,12 +117,15 @@ __device__ __forceinline__ bool qr_bar_wait(uint64_t* bar, uint32_t parity) {
 // r ~ 1 / (x + nrm |alpha|), good to 2^-20, and one third-order step each -- Halley's iteration
 // nrm = t + t (e / 2 + 3 e^2 / 8), t = x y, e = 1 - t y, and the Neumann series g = r (1 + f + f^2),
 // f = 1 - (x + nrm |alpha|) r.  The third powers left out and the truncations are below 2^-57 of the results,
-// which are then rounded to FP64.  Outside the range where this is safe (and for infinities and NaN) the plain
-// operations are used.
-__device__ __forceinline__ void qr_scalars(double alpha, double x, double& nrm, double& g) {
+// which are then rounded to FP64.  Outside qr_in_range the plain operations are used and false is returned.
+__device__ __forceinline__ bool qr_in_range(double x) {   // x >= 0 or NaN
+    const int xe = (__double2hiint(x) >> 20) - 1023;
+    return xe >= -900 && xe <= 900;
+}
+__device__ __forceinline__ bool qr_scalars(double alpha, double x, double& nrm, double& g) {
     const unsigned long long xb = static_cast<unsigned long long>(__double_as_longlong(x));
     const int xe = static_cast<int>(xb >> 52) - 1023, k = xe & ~1;
-    if (xe >= -900 && xe <= 900) {   // (x >= 0: the sign bit is clear, or x is NaN and out of this range)
+    if (qr_in_range(x)) {
         constexpr unsigned long long kFrac = (1ull << 52) - 1, kOne = 1ull << 52;
         const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(alpha));
         const int ae = static_cast<int>((ab >> 52) & 0x7FF), sh = ae - 1023 - k / 2 + 9;
@@ -150,14 +153,19 @@ __device__ __forceinline__ void qr_scalars(double alpha, double x, double& nrm, 
         const unsigned long long M = G << lz;   // rounded below without leaving 64 bits: M may be 2^64 - 1
         g = __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(1022 - lz - k) << 52) + (M >> 11) +
                                                         ((M >> 10) & 1)));
-    } else {
-        nrm = sqrt(x);
-        g = 1.0 / (nrm * (nrm + fabs(alpha)));
+        return true;
     }
+    nrm = sqrt(x);
+    g = 1.0 / (nrm * (nrm + fabs(alpha)));
+    return false;
 }
 
 // Factor the panel of columns k0 .. k0 + nb - 1 (rows k0 .. s - 1) of W (column-major, ld lds) by the calling
 // CTA as CTA `rank` of `csize` (CLUSTER: a thread-block cluster, csize a power of two <= 16; otherwise one CTA).
+// A column whose remaining norm is outside [2^-450, 2^450] is scaled by a power of two and its products are formed again
+// (at most twice, which brings any column into the range): unscaled, g and the products over- or underflow.  H_j does
+// not depend on the scale of v_j; R's entry takes it back.  Where the sum of squares itself overflows, R's diagonal entry
+// is infinite and the sketch counts as singular.
 // W's panel columns become V (v_j from row j down, vp on the diagonal; g_j = 0 where nothing is reflected) with R
 // above the diagonal; L[j * ldl + k] = v_j^T v_k (k < j), g and betas[k0 + j].  SMEM: panel is shared memory for
 // this CTA's rows (kQrLd doubles each); otherwise the panel is worked on in place.
@@ -258,90 +266,130 @@ __device__ __forceinline__ bool qr_panel(double* W, int64_t lds, int s, int k0, 
         sh.part[q][lane] = mine ? (d[0] + d[1]) + (d[2] + d[3]) : 0.0;
     };
     int pg = -g0, pend = rg;                     // the pivot row's group within this CTA, and that group's end
-    if (pg >= 0 && pg < ng && warp == pg % NW) {
-        const double v = mine ? Pl[(0 - rbeg) * kSi] : 0.0;
-        if constexpr (CLUSTER) sh.row_out[lane] = v;
-        else sh.row[0][lane] = v;
-    }
-    for (int q = warp; q < ng; q += NW) rows_step(std::false_type{}, q, -1, 0.0);
-    for (int j = 0; j < nb; ++j) {
-        const int par = j & 1;
-        const bool owner_cta = pg >= 0 && pg < ng, owner = owner_cta && warp == pg % NW;
-        __syncthreads();
-        for (int e = tid; e < ng / 4 * 128; e += NT) {
-            const int q = e >> 7, col = (e & 127) >> 2, sub = e & 3;
-            if constexpr (CLUSTER) {
-                if (owner_cta && q == 0) {
-                    const double v = sh.row_out[col];
+    // Pivot row j and the products of column j with every column, formed from the panel for exchange `ex`.
+    auto products = [&](int j, int ex) {
+        if (pg >= 0 && pg < ng && warp == pg % NW) {
+            const double v = mine ? Pl[(j - rbeg) * kSi] : 0.0;
+            if constexpr (CLUSTER) sh.row_out[lane] = v;
+            else sh.row[ex & 1][lane] = v;
+        }
+        for (int q = warp; q < ng; q += NW) rows_step(std::false_type{}, q, j - 1, 0.0);
+    };
+    // The columns from j0 on; ex: exchanges so far.  Returns nb, or (not SCALE) the column that needs scaling, its exchange
+    // made.  SCALE is a loop of its own, so that the usual one holds nothing of it (3 us a panel otherwise).
+    auto columns = [&](auto scale_t, int j0, int ex) -> int {
+        constexpr bool SCALE = decltype(scale_t)::value;
+        int tries = 0;                               // scalings of the current column
+        double unscale = 1.0;                        // what takes them back
+        for (int j = j0; j < nb;) {
+            const int par = ex & 1;
+            const bool owner_cta = pg >= 0 && pg < ng, owner = owner_cta && warp == pg % NW;
+            __syncthreads();
+            for (int e = tid; e < ng / 4 * 128; e += NT) {
+                const int q = e >> 7, col = (e & 127) >> 2, sub = e & 3;
+                if constexpr (CLUSTER) {
+                    if (owner_cta && q == 0) {
+                        const double v = sh.row_out[col];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if ((tid & 3) + 4 * i < csize)
+                                st_async(remote[i] + at(&sh.row[par][col]), remote[i] + at(&sh.bar[par]), v);
+                    }
+                }
+                double v = sh.part[4 * q + sub][col];
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                if constexpr (CLUSTER) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         if ((tid & 3) + 4 * i < csize)
-                            st_async(remote[i] + at(&sh.row[par][col]), remote[i] + at(&sh.bar[par]), v);
+                            st_async(remote[i] + at(&sh.quad[par][g0 / 4 + q][col]), remote[i] + at(&sh.bar[par]), v);
+                } else {
+                    if (sub == 0) sh.quad[par][q][col] = v;
                 }
             }
-            double v = sh.part[4 * q + sub][col];
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
             if constexpr (CLUSTER) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if ((tid & 3) + 4 * i < csize)
-                        st_async(remote[i] + at(&sh.quad[par][g0 / 4 + q][col]), remote[i] + at(&sh.bar[par]), v);
+                if (ok) ok = qr_bar_wait(&sh.bar[par], static_cast<uint32_t>((ex >> 1) & 1));
+                __syncwarp();
             } else {
-                if (sub == 0) sh.quad[par][q][col] = v;
+                __syncthreads();
             }
-        }
-        if constexpr (CLUSTER) {
-            if (ok) ok = qr_bar_wait(&sh.bar[par], static_cast<uint32_t>((j >> 1) & 1));
-            __syncwarp();
-        } else {
+            if (tid < 128) {
+                const int col = tid >> 2, sub = tid & 3;
+                double v = (sh.quad[par][sub][col] + sh.quad[par][sub + 4][col]) +
+                           (sh.quad[par][sub + 8][col] + sh.quad[par][sub + 12][col]);
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                if (sub == 0) sh.D[col] = v;
+            }
             __syncthreads();
-        }
-        if (tid < 128) {
-            const int col = tid >> 2, sub = tid & 3;
-            double v = (sh.quad[par][sub][col] + sh.quad[par][sub + 4][col]) +
-                       (sh.quad[par][sub + 8][col] + sh.quad[par][sub + 12][col]);
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            if (sub == 0) sh.D[col] = v;
-        }
-        __syncthreads();
-        // every thread has seen this phase; the next one of this barrier cannot complete before it is armed
-        if (CLUSTER && tid == 0) qr_bar_arm(&sh.bar[par]);
-        // v = x - beta e_j with beta = -sign(alpha) nrm; t = v^T a_k, w = g t
-        const double rk = sh.row[par][lane], alpha = sh.row[par][j], sigma = sh.D[j];
-        const double u = fma(alpha, rk, sh.D[lane]);
-        double nrm = 0.0, gj = 0.0;
-        if (sigma != 0.0) qr_scalars(alpha, fma(alpha, alpha, sigma), nrm, gj);   // else nothing to reflect: v = 0
-        const double sn = alpha >= 0.0 ? nrm : -nrm;
-        const double t = sigma != 0.0 ? fma(sn, rk, u) : 0.0;
-        const double vp = sigma != 0.0 ? alpha + sn : 0.0;
-        const double w = (lane > j && mine) ? gj * t : 0.0;
-        if (rank == 0 && warp == 0) {
-            if (lane < j) L[j * ldl + lane] = t;
-            if (lane == j) {
-                g[j] = gj;
-                betas[k0 + j] = sigma != 0.0 ? -sn : alpha;
+            // every thread has seen this phase; the next one of this barrier cannot complete before it is armed
+            if (CLUSTER && tid == 0) qr_bar_arm(&sh.bar[par]);
+            ++ex;
+            // v = x - beta e_j with beta = -sign(alpha) nrm; t = v^T a_k, w = g t
+            const double rk = sh.row[par][lane], alpha = sh.row[par][j], sigma = sh.D[j];
+            const double u = fma(alpha, rk, sh.D[lane]), x = fma(alpha, alpha, sigma);
+            const bool reflect = (__double_as_longlong(sigma) << 1) != 0;   // else nothing to reflect: v = 0
+            double nrm = 0.0, gj = 0.0;
+            const bool in_range = reflect ? qr_scalars(alpha, x, nrm, gj) : qr_in_range(x);
+            if (!in_range) {   // (the same x in every thread of every CTA)
+                if constexpr (!SCALE) return j;
+                if (tries < 2 && isfinite(x)) {
+                    const bool up = x < 1.0;
+                    const double f = up ? 0x1p500 : 0x1p-600;
+                    unscale *= up ? 0x1p-500 : 0x1p600;
+                    ++tries;
+                    for (int q = warp; q < ng; q += NW) {
+                        const int ib = (g0 + q) * rg > j ? (g0 + q) * rg : j;
+                        const int ie = (g0 + q + 1) * rg < nrows ? (g0 + q + 1) * rg : nrows;
+                        for (int i = ib + lane; i < ie; i += 32) P[(i - rbeg) * kSi + j * sc] *= f;
+                    }
+                    __syncwarp();
+                    products(j, ex);
+                    continue;
+                }
             }
-        }
-        if (owner && mine && lane >= j) Pl[(j - rbeg) * kSi] = lane == j ? vp : fma(-vp, w, rk);
-        if (j + 1 == nb) break;
-        // the next pivot row first
-        if (j + 1 == pend) {
-            ++pg;
-            pend += rg;
-        }
-        if (pg >= 0 && pg < ng && warp == pg % NW) {
-            double v = 0.0;
-            if (mine) {
-                v = fma(-P[(j + 1 - rbeg) * kSi + j * sc], w, Pl[(j + 1 - rbeg) * kSi]);
-                Pl[(j + 1 - rbeg) * kSi] = v;
+            const double sn = alpha >= 0.0 ? nrm : -nrm;
+            const double t = reflect ? fma(sn, rk, u) : 0.0;
+            const double vp = reflect ? alpha + sn : 0.0;
+            const double w = (lane > j && mine) ? gj * t : 0.0;
+            if (rank == 0 && warp == 0) {
+                if (lane < j) L[j * ldl + lane] = t;
+                if (lane == j) {
+                    g[j] = gj;
+                    const double d = reflect ? -sn : alpha;
+                    betas[k0 + j] = SCALE ? d * unscale : d;
+                }
             }
-            if constexpr (CLUSTER) sh.row_out[lane] = v;
-            else sh.row[par ^ 1][lane] = v;
+            if (owner && mine && lane >= j) Pl[(j - rbeg) * kSi] = lane == j ? vp : fma(-vp, w, rk);
+            if (j + 1 == nb) break;
+            // the next pivot row first
+            if (j + 1 == pend) {
+                ++pg;
+                pend += rg;
+            }
+            if (pg >= 0 && pg < ng && warp == pg % NW) {
+                double v = 0.0;
+                if (mine) {
+                    v = fma(-P[(j + 1 - rbeg) * kSi + j * sc], w, Pl[(j + 1 - rbeg) * kSi]);
+                    Pl[(j + 1 - rbeg) * kSi] = v;
+                }
+                if constexpr (CLUSTER) sh.row_out[lane] = v;
+                else sh.row[par ^ 1][lane] = v;
+            }
+            for (int q = warp; q < ng; q += NW) rows_step(std::true_type{}, q, j, w);
+            __syncwarp();
+            ++j;
+            tries = 0;
+            unscale = 1.0;
         }
-        for (int q = warp; q < ng; q += NW) rows_step(std::true_type{}, q, j, w);
-        __syncwarp();
+        return nb;
+    };
+    products(0, 0);
+    const int stop = columns(std::false_type{}, 0, 0);
+    if (stop < nb) {   // from here on, this column's products once more
+        products(stop, stop + 1);
+        columns(std::true_type{}, stop, stop + 1);
     }
     __syncthreads();
     if constexpr (SMEM) {
