@@ -304,13 +304,32 @@ __device__ __forceinline__ double scale_pow2_int(long long I, int e) {
     return __longlong_as_double(static_cast<long long>(b | (neg << 63)));
 }
 
+// One window's value w added to an int64 total.  Operands reach their power-of-two bounds, so units of 2^-53 of the scale
+// hold the sum of 1024 terms and no more; HALF (K up to 2048): the total is 2 acc + bit, the bit in bit j of `bits`.
+template <bool HALF>
+__device__ __forceinline__ void add_window(long long& acc, uint32_t& bits, int j, long long w) {
+    if constexpr (HALF) {
+        const long long t = w + ((bits >> j) & 1u);
+        acc += t >> 1;
+        bits = (bits & ~(1u << j)) | (static_cast<uint32_t>(t & 1) << j);
+    } else {
+        acc += w;
+    }
+}
+// That total times 2^e.
+template <bool HALF>
+__device__ __forceinline__ double scale_total(long long acc, uint32_t bits, int j, int e) {
+    if (!HALF) return scale_pow2(acc, e);
+    const bool fits = acc < (1ll << 61) && acc >= -(1ll << 61);   // else the bit is below the result's last place
+    return fits ? scale_pow2(2 * acc + ((bits >> j) & 1u), e) : scale_pow2(acc, e + 1);
+}
+
 // Add the TMEM group sums of this thread's row and its NC columns (col0.. of the 64-column tile,
-// read CW at a time) to int64 accumulators in units of 2^-53 (U53) or 2^-49 of the operand scale.
-// The sliced operands are below 0.51 of their power-of-two bounds, so a K-term sum stays below
-// 0.26 K scale: units of 2^-53 hold K < 2^10 / 0.26 (about 3900) terms -- the products take K <= 2048,
-// a factor 2 below -- and units of 2^-49 hold 2^14 (a 64-window flush of the Gram).
-template <bool U53, int NC, int CW = 8>
-__device__ __forceinline__ void drain_acc(uint32_t tmem, int warp, int col0, long long (&acc)[NC]) {
+// read CW at a time) to int64 accumulators in units of 2^-53 (U53; HALF and bits: add_window) or 2^-49 of the
+// operand scale, which hold 2^14 terms (a 64-window flush of the Gram takes 2^13).
+template <bool U53, int NC, int CW = 8, bool HALF = false>
+__device__ __forceinline__ void drain_acc(uint32_t tmem, int warp, int col0, long long (&acc)[NC], uint32_t& bits) {
+    static_assert(!HALF || NC <= 32, "one bit a column");
 #pragma unroll
     for (int c0 = 0; c0 < NC; c0 += CW) {
         float mg[kGroups][CW];
@@ -324,7 +343,7 @@ __device__ __forceinline__ void drain_acc(uint32_t tmem, int warp, int col0, lon
             float grp[kGroups];
 #pragma unroll
             for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][j];
-            acc[c0 + j] += combine_units<U53 ? 53 : 49>(grp);
+            add_window<HALF>(acc[c0 + j], bits, c0 + j, combine_units<U53 ? 53 : 49>(grp));
         }
     }
 }
@@ -517,22 +536,22 @@ __device__ __forceinline__ void prefetch_x(const double* X, int64_t ldx, int64_t
 // Write the finished tile (rows row0 + 0..127, columns 64 tn + 0..63) of C = X Y through the staging
 // buffer W (run by the NT producer threads): each thread puts its row's NC values into W, then the tile
 // is written in whole rows.  The values come from the TMEM accumulators (single window) or from acc (WIN).
-template <bool WIN, bool SUB, int NT, int NC>
+template <bool WIN, bool SUB, bool HALF, int NT, int NC>
 __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid, int64_t row0, int tn, int E,
                                                 int N, const int32_t* __restrict__ yexp, const double* B,
                                                 int64_t ldb, double* C, int64_t ldc, int64_t m, double* W,
-                                                long long (&acc)[NC]) {
+                                                long long (&acc)[NC], uint32_t& bits) {
     const int lr = tid & (kTileM - 1), rq = tid / kTileM;
     const int col0 = tn * kTileN;
     const int ncols = N - col0 < kTileN ? N - col0 : kTileN;
     double* wr = W + lr * kEpiLd + NC * rq;
     if (WIN) {
-        drain_acc<true, NC, 4>(tmem, warp, NC * rq, acc);
+        drain_acc<true, NC, 4, HALF>(tmem, warp, NC * rq, acc, bits);
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
             const int col = col0 + NC * rq + j;
             const int ey = col < N ? yexp[col] : kNoExp;
-            const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2(acc[j], E + ey - 53) : 0.0;
+            const double v = (E > kNoExp && ey > kNoExp) ? scale_total<HALF>(acc[j], bits, j, E + ey - 53) : 0.0;
             wr[j] = v;
         }
     } else {
@@ -580,8 +599,8 @@ __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid
 // X: m x K FP64 (ldx) with row exponent bounds xexp[m] (max over the K columns used);
 // Y: pre-sliced by k_ozaki_slice_cols (K x N, column bounds yexp[N]);
 // B, C: m x N FP64 (ldb, ldc); C may equal B.  Persistent grid over 128-row x 64-column tiles.
-// WIN (128 < K <= 1024): the K range is cut into exactness windows of 128, each drained into int64
-// accumulators in units of 2^-53 of the scale (the same resolution as a single window).
+// WIN (128 < K <= 2048): the K range is cut into exactness windows of 128, each drained into int64
+// accumulators in units of 2^-53 of the scale (the same resolution as a single window; HALF above K = 1024).
 // The CTA's (tile, K-stage) sequence is one stream of stages over two shared-memory buffers: stage g is
 // sliced while the MMAs of stage g - 1 run; when stage g opens a new exactness window (or a new tile)
 // the previous window's accumulators are drained (into int64, or out to C at a tile end) before its
@@ -632,7 +651,7 @@ struct StageWalk {
     }
 };
 
-template <bool WIN, bool SUB>
+template <bool WIN, bool SUB, bool HALF = false>
 __global__ void __launch_bounds__((WIN ? kThreadsWin : kThreads) + 32, 1)
 k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, int K,
                 const uint8_t* __restrict__ yblocks, const int32_t* __restrict__ yexp, int N, const double* B,
@@ -710,6 +729,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
         bool pending[2] = {false, false};
         bool timed_out = false;
         long long acc[NC];
+        uint32_t bits = 0;
 #pragma unroll
         for (int j = 0; j < NC; ++j) acc[j] = 0;
         int64_t cur_row0 = 0;               // the tile whose accumulators are in TMEM
@@ -780,12 +800,13 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
                 tc_after_sync();
                 if (kw == 0) {
                     // every MMA so far is complete: stage sp's buffer stages the output tile
-                    gemm_store_tile<WIN, SUB, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
-                                                 reinterpret_cast<double*>(stA[sp]), acc);
+                    gemm_store_tile<WIN, SUB, HALF, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
+                                                 reinterpret_cast<double*>(stA[sp]), acc, bits);
+                    bits = 0;
 #pragma unroll
                     for (int j = 0; j < NC; ++j) acc[j] = 0;
                 } else if (WIN) {
-                    drain_acc<true, NC, 4>(tmem, warp, NC * rq, acc);
+                    drain_acc<true, NC, 4, HALF>(tmem, warp, NC * rq, acc, bits);
                 }
             }
             if (kw == 0) {
@@ -811,8 +832,8 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
                 }
             if (!timed_out) {
                 tc_after_sync();
-                gemm_store_tile<WIN, SUB, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
-                                             reinterpret_cast<double*>(stA[0]), acc);
+                gemm_store_tile<WIN, SUB, HALF, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
+                                             reinterpret_cast<double*>(stA[0]), acc, bits);
             }
         }
         if (timed_out) abort_s = 1;
@@ -886,9 +907,9 @@ __device__ __forceinline__ long long shift_round(long long I, int sh) {
 // Add one window's group sums of this thread's row (TMEM address taddr: set + lane quarter) and
 // columns col0 .. col0 + NC - 1 of the 32-column tile to int64 accumulators in units of 2^-53 (U49: 2^-49)
 // of the window's scale, shifted down by sh bits (a window sliced against a row bound 2^sh below the
-// tile's).
-template <int NC, bool U49 = false>
-__device__ __forceinline__ void drain_set32(uint32_t taddr, int col0, int sh, long long (&acc)[NC]) {
+// tile's).  HALF and bits: add_window.
+template <int NC, bool U49 = false, bool HALF = false>
+__device__ __forceinline__ void drain_set32(uint32_t taddr, int col0, int sh, long long (&acc)[NC], uint32_t& bits) {
 #pragma unroll
     for (int c0 = 0; c0 < NC; c0 += 8) {
         float mg[kGroups][8];
@@ -900,7 +921,7 @@ __device__ __forceinline__ void drain_set32(uint32_t taddr, int col0, int sh, lo
             float grp[kGroups];
 #pragma unroll
             for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][j];
-            acc[c0 + j] += shift_round(combine_units<U49 ? 49 : 53>(grp), sh);
+            add_window<HALF>(acc[c0 + j], bits, c0 + j, shift_round(combine_units<U49 ? 49 : 53>(grp), sh));
         }
     }
 }
@@ -918,7 +939,7 @@ __device__ __forceinline__ bool epi_sync_or(bool v) {
     return r != 0;
 }
 
-template <bool SUB>
+template <bool SUB, bool HALF>
 __global__ void __launch_bounds__(kDbThreads, 1)
 k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xexp, int K,
                 const uint8_t* __restrict__ yblocks, const int32_t* __restrict__ yexp, int N, const double* B,
@@ -1075,6 +1096,7 @@ k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xe
                 }
             }
             long long acc[kDbCols];
+            uint32_t bits = 0;
 #pragma unroll
             for (int j = 0; j < kDbCols; ++j) acc[j] = 0;
             for (int w = 0; w < nwin; ++w, ++wc) {
@@ -1090,8 +1112,8 @@ k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xe
                     const int ew = bexp[w * ld_bexp + row];
                     sh = ew > kNoExp ? E - ew : 63;
                 }
-                drain_set32<kDbCols>(tmem + lane_off + static_cast<uint32_t>(set) * kDbSetCols, kDbCols * h, sh,
-                                     acc);
+                drain_set32<kDbCols, false, HALF>(tmem + lane_off + static_cast<uint32_t>(set) * kDbSetCols, kDbCols * h, sh,
+                                                  acc, bits);
                 tc_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[set]);
@@ -1116,7 +1138,7 @@ k_ozaki_gemm_db(const uint8_t* __restrict__ aimg, const int32_t* __restrict__ xe
                 const int col = col0 + kDbCols * h + j;
                 const int ey = col < N ? yexp[col] : kNoExp;
                 W[lr * kDbEpiLd + kDbCols * h + j] =
-                    (E > kNoExp && ey > kNoExp) ? scale_pow2(acc[j], E + ey - 53) : 0.0;
+                    (E > kNoExp && ey > kNoExp) ? scale_total<HALF>(acc[j], bits, j, E + ey - 53) : 0.0;
             }
             epi_sync();
 #pragma unroll
@@ -1509,6 +1531,7 @@ k_ozaki_gram_db(int64_t m, int n, int np, const int32_t* __restrict__ colexp, in
         long long acc[kDbCols];
 #pragma unroll
         for (int j = 0; j < kDbCols; ++j) acc[j] = 0;
+        uint32_t no_bits = 0;
         bool flushed = accum != 0, ok = true;
         // acc into the FP64 partial (the first flush of a launch that does not accumulate initialises it)
         auto flush = [&]() {
@@ -1537,7 +1560,7 @@ k_ozaki_gram_db(int64_t m, int n, int np, const int32_t* __restrict__ colexp, in
             }
             tc_after_sync();
             drain_set32<kDbCols, true>(tmem + lane_off + static_cast<uint32_t>(set) * kDbSetCols, kDbCols * h, 0,
-                                       acc);
+                                       acc, no_bits);
             tc_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[set]);
@@ -1659,9 +1682,10 @@ k_ozaki_gram(const double* __restrict__ X, int64_t ldx, int64_t m, int n, int np
         // Drain the window just finished (its MMAs complete) into acc; every 64 windows, and at the end,
         // add acc into the CTA's FP64 partial (the first flush initialises it) and clear it.
         bool flushed = false;
+        uint32_t no_bits = 0;
         auto drain_window = [&](bool flush) {
             tc_after_sync();
-            drain_acc<false, kCols, 4>(tmem, warp, kCols * rq, acc);
+            drain_acc<false, kCols, 4>(tmem, warp, kCols * rq, acc, no_bits);
             if (flush && p < np) {
                 double* out = gpart + static_cast<size_t>(rr) * np * np + static_cast<size_t>(p) * np;
 #pragma unroll
@@ -2094,8 +2118,8 @@ cudaError_t launch_ozaki_gemm(bool sub, const double* X, int64_t ldx, const int3
                               int64_t ldb, double* C, int64_t ldc, int64_t m, int32_t* info, int grid,
                               cudaStream_t st, long spin, bool y_upper, const uint8_t* aimg, int img_nkw,
                               const int32_t* bexp, int64_t ld_bexp) {
-    if (K > 64 * oz::kKW) return cudaErrorInvalidValue;   // int64 accumulators hold K <= 2048 (see drain_acc)
-    const bool win = K > 4 * oz::kKW;
+    if (K > 64 * oz::kKW) return cudaErrorInvalidValue;   // the totals hold K <= 2048 (add_window)
+    const bool win = K > 4 * oz::kKW, half = K > 32 * oz::kKW;
     const int nt = win ? oz::kThreadsWin : oz::kThreads;
     cudaError_t err;
     if (sub && K <= oz::kKW && N <= oz::kUpdMaxN) {
@@ -2109,7 +2133,8 @@ cudaError_t launch_ozaki_gemm(bool sub, const double* X, int64_t ldx, const int3
     }
     if (aimg) {
         // pre-sliced X: the double-buffered kernel over 128 x 32 tiles
-        auto kdb = sub ? oz::k_ozaki_gemm_db<true> : oz::k_ozaki_gemm_db<false>;
+        auto kdb = half ? (sub ? oz::k_ozaki_gemm_db<true, true> : oz::k_ozaki_gemm_db<false, true>)
+                        : (sub ? oz::k_ozaki_gemm_db<true, false> : oz::k_ozaki_gemm_db<false, false>);
         err = cudaFuncSetAttribute(kdb, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::kDbSmem);
         if (err != cudaSuccess) return err;
         const int64_t tiles = ((m + oz::kTileM - 1) / oz::kTileM) * ((N + oz::kDbN - 1) / oz::kDbN);
@@ -2120,7 +2145,8 @@ cudaError_t launch_ozaki_gemm(bool sub, const double* X, int64_t ldx, const int3
                                                     y_upper ? 1 : 0, img_nkw, bexp, ld_bexp);
         return cudaGetLastError();
     }
-    auto kern = win ? (sub ? oz::k_ozaki_gemm_ws<true, true> : oz::k_ozaki_gemm_ws<true, false>)
+    auto kern = half ? (sub ? oz::k_ozaki_gemm_ws<true, true, true> : oz::k_ozaki_gemm_ws<true, false, true>)
+                : win ? (sub ? oz::k_ozaki_gemm_ws<true, true> : oz::k_ozaki_gemm_ws<true, false>)
                     : (sub ? oz::k_ozaki_gemm_ws<false, true> : oz::k_ozaki_gemm_ws<false, false>);
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::kGemmSmem);
     if (err != cudaSuccess) return err;
