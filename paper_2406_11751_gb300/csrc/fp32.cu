@@ -16,6 +16,7 @@ namespace rpq {
 
 constexpr int kF32Blk = 32;      // column block of the row solves
 constexpr int kSyrkRows = 8;     // rows summed in plain FP32
+constexpr int kSyrkSpillRows = 256;   // rows between looks at the pairs' size
 
 __host__ __device__ constexpr int pad32(int n) { return (n + 31) / 32 * 32; }
 
@@ -238,10 +239,34 @@ k_syrk_f32(const float* __restrict__ X, int64_t ldx, int64_t m, int n, int np64,
                 }
         }
     };
+    // The pairs into this thread's FP64 partials: at the end, and before that when they have grown to where an FP32 total
+    // of the range could overflow (rows far heavier than the sampled ones).
+    double* out = gpart + static_cast<size_t>(blockIdx.y) * np64 * np64;
+    bool flushed = false;
+    auto flush = [&]() {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                double& o = out[static_cast<size_t>(64 * I + 8 * ty + i) * np64 + 64 * J + 4 * tx + j];
+                const double v = isfinite(hi[i][j]) ? static_cast<double>(hi[i][j]) + lo[i][j] : hi[i][j];   // an overflow stays one
+                o = flushed ? o + v : v;
+                hi[i][j] = lo[i][j] = 0.0f;
+            }
+        flushed = true;
+    };
     if (rb < re) stage(rb, 0);
     cp_async_commit();
     int b = 0;
     for (int64_t k0 = rb; k0 < re; k0 += 32, b ^= 1) {
+        if ((k0 - rb) % kSyrkSpillRows == 0) {
+            float most = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) most = fmaxf(most, fabsf(hi[i][j]));
+            if (most > 0x1p100f) flush();
+        }
         cp_async_wait_all();
         __syncthreads();   // chunk k0 has landed, and every thread is done with xs[b ^ 1]
         if (k0 + 32 < re) stage(k0 + 32, b ^ 1);
@@ -276,14 +301,7 @@ k_syrk_f32(const float* __restrict__ X, int64_t ldx, int64_t m, int n, int np64,
         }
     }
     cp_async_wait_all();
-    double* out = gpart + static_cast<size_t>(blockIdx.y) * np64 * np64;
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int p = 64 * I + 8 * ty + i, q = 64 * J + 4 * tx + j;
-            out[static_cast<size_t>(p) * np64 + q] = isfinite(hi[i][j]) ? static_cast<double>(hi[i][j]) + lo[i][j] : hi[i][j];   // an overflow stays one
-        }
+    flush();
 }
 
 // dst (n x n float, ld ldd) = float(src) (n x n, ld lds)
