@@ -1242,8 +1242,8 @@ static rpcholqr_status factor_split(rpcholqr_plan p, const double* A, int64_t m,
     launch_split_solve_prep(p->Rs, np, n, p->sstab, info, st);
     ++p->launches;
     pm.mark(RPCHOLQR_PHASE_PASS1);
-    rc = p->aimg ? solve_split_wide(p, A, lda, p->Rs, np, m, n, A1, ld1, info, st, &pm)
-                 : solve_split(p, A, lda, p->Rs, np, m, n, A1, ld1, info, st, &pm);
+    rc = np > kMaxNP ? solve_split_wide(p, A, lda, p->Rs, np, m, n, A1, ld1, info, st, &pm)
+                     : solve_split(p, A, lda, p->Rs, np, m, n, A1, ld1, info, st, &pm);
     if (rc != RPCHOLQR_OK) return rc;
     pm.mark(RPCHOLQR_PHASE_GRAM_REDUCE);
     if ((rc = ozaki_gram_internal(p, A1, m, n, ld1, p->G, np, info, st, true)) != RPCHOLQR_OK) return rc;

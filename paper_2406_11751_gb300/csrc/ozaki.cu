@@ -282,6 +282,33 @@ __device__ __forceinline__ long long combine_units53_k32(const float (&m)[kGroup
     return combine_ints<53>(v);
 }
 
+// The first pass's products keep the pairs with a + b = 9 too (an eighth accumulator, K <= 128): their error reaches A_1
+// multiplied by kappa(A), and the dropped pairs were most of it.  Distance of Q from its value in 80 bits, A_1 by this pass and
+// the rest exact, 1200 rows, kappa = 1e5: n = 33 0.97 -> 0.38e-12, 64 1.05 -> 0.34, 100 1.18 -> 0.42, 128 1.10 -> 0.41 (FP64
+// substitution: 0.41, 0.51, 0.59, 0.68).
+constexpr int kGroups9 = kGroups + 1;
+// Its seven group sums and M_9, in units of 2^-53.
+__device__ __forceinline__ long long combine_units53_d9(const float (&m)[kGroups9]) {
+    int v[kGroups];
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) v[g] = __float2int_rn(m[g]);
+    v[6] += (__float2int_rn(m[7]) + 128) >> 8;
+    return combine_ints<53>(v);
+}
+// The same for K <= 32 in units of 2^-55, |result| <= 2^60: |M_d| <= min(d - 1, 15 - d) 2^19, so two neighbouring sums fit int32,
+// and the integers come from the bit patterns of M + 1.5 2^23 (combine_units53_k32), their offset taken off the pair.
+__device__ __forceinline__ long long combine_units55_k32(const float (&m)[kGroups9]) {
+    constexpr uint32_t kOff = 0x4B400000u;
+    uint32_t b[kGroups9];
+#pragma unroll
+    for (int g = 0; g < kGroups9; ++g) b[g] = __float_as_uint(m[g] + 12582912.0f);
+    const int u = static_cast<int>(b[0] * 256u + (b[1] - 257u * kOff));          // 2^-22
+    const int t = static_cast<int>(b[2] * 256u + (b[3] - 257u * kOff));          // 2^-38
+    const int w = static_cast<int>(b[4] * 512u + (b[5] * 2u - 514u * kOff));     // 2^-55
+    const int l = static_cast<int>(b[6] * 256u + (b[7] - 257u * kOff + 16384u)); // 2^-70, for rounding
+    return (static_cast<long long>(u) << 33) + static_cast<long long>(t) * (1 << 17) + static_cast<long long>(w + (l >> 15));
+}
+
 // I * 2^e: I converted to FP64 (rounded to nearest above 2^53), exponent added in the bit pattern
 // when the result stays normal (the usual case), ldexp otherwise.
 __device__ __forceinline__ double scale_pow2(long long I, int e) {
@@ -354,14 +381,16 @@ __device__ __forceinline__ void drain_acc(uint32_t tmem, int warp, int col0, lon
 // MMA with N = 64 nb multiplies slice a by nb consecutive B slices at once (N <= 256, so slices 1-4 and 5-7 are two
 // MMAs).  first_window: the stage starts an exactness window (slice 1's MMAs clear all seven accumulators).  The
 // descriptors of the stage's two base addresses are formed once; every MMA adds its (constant) offset to the 14-bit
-// start field, which cannot carry (shared memory < 256 KB).
+// start field, which cannot carry (shared memory < 256 KB).  D9: the six pairs with a + b = 9 too, in an eighth
+// accumulator, which slice 2's last pair clears.
+template <bool D9 = false>
 __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t a_base, uint32_t b_base, bool first_window) {
     const uint64_t a0 = sdesc(a_base), b0 = sdesc(b_base);
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
         for (int a = 1; a <= kSlices; ++a) {
-            const int nb = kSlices + 1 - a;
+            const int nb = !D9 ? kSlices + 1 - a : a == 1 ? kSlices : a == 2 ? kSlices - 1 : kSlices + 2 - a;
             const int n1 = nb < 4 ? nb : 4;
             const uint64_t ad = a0 + static_cast<uint32_t>(((a - 1) * kASlice + kk * 256) >> 4);
             const uint32_t acc = (first_window && kk == 0 && a == 1) ? 0u : 1u;
@@ -370,6 +399,10 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t a_base, uint
                 mma_f16_n(tmem + (a + 3) * kTileN, ad,
                           b0 + static_cast<uint32_t>((4 * kBSlice) >> 4) + static_cast<uint32_t>(kk * 16),
                           idesc_f16(kTileN * (nb - 4)), acc);
+            if (D9 && a == 2)
+                mma_f16_n(tmem + 7 * kTileN, ad,
+                          b0 + static_cast<uint32_t>((6 * kBSlice) >> 4) + static_cast<uint32_t>(kk * 16), idesc_f16(kTileN),
+                          (first_window && kk == 0) ? 0u : 1u);
         }
     }
 }
@@ -555,22 +588,25 @@ __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid
             wr[j] = v;
         }
     } else {
+        constexpr int NG = SUB ? kGroups9 : kGroups;
 #pragma unroll 1
         for (int c0 = 0; c0 < NC; c0 += 8) {
-            float mg[kGroups][8];
+            float mg[NG][8];
 #pragma unroll
-            for (int g = 0; g < kGroups; ++g)
+            for (int g = 0; g < NG; ++g)
                 tmem_ld8(tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + g * kTileN + NC * rq + c0, mg[g]);
             tmem_wait_ld();
             if (col0 + NC * rq + c0 >= N) continue;   // (warp-uniform) no valid column in this chunk
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int col = col0 + NC * rq + c0 + j;
-                float grp[kGroups];
+                float grp[NG];
 #pragma unroll
-                for (int g = 0; g < kGroups; ++g) grp[g] = mg[g][j];
+                for (int g = 0; g < NG; ++g) grp[g] = mg[g][j];
                 if (col < N) {
-                    const long long I = combine_units<53>(grp);
+                    long long I;
+                    if constexpr (SUB) I = combine_units53_d9(grp);
+                    else I = combine_units<53>(grp);
                     const int ey = yexp[col];
                     const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2(I, E + ey - 53) : 0.0;
                     wr[c0 + j] = v;
@@ -714,7 +750,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
                 }
                 fphase[s] ^= 1u;
                 tc_after_sync();
-                issue_stage(tmem, smem_u32(stA[s]), smem_u32(stB[s]), (wk.kw & 3) == 0);
+                issue_stage<!WIN && SUB>(tmem, smem_u32(stA[s]), smem_u32(stB[s]), (wk.kw & 3) == 0);
                 mma_commit(&empty_bar[s]);
             }
             // every MMA issued here is complete before the tensor memory is released
@@ -859,7 +895,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
 // warp 9 lane 0 issues the MMAs (7 per K = 16 step: Y's seven 32-column slices are stacked, N = 32 (8 - a)
 // for slice a of X).  Barriers: load[s] (bytes landed) and empty[s] (MMAs of the stage done) per stage
 // buffer; acc_full[b] (the window's MMAs done) and acc_empty[b] (the set read out) per accumulator set.
-// The arithmetic is that of k_ozaki_gemm_ws: the same slices, exact group sums per window of 128, the
+// The arithmetic is that of k_ozaki_gemm_ws above K = 128: the same slices, exact group sums per window of 128, the
 // same int64 combination in units of 2^-53, so the results are the same bits.
 constexpr int kDbN = 32;
 constexpr int kDbBSlice = kDbN * kKW * 2;            // 2 KB: one slice of a 32-column tile's stage
@@ -1869,27 +1905,33 @@ __device__ __forceinline__ void ss_issue(uint32_t tset, uint32_t st, uint32_t B,
 #pragma unroll
     for (int kk = 0; kk < NKK; ++kk)
 #pragma unroll
-        for (int s = 1; s <= kSlices; ++s)
-            mma_f16_n(tset + (s - 1) * N, a0 + static_cast<uint32_t>(((s - 1) * kASlice + kk * 256) >> 4),
-                      b0 + static_cast<uint32_t>(kk * 16), idesc_f16(N * (kSlices + 1 - s)), (kk == 0 && s == 1) ? 0u : 1u);
+        for (int s = 1; s <= kSlices; ++s) {
+            // slices 1 .. nb of T: pairs up to s + b = 9; of slice 2's, the last starts the eighth accumulator
+            const int nb = s == 1 ? kSlices : s == 2 ? kSlices - 1 : kSlices + 2 - s;
+            const uint64_t ad = a0 + static_cast<uint32_t>(((s - 1) * kASlice + kk * 256) >> 4);
+            mma_f16_n(tset + (s - 1) * N, ad, b0 + static_cast<uint32_t>(kk * 16), idesc_f16(N * nb), (kk == 0 && s == 1) ? 0u : 1u);
+            if (s == 2)
+                mma_f16_n(tset + 7 * N, ad, b0 + static_cast<uint32_t>((6 * N * kKW * 2) >> 4) + static_cast<uint32_t>(kk * 16),
+                          idesc_f16(N), kk == 0 ? 0u : 1u);
+        }
     mma_commit(bar);
 }
-// Columns [from, to) of the thread's row (multiples of 4): P[c * kSsLd] -= the update's result (group d at TMEM columns d N).
+// Columns [from, to) of the thread's row (multiples of 4): P[c * kSsLd] -= the update's result (group d at TMEM columns (d - 2) N).
 template <int N>
 __device__ __forceinline__ void ss_drain(uint32_t tl, int from, int to, int E, const int32_t* ey, double* P) {
 #pragma unroll 1
     for (int c0 = from; c0 < to; c0 += 4) {
-        float mg[kGroups][4];
+        float mg[kGroups9][4];
 #pragma unroll
-        for (int q = 0; q < kGroups; ++q) tmem_ld4(tl + q * N + c0, mg[q]);
+        for (int q = 0; q < kGroups9; ++q) tmem_ld4(tl + q * N + c0, mg[q]);
         tmem_wait_ld();
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            float grp[kGroups];
+            float grp[kGroups9];
 #pragma unroll
-            for (int q = 0; q < kGroups; ++q) grp[q] = mg[q][i];
+            for (int q = 0; q < kGroups9; ++q) grp[q] = mg[q][i];
             const int e = ey[c0 + i];
-            if (E > kNoExp && e > kNoExp) P[(c0 + i) * kSsLd] -= scale_pow2_int(combine_units53_k32(grp), E + e - 53);
+            if (E > kNoExp && e > kNoExp) P[(c0 + i) * kSsLd] -= scale_pow2_int(combine_units55_k32(grp), E + e - 55);
         }
     }
 }
