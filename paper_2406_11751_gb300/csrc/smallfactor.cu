@@ -34,7 +34,7 @@ k_chol_panel(double* R, double* W, double* __restrict__ D, int n, int np, int k,
     if (blockIdx.x == 0) {
         for (int e = tid; e < kCb * kCb; e += 128) {
             const int i = e / kCb, j = e % kCb;
-            D[static_cast<int64_t>(k) * kCb * kCb + e] = i <= j ? sh.d[i][j] : 0.0;
+            D[static_cast<int64_t>(k) * kCb * kCb + e] = i <= j && j < nk ? sh.d[i][j] : 0.0;
         }
         if (tid == 0 && sh.bad < nk) set_status(info, RPCHOLQR_ERR_NOT_SPD, k0 + sh.bad);
     }

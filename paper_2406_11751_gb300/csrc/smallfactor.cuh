@@ -49,7 +49,7 @@ __device__ __forceinline__ void root_and_inverse(double x, double& root, double&
 }
 
 struct CholShared {
-    double d[kCb][kCbLd];    // R_kk (upper), rows written as they are finished
+    double d[kCb][kCbLd];    // R_kk (upper, its nk rows), rows written as they are finished
     double inv[kCb];         // 1 / diag
     int bad;                 // first pivot that is not > 0, or kCb
 };
@@ -70,6 +70,7 @@ __device__ __forceinline__ void chol_diag32(const double* A, int64_t lda, int nk
         }
 #pragma unroll
         for (int i = 0; i < kCb; ++i) {
+            if (i == nk) break;   // (a short block's padding is never read)
             if (warp == (i & 3)) {
                 const double piv = __shfl_sync(0xffffffffu, a[i >> 2], i);
                 double root = 1.0, inv = 1.0;
@@ -82,7 +83,6 @@ __device__ __forceinline__ void chol_diag32(const double* A, int64_t lda, int nk
             asm volatile("bar.sync 3, 128;\n" ::: "memory");
             if (i + 1 < kCb) {
                 const double x = -sh.d[i][lane];
-                // the next pivot's row first
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     if (4 * u + 3 <= i) continue;                    // (every row of this u is finished)
