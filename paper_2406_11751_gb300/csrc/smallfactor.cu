@@ -72,6 +72,29 @@ k_chol_trail(double* R, double* W, int n, int np, int k, const int32_t* info) {
     }
 }
 
+// The whole of it for one block, n <= 32: the same steps by one CTA in one launch instead of three (n = 1 14.5 -> 10.3 us, 16 25.0 -> 17.0).
+__global__ void __launch_bounds__(128)
+k_chol_one(const double* __restrict__ G, int64_t ldg, int n, int np, double* __restrict__ R, double* __restrict__ W,
+           double* __restrict__ R_user, int32_t* info) {
+    __shared__ CholShared sh;
+    if (cta_stopped(info)) return;
+    const int tid = threadIdx.x, j0 = 8 * (tid >> 5);
+    chol_diag32(G, ldg, n, sh);
+    if (sh.bad < n) {
+        if (tid == 0) set_status(info, RPCHOLQR_ERR_NOT_SPD, sh.bad);
+        return;
+    }
+    for (int e = tid; e < np * np; e += 128) {
+        const int r = e / np, c = e - r * np;
+        const bool in = r < n && c < n;
+        const double v = in ? (r <= c ? sh.d[r][c] : 0.0) : (r == c ? 1.0 : 0.0);
+        R[e] = v;
+        if (R_user && in) R_user[r * n + c] = v;
+        if (W && !in) W[e] = v;
+    }
+    if (W && j0 < n) chol_rows8(W + static_cast<int64_t>(j0) * np, 1, np, n, n - j0, true, j0, sh);
+}
+
 // The diagonal blocks into R, and (nullable) the n x n factor for the caller.
 __global__ void k_chol_finish(double* __restrict__ R, const double* __restrict__ D, int n, int np, double* __restrict__ R_user,
                               const int32_t* info) {
@@ -98,12 +121,16 @@ __global__ void k_triu_mul(const double* __restrict__ R1, int64_t ld1, const dou
 }
 
 // ---- host launchers ------------------------------------------------------------------------------
-int cholesky_launches(int n) { return 2 * ((n + kCb - 1) / kCb) + 1; }
+int cholesky_launches(int n) { return n <= kCb ? 1 : 2 * ((n + kCb - 1) / kCb) + 1; }
 
 // R (np x np) = chol(G), identity padding; W (nullable, np x np): R^{-1}, identity padding; R_user (nullable, n x n).
 // D: workspace of np x 32 doubles.
 cudaError_t launch_cholesky(const double* G, int64_t ldg, int n, int np, double* R, double* W, double* D, double* R_user,
                             int32_t* info, cudaStream_t st) {
+    if (n <= kCb) {
+        k_chol_one<<<1, 128, 0, st>>>(G, ldg, n, np, R, W, R_user, info);
+        return cudaGetLastError();
+    }
     const int64_t tot = static_cast<int64_t>(np) * np;
     k_chol_init<<<static_cast<unsigned>((tot + 255) / 256), 256, 0, st>>>(G, ldg, n, np, R, W, info);
     const int nb = (n + kCb - 1) / kCb;
