@@ -199,6 +199,67 @@ k_rowsolve_f32(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, in
     if (__syncthreads_or(check_finite && bad) && threadIdx.x == 0) set_status(info, RPCHOLQR_ERR_NONFINITE);
 }
 
+// The same for up to W <= 16 columns, one row per thread in registers: the panels above have nothing to share there and keep
+// few rows in flight (2^20 x 8: 117 us against 21 here, 2^20 x 16: 119 and 34; HBM alone would take 10 and 20).
+template <int W>
+__global__ void __launch_bounds__(256)
+k_rowsolve_f32_narrow(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, int n, const float* __restrict__ T32,
+                      int np32, const float* __restrict__ rinv32, int32_t* info, bool check_finite, bool vec_in,
+                      bool vec_out) {
+    __shared__ float4 ts[W][W / 4];
+    __shared__ float ri[W];
+    if (cta_stopped(info)) return;
+    const int tid = threadIdx.x;
+    if (tid < W * W / 4)
+        ts[tid / (W / 4)][tid % (W / 4)] =
+            *reinterpret_cast<const float4*>(T32 + static_cast<size_t>(tid / (W / 4)) * np32 + 4 * (tid % (W / 4)));
+    if (tid < W) ri[tid] = rinv32[tid];
+    __syncthreads();
+    const int64_t row = static_cast<int64_t>(blockIdx.x) * 256 + tid;
+    bool bad = false;
+    if (row < m) {
+        const float* xr = X + row * ldx;
+        float* yr = Y + row * ldy;
+        float x[W];
+#pragma unroll
+        for (int c = 0; c < W; c += 4) {
+            if (vec_in && c + 3 < n) {
+                const float4 v = *reinterpret_cast<const float4*>(xr + c);
+                x[c] = v.x; x[c + 1] = v.y; x[c + 2] = v.z; x[c + 3] = v.w;
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[c + u] = c + u < n ? xr[c + u] : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < W; ++c) bad |= !isfinite(x[c]);
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            x[j] *= ri[j];
+            const float xj = -x[j];
+#pragma unroll
+            for (int q = (j + 1) / 4; q < W / 4; ++q) {
+                const float4 tv = ts[j][q];
+                if (4 * q + 0 > j) x[4 * q + 0] = fmaf(xj, tv.x, x[4 * q + 0]);
+                if (4 * q + 1 > j) x[4 * q + 1] = fmaf(xj, tv.y, x[4 * q + 1]);
+                if (4 * q + 2 > j) x[4 * q + 2] = fmaf(xj, tv.z, x[4 * q + 2]);
+                if (4 * q + 3 > j) x[4 * q + 3] = fmaf(xj, tv.w, x[4 * q + 3]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < W; c += 4) {
+            if (vec_out && c + 3 < n) {
+                *reinterpret_cast<float4*>(yr + c) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (c + u < n) yr[c + u] = x[c + u];
+            }
+        }
+    }
+    if (__syncthreads_or(check_finite && bad) && tid == 0) set_status(info, RPCHOLQR_ERR_NONFINITE);
+}
+
 // Partials of G = X^T X: CTA (tile, range) accumulates the 64 x 64 tile (I, J), I <= J, over the rows
 // [range*rows_per, ...) and writes gpart[range][p][q] (ld np64, FP64) for its tile.  Thread (ty, tx) of 8 x 16 owns the
 // 8 x 4 outputs p = 64 I + 8 ty + i, q = 64 J + 4 tx + j: three 16-byte reads for 32 multiply-adds (4 x 4 outputs
@@ -342,6 +403,14 @@ static cudaError_t launch_rowsolve_f32_r(const float* X, int64_t ldx, float* Y, 
 cudaError_t launch_rowsolve_f32(const float* X, int64_t ldx, float* Y, int64_t ldy, int64_t m, int n,
                                 const float* T32, const float* rinv32, int32_t* info, bool check_finite, int sms,
                                 cudaStream_t st) {
+    if (n <= 16) {
+        const bool vec_in = reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0;
+        const bool vec_out = reinterpret_cast<uintptr_t>(Y) % 16 == 0 && ldy % 4 == 0;
+        auto kern = n <= 8 ? k_rowsolve_f32_narrow<8> : k_rowsolve_f32_narrow<16>;
+        kern<<<static_cast<unsigned>((m + 255) / 256), 256, 0, st>>>(X, ldx, Y, ldy, m, n, T32, pad32(n), rinv32, info,
+                                                                    check_finite, vec_in, vec_out);
+        return cudaGetLastError();
+    }
     if (m < static_cast<int64_t>(sms) * 64) return launch_rowsolve_f32_r<32>(X, ldx, Y, ldy, m, n, T32, rinv32, info, check_finite, st);
     if (n > 192 || m < static_cast<int64_t>(sms) * 256)
         return launch_rowsolve_f32_r<64>(X, ldx, Y, ldy, m, n, T32, rinv32, info, check_finite, st);
