@@ -38,13 +38,9 @@ void launch_prep_blocks(const double* T, int64_t ldt, int n, int blk, double* fr
                         cudaStream_t st);
 cudaError_t launch_rowpass(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                            int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                           int32_t* info, int sms, cudaStream_t st);
+                           int32_t* info, int sms, cudaStream_t st, bool check_finite);
 void launch_gram_reduce(const double* gpart, int nparts, int np, int n, double* G, int64_t ldg,
                         const int32_t* info, cudaStream_t st);
-cudaError_t launch_rowpass_ex(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
-                              int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                              int32_t* info, int sms, cudaStream_t st, bool check_finite, int32_t* rowexp,
-                              int rowexp_mode, int32_t* colexp);
 void launch_fill_noexp(int32_t* p, int n, cudaStream_t st);
 // probe.cu
 cudaError_t run_fp64_mma_probe(int iters, double* flops_per_s);
@@ -925,8 +921,8 @@ static rpcholqr_status ozaki_gemm_internal(rpcholqr_plan p, bool sub, const doub
 // Diagonal-block setups for the blocked solve with T (n x n, ld ldt): block J (64 columns, the last
 // one ragged) gets frag + 4096 J and diag + 512 J.
 static void prep_blocks(rpcholqr_plan_s* p, const double* T, int64_t ldt, int n, double* frag, double* diag,
-                        const int32_t* info, cudaStream_t st, int blk = kBlk) {
-    launch_prep_blocks(T, ldt, n, blk, frag, diag, info, st);
+                        const int32_t* info, cudaStream_t st) {
+    launch_prep_blocks(T, ldt, n, kBlk, frag, diag, info, st);
     ++p->launches;
 }
 
@@ -1045,9 +1041,8 @@ static rpcholqr_status solve_blocked(rpcholqr_plan_s* p, const double* X, int64_
         }
         {
             KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(m) * nj * nj);
-            if (launch_rowpass_ex(false, pad16(nj), src, lsrc, Y + c0, ldy, m, nj, frag + J * kBlk * kBlk,
-                                  diag + J * (kBlk / 8) * 64, nullptr, info, grid, st, check_finite,
-                                  nullptr, 0, nullptr) != cudaSuccess)
+            if (launch_rowpass(false, pad16(nj), src, lsrc, Y + c0, ldy, m, nj, frag + J * kBlk * kBlk,
+                               diag + J * (kBlk / 8) * 64, nullptr, info, grid, st, check_finite) != cudaSuccess)
                 return RPCHOLQR_ERR_CUDA;
         }
         ++p->launches;
@@ -1103,7 +1098,7 @@ static rpcholqr_status precondition_internal(rpcholqr_plan p, const double* A, i
     if (pm) pm->mark(RPCHOLQR_PHASE_PASS1);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, 2.0 * m * n * n);
-        if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, p->frag_s, p->diag_s, p->gpart, info, p->grid, st) !=
+        if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, p->frag_s, p->diag_s, p->gpart, info, p->grid, st, true) !=
             cudaSuccess)
             return RPCHOLQR_ERR_CUDA;
     }
@@ -1134,7 +1129,7 @@ static rpcholqr_status solve_internal(rpcholqr_plan p, const double* X, int64_t 
     if (pm) pm->mark(RPCHOLQR_PHASE_PASS2);
     {
         KTimer kt(p, st, RPCHOLQR_KERNEL_ROWPASS, static_cast<double>(m) * n * n);
-        if (launch_rowpass(false, np, X, ldx, Y, ldy, m, n, p->frag_1, p->diag_1, nullptr, info, p->grid, st) !=
+        if (launch_rowpass(false, np, X, ldx, Y, ldy, m, n, p->frag_1, p->diag_1, nullptr, info, p->grid, st, false) !=
             cudaSuccess)
             return RPCHOLQR_ERR_CUDA;
     }
@@ -1786,7 +1781,7 @@ static rpcholqr_status cholqr_step(rpcholqr_plan p, const double* X, int64_t m, 
         return solve_internal(p, X, m, n, ldx, R_out, np, Q, ldq, info, st, nullptr);
     }
     launch_prep_tri(nullptr, 0, 0, np, p->frag_s, p->diag_s, info, st);   // identity preconditioner
-    if (launch_rowpass(true, np, X, ldx, Q, ldq, m, n, p->frag_s, p->diag_s, p->gpart, info, p->grid, st) !=
+    if (launch_rowpass(true, np, X, ldx, Q, ldq, m, n, p->frag_s, p->diag_s, p->gpart, info, p->grid, st, true) !=
         cudaSuccess)
         return RPCHOLQR_ERR_CUDA;
     launch_gram_reduce(p->gpart, rowpass_parts(np, m, p->grid), np, n, p->G, np, info, st);

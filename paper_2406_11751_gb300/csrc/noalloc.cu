@@ -26,7 +26,7 @@ void launch_prep_tri(const double* T, int64_t ldt, int n, int np, double* frag, 
                      const int32_t* info, cudaStream_t st);
 cudaError_t launch_rowpass(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                            int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                           int32_t* info, int sms, cudaStream_t st);
+                           int32_t* info, int sms, cudaStream_t st, bool check_finite);
 void launch_gram_reduce(const double* gpart, int nparts, int np, int n, double* G, int64_t ldg,
                         const int32_t* info, cudaStream_t st);
 
@@ -99,7 +99,7 @@ extern "C" rpcholqr_status rpcholqr_precondition_gram_noalloc(const double* A, i
     if (cudaGetLastError() != cudaSuccess) return RPCHOLQR_ERR_CUDA;
     // the fused pass leaves one Gram partial per CTA, at most one CTA per SM
     const int ctas = sms < kNoAllocMaxCtas ? sms : kNoAllocMaxCtas;
-    if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, frag, diag, gpart, info, ctas, st) != cudaSuccess)
+    if (launch_rowpass(true, np, A, lda, A1, ld1, m, n, frag, diag, gpart, info, ctas, st, true) != cudaSuccess)
         return RPCHOLQR_ERR_CUDA;
     launch_gram_reduce(gpart, rowpass_parts(np, m, ctas), np, n, G, n, info, st);
     return cudaGetLastError() == cudaSuccess ? RPCHOLQR_OK : RPCHOLQR_ERR_CUDA;

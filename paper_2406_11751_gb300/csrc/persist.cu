@@ -229,10 +229,9 @@ __device__ __forceinline__ bool item_rows(int short_warps, const double* X, int6
     static_assert(kRowpassWarps * 32 == kPThreads, "the big panels take every warp of the CTA");
     constexpr int W = kRowpassWarps;
     return short_warps ? rowpass_panels<NP, SYRK, 16, W, false, false>(short_warps, W, X, ldx, Y, ldy, m, n, frag, diag, check,
-                                                                       nullptr, 0, nullptr, part, parts, psm, before, emit)
+                                                                       part, parts, psm, before, emit)
                        : rowpass_panels<NP, SYRK, rowpass_rows_per_warp(NP), W, true, false>(
-                             W, W, X, ldx, Y, ldy, m, n, frag, diag, check, nullptr, 0, nullptr, part, parts, psm, before,
-                             emit);
+                             W, W, X, ldx, Y, ldy, m, n, frag, diag, check, part, parts, psm, before, emit);
 }
 
 template <bool SYRK, class BeforeEmit, class Emit>

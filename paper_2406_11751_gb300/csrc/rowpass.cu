@@ -38,15 +38,14 @@ template <int NP, bool SYRK, bool SHORT>
 __global__ void __launch_bounds__(kRowpassWarps * 32, SHORT ? 1 : rowpass_ctas_per_sm(NP, SYRK))
 k_rowpass(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m, int n,
           const double* __restrict__ frag, const double* __restrict__ diag,
-          double* __restrict__ gpart, int32_t* info, bool check_finite, int32_t* rowexp, int rowexp_mode,
-          int32_t* colexp) {
+          double* __restrict__ gpart, int32_t* info, bool check_finite) {
     extern __shared__ double panel[];
     if (cta_stopped(info)) return;
     double* out = SYRK ? gpart + static_cast<size_t>(blockIdx.x) * NP * NP : nullptr;
     const int nw = SHORT ? blockDim.x >> 5 : kRowpassWarps;
     const bool bad = rowpass_panels<NP, SYRK, SHORT ? 16 : rowpass_rows_per_warp(NP),
                                     SHORT ? kRowpassMinWarps : kRowpassWarps, true, true>(
-        nw, nw, X, ldx, Y, ldy, m, n, frag, diag, check_finite, rowexp, rowexp_mode, colexp, blockIdx.x, gridDim.x, panel,
+        nw, nw, X, ldx, Y, ldy, m, n, frag, diag, check_finite, blockIdx.x, gridDim.x, panel,
         [] {}, [out](int pr, int pc, double v) { out[pr * NP + pc] = v; });
     if (__syncthreads_or(bad) && threadIdx.x == 0) set_status(info, RPCHOLQR_ERR_NONFINITE);
 }
@@ -100,8 +99,7 @@ void launch_prep_blocks(const double* T, int64_t ldt, int n, int blk, double* fr
 template <int NP, bool SYRK, bool SHORT>
 static cudaError_t launch_rowpass_t(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
                                     int n, const double* frag, const double* diag, double* gpart,
-                                    int32_t* info, int sms, cudaStream_t st, bool check, int32_t* rowexp,
-                                    int rowexp_mode, int32_t* colexp) {
+                                    int32_t* info, int sms, cudaStream_t st, bool check) {
     const int rows = rowpass_rows(NP, m, sms), warps = SHORT ? rows / 16 : kRowpassWarps;
     auto kern = k_rowpass<NP, SYRK, SHORT>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -109,21 +107,20 @@ static cudaError_t launch_rowpass_t(const double* X, int64_t ldx, double* Y, int
     if (err != cudaSuccess) return err;
     const int64_t panels = (m + rows - 1) / rows, cap = static_cast<int64_t>(sms) * (SHORT ? 1 : rowpass_ctas_per_sm(NP, SYRK));
     kern<<<static_cast<unsigned>(panels < cap ? panels : cap), 32 * warps, rowpass_smem_bytes(NP, rows), st>>>(
-        X, ldx, Y, ldy, m, n, frag, diag, gpart, info, check, rowexp, rowexp_mode, colexp);
+        X, ldx, Y, ldy, m, n, frag, diag, gpart, info, check);
     return cudaGetLastError();
 }
 
 template <bool SYRK>
 static cudaError_t launch_rowpass_np(int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                                      int64_t m, int n, const double* frag, const double* diag,
-                                     double* gpart, int32_t* info, int sms, cudaStream_t st, bool check,
-                                     int32_t* rowexp, int rowexp_mode, int32_t* colexp) {
+                                     double* gpart, int32_t* info, int sms, cudaStream_t st, bool check) {
     const bool brief = rowpass_short_warps(np, m, sms) != 0;
     switch (np) {
 #define RPQ_CASE(V)                                                                                     \
     case V:                                                                                             \
         return (brief ? launch_rowpass_t<V, SYRK, true> : launch_rowpass_t<V, SYRK, false>)(            \
-            X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st, check, rowexp, rowexp_mode, colexp);
+            X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st, check);
         RPQ_CASE(16) RPQ_CASE(32) RPQ_CASE(48) RPQ_CASE(64) RPQ_CASE(80) RPQ_CASE(96) RPQ_CASE(112)
         RPQ_CASE(128)
 #undef RPQ_CASE
@@ -132,25 +129,12 @@ static cudaError_t launch_rowpass_np(int np, const double* X, int64_t ldx, doubl
 }
 
 // sms: SMs to use; the fused Gram pass leaves rowpass_parts(np, m, sms) partials in gpart.
-// check_finite: set NONFINITE when an input entry is NaN/Inf.  rowexp (optional): exponent bound of
-// every solved row over its n columns, stored (rowexp_mode 1) or max-merged (2); colexp (optional,
-// pre-filled with kNoExp): exponent bound of every column over all rows (atomicMax).
-cudaError_t launch_rowpass_ex(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
-                              int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                              int32_t* info, int sms, cudaStream_t st, bool check_finite, int32_t* rowexp,
-                              int rowexp_mode, int32_t* colexp) {
-    return syrk ? launch_rowpass_np<true>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st,
-                                          check_finite, rowexp, rowexp_mode, colexp)
-                : launch_rowpass_np<false>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st,
-                                           check_finite, rowexp, rowexp_mode, colexp);
-}
-
-// The fused Gram pass checks its input for NaN/Inf, the plain solve does not.
+// check_finite: set NONFINITE when an input entry is NaN/Inf.
 cudaError_t launch_rowpass(bool syrk, int np, const double* X, int64_t ldx, double* Y, int64_t ldy,
                            int64_t m, int n, const double* frag, const double* diag, double* gpart,
-                           int32_t* info, int sms, cudaStream_t st) {
-    return launch_rowpass_ex(syrk, np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st, syrk, nullptr, 0,
-                             nullptr);
+                           int32_t* info, int sms, cudaStream_t st, bool check_finite) {
+    return syrk ? launch_rowpass_np<true>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st, check_finite)
+                : launch_rowpass_np<false>(np, X, ldx, Y, ldy, m, n, frag, diag, gpart, info, sms, st, check_finite);
 }
 
 void launch_gram_reduce(const double* gpart, int nparts, int np, int n, double* G, int64_t ldg,

@@ -63,7 +63,6 @@ template <int NP, bool SYRK, int RPW, int TW, bool FULL, bool LDG, class BeforeE
 __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
                                                int n, const double* __restrict__ frag,
                                                const double* __restrict__ diag, bool check_finite,
-                                               int32_t* rowexp, int rowexp_mode, int32_t* colexp,
                                                int64_t p_first, int64_t p_stride, double* panel,
                                                BeforeEmit before_emit, Emit emit) {
     constexpr int S = NP + 4;    // shared-memory row stride in doubles
@@ -72,7 +71,6 @@ __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, 
     constexpr int NB = NP / 8;         // 8-column blocks
     constexpr int NT = upper_tiles(NP);
     constexpr int TPW = (NT + TW - 1) / TW;
-    constexpr int NCM = (NP + 31) / 32;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
@@ -91,11 +89,6 @@ __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, 
         }
     }
     bool bad = false;
-    int cm[SYRK ? 1 : NCM];   // exponent bounds of columns lane, lane + 32, ... over the rows this warp solved
-    if constexpr (!SYRK) {
-#pragma unroll
-        for (int i = 0; i < NCM; ++i) cm[i] = kNoExp;
-    }
 
     for (int64_t p = p_first; p < npanels; p += p_stride) {
         const int64_t row0 = p * ROWS;
@@ -111,7 +104,6 @@ __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, 
 
         // ---- blocked forward substitution of this warp's rows ----
         const int wr0 = warp * RPW;
-        int re = kNoExp;   // exponent bound of this lane's row
         for (int J = 0; J < NB && solver; ++J) {
             double acc[MT][4], acc2[MT][4];
 #pragma unroll
@@ -185,22 +177,6 @@ __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, 
                 }
 #pragma unroll
                 for (int c = 0; c < 8; ++c) xr[c] = x[c];
-                // power-of-two bounds of the solved rows and columns, for the split products that read them next
-                if constexpr (!SYRK) {
-                    if (rowexp) {
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const int e = exp_bound(x[c]);
-                            re = e > re ? e : re;
-                            const int ce = __reduce_max_sync(0xffffffffu, e);
-                            if (((8 * J + c) & 31) == lane) {
-#pragma unroll
-                                for (int q = 0; q < NCM; ++q)
-                                    if (q == (8 * J + c) >> 5) cm[q] = ce > cm[q] ? ce : cm[q];
-                            }
-                        }
-                    }
-                }
             } else {
                 // two lanes per row: lane r + 16 h holds columns h, h + 2, h + 4, h + 6 of the block
                 const int r = lane & 15, h = lane >> 4;
@@ -221,36 +197,8 @@ __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, 
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) xr[2 * i] = x[i];
-                if constexpr (!SYRK) {
-                    if (rowexp) {
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const int e = h == (c & 1) ? exp_bound(x[c >> 1]) : kNoExp;
-                            re = e > re ? e : re;
-                            const int ce = __reduce_max_sync(0xffffffffu, e);
-                            if (((8 * J + c) & 31) == lane) {
-#pragma unroll
-                                for (int q = 0; q < NCM; ++q)
-                                    if (q == (8 * J + c) >> 5) cm[q] = ce > cm[q] ? ce : cm[q];
-                            }
-                        }
-                    }
-                }
             }
             __syncwarp();
-        }
-        if constexpr (!SYRK) {
-            if (rowexp && solver) {
-                if (RPW == 16) {
-                    const int o = __shfl_xor_sync(0xffffffffu, re, 16);
-                    re = o > re ? o : re;
-                }
-                const int64_t gr = row0 + wr0 + lane;
-                if (lane < RPW && gr < m) {
-                    if (rowexp_mode == 2 && rowexp[gr] > re) re = rowexp[gr];
-                    rowexp[gr] = re;
-                }
-            }
         }
         __syncthreads();
 
@@ -294,17 +242,6 @@ __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, 
                 }
             }
         }
-    } else if (colexp) {
-        // the warps' column bounds to one atomic per column of the CTA (the panel is free)
-        int* cs = reinterpret_cast<int*>(panel);
-        for (int c = threadIdx.x; c < n; c += blockDim.x) cs[c] = kNoExp;
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < NCM; ++q)
-            if (solver && lane + 32 * q < n) atomicMax(&cs[lane + 32 * q], cm[q]);
-        __syncthreads();
-        for (int c = threadIdx.x; c < n; c += blockDim.x)
-            if (cs[c] > kNoExp) atomicMax(&colexp[c], cs[c]);
     }
     return bad;
 }
