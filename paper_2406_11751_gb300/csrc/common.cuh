@@ -58,6 +58,49 @@ __device__ __forceinline__ int exp_bound(double v) {
     return ex == 0 ? kNoExp : ex - 1022;
 }
 
+// ---- square roots in 64-bit fixed point (sketch QR, Cholesky) -------------------------------------
+// Both steps wait for a root and a reciprocal in every column.  An FP64 operation takes 65 clocks on GB300 and holds its
+// scheduler's FP64 unit for 64 of them, and a square root or a division is a long sequence of them; a 64 x 64-bit high
+// product takes about 30.  x = X 2^(k - 61) with X / 2^61 in [1, 4); an FP32 seed y ~ x^{-1/2} good to 2^-20 and one step of
+// Halley's iteration t + t h, t = x y, h = e / 2 + 3 e^2 / 8, e = 1 - t y.  The third power left out and the truncations are
+// below 2^-57 of the root.
+__device__ __forceinline__ bool root_in_range(double x) {   // x >= 0 or NaN
+    const int xe = (__double2hiint(x) >> 20) - 1023;
+    return xe >= -900 && xe <= 900;
+}
+struct FixedRoot {
+    unsigned long long X, Y, N;   // x (Q61), y (Q64), sqrt(x) (Q61), all of x's scaled value
+    long long h;                  // Q61
+    int k;                        // x's power of two, even
+    float xf, yf;                 // the scaled x and its seed
+};
+__device__ __forceinline__ FixedRoot fixed_root(double x) {   // root_in_range(x)
+    FixedRoot r;
+    const unsigned long long xb = static_cast<unsigned long long>(__double_as_longlong(x));
+    const int xe = static_cast<int>(xb >> 52) - 1023;
+    r.k = xe & ~1;
+    r.X = ((xb & ((1ull << 52) - 1)) | (1ull << 52)) << (9 + (xe - r.k));
+    r.xf = static_cast<float>(static_cast<uint32_t>(r.X >> 32)) * 0x1p-29f;
+    r.yf = fminf(rsqrtf(r.xf), 0x1.fffffep-1f);
+    r.Y = static_cast<unsigned long long>(__float2uint_rz(r.yf * 0x1p32f)) << 32;
+    const unsigned long long T = __umul64hi(r.X, r.Y);
+    const long long E = static_cast<long long>((1ull << 61) - __umul64hi(T, r.Y));
+    const long long eh = E >> 20;
+    r.h = (E >> 1) + ((3 * ((eh * eh) >> 21)) >> 3);
+    r.N = T + static_cast<unsigned long long>(__mul64hi(static_cast<long long>(T), r.h << 3));
+    return r;
+}
+__device__ __forceinline__ double fixed_root_value(const FixedRoot& r) {
+    return __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(1022 + r.k / 2) << 52) + ((r.N + 256) >> 9)));
+}
+// The Q63 number v > 0 times 2^p in FP64, rounded to nearest without leaving 64 bits (v's leading 64 bits may be 2^64 - 1).
+__device__ __forceinline__ double from_q63(unsigned long long v, int p) {
+    const int lz = __clzll(static_cast<long long>(v));
+    const unsigned long long M = v << lz;
+    return __longlong_as_double(
+        static_cast<long long>((static_cast<unsigned long long>(1022 - lz + p) << 52) + (M >> 11) + ((M >> 10) & 1)));
+}
+
 // ---- status word: info[0] = status, info[1] = pivot ---------------------------------------------
 __device__ __forceinline__ int load_status(const int32_t* info) {
     return *reinterpret_cast<const volatile int32_t*>(info);

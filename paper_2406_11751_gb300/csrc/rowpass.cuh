@@ -161,7 +161,7 @@ __device__ __forceinline__ bool rowpass_panels(int nw, int tw, const double* X, 
             }
             __syncwarp();
             // the 8 x 8 diagonal block, right-looking: each solved column is subtracted from the later ones at
-            // once (independent multiply-adds; a dependent FP64 operation takes about 150 clocks, its issue 64)
+            // once (independent multiply-adds; a dependent one waits 65 clocks for the one before and 64 for the scheduler's other warp)
             const double* d = diag + J * 64;
             auto dg = [&](int i) { return LDG ? __ldg(d + i) : d[i]; };
             if constexpr (RPW == 32) {

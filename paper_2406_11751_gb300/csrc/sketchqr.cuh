@@ -111,48 +111,25 @@ __device__ __forceinline__ bool qr_bar_wait(uint64_t* bar, uint32_t parity) {
     return done != 0;
 }
 
-// nrm = sqrt(x) and g = 1 / (x + nrm |alpha|) for x = alpha^2 + sigma.  Both are on the critical path of every
-// column, and a dependent FP64 operation takes about 150 clocks here, so they are formed in 64-bit fixed point
-// (a 64 x 64-bit high product is about 30): x scaled by a power of four into [1, 4), FP32 seeds y ~ x^{-1/2} and
-// r ~ 1 / (x + nrm |alpha|), good to 2^-20, and one third-order step each -- Halley's iteration
-// nrm = t + t (e / 2 + 3 e^2 / 8), t = x y, e = 1 - t y, and the Neumann series g = r (1 + f + f^2),
-// f = 1 - (x + nrm |alpha|) r.  The third powers left out and the truncations are below 2^-57 of the results,
-// which are then rounded to FP64.  Outside qr_in_range the plain operations are used and false is returned.
-__device__ __forceinline__ bool qr_in_range(double x) {   // x >= 0 or NaN
-    const int xe = (__double2hiint(x) >> 20) - 1023;
-    return xe >= -900 && xe <= 900;
-}
+// nrm = sqrt(x) (fixed_root) and g = 1 / (x + nrm |alpha|) for x = alpha^2 + sigma, both on the critical path of every column:
+// an FP32 seed r ~ g, good to 2^-20, and the Neumann series g = r (1 + f + f^2), f = 1 - (x + nrm |alpha|) r.  Outside
+// root_in_range the plain operations are used and false is returned.
 __device__ __forceinline__ bool qr_scalars(double alpha, double x, double& nrm, double& g) {
-    const unsigned long long xb = static_cast<unsigned long long>(__double_as_longlong(x));
-    const int xe = static_cast<int>(xb >> 52) - 1023, k = xe & ~1;
-    if (qr_in_range(x)) {
-        constexpr unsigned long long kFrac = (1ull << 52) - 1, kOne = 1ull << 52;
+    if (root_in_range(x)) {
         const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(alpha));
-        const int ae = static_cast<int>((ab >> 52) & 0x7FF), sh = ae - 1023 - k / 2 + 9;
-        const unsigned long long X = ((xb & kFrac) | kOne) << (9 + (xe - k));                    // x, Q61
-        const unsigned long long am = ae ? (ab & kFrac) | kOne : 0ull;
+        const FixedRoot q = fixed_root(x);
+        const int ae = static_cast<int>((ab >> 52) & 0x7FF), sh = ae - 1023 - q.k / 2 + 9;
+        const unsigned long long am = ae ? (ab & ((1ull << 52) - 1)) | (1ull << 52) : 0ull;
         const unsigned long long Al = sh >= 0 ? am << sh : (sh > -64 ? am >> -sh : 0ull);        // |alpha| <= 2, Q61
-        const float xf = static_cast<float>(static_cast<uint32_t>(X >> 32)) * 0x1p-29f;
         const float af = static_cast<float>(static_cast<uint32_t>(Al >> 32)) * 0x1p-29f;
-        const float yf = fminf(rsqrtf(xf), 0x1.fffffep-1f);
-        const float rf = fminf(__frcp_rn(fmaf(xf * yf, af, xf)), 0x1.fffffep-1f);
-        const unsigned long long Y = static_cast<unsigned long long>(__float2uint_rz(yf * 0x1p32f)) << 32;   // Q64
+        const float rf = fminf(__frcp_rn(fmaf(q.xf * q.yf, af, q.xf)), 0x1.fffffep-1f);
         const unsigned long long R = static_cast<unsigned long long>(__float2uint_rz(rf * 0x1p32f)) << 32;
-        const unsigned long long T = __umul64hi(X, Y);
-        const long long E = static_cast<long long>((1ull << 61) - __umul64hi(T, Y));
-        const long long eh = E >> 20, h = (E >> 1) + ((3 * ((eh * eh) >> 21)) >> 3);
-        const unsigned long long N = T + static_cast<unsigned long long>(__mul64hi(static_cast<long long>(T), h << 3));
-        nrm = __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(1022 + k / 2) << 52) +
-                                                          ((N + 256) >> 9)));
-        const unsigned long long Dn = (X >> 1) + __umul64hi(N << 1, Al << 1);                     // <= 8, Q60
+        nrm = fixed_root_value(q);
+        const unsigned long long Dn = (q.X >> 1) + __umul64hi(q.N << 1, Al << 1);                 // <= 8, Q60
         const long long F = static_cast<long long>((1ull << 60) - __umul64hi(Dn, R));
         const long long fh = F >> 20;
         const unsigned long long S = (1ull << 60) + static_cast<unsigned long long>(F + ((fh * fh) >> 20));
-        const unsigned long long G = __umul64hi(S << 3, R);                                       // Q63, in [1/8, 1]
-        const int lz = __clzll(static_cast<long long>(G));
-        const unsigned long long M = G << lz;   // rounded below without leaving 64 bits: M may be 2^64 - 1
-        g = __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(1022 - lz - k) << 52) + (M >> 11) +
-                                                        ((M >> 10) & 1)));
+        g = from_q63(__umul64hi(S << 3, R), -q.k);                                               // in [1/8, 1]
         return true;
     }
     nrm = sqrt(x);
@@ -331,7 +308,7 @@ __device__ __forceinline__ bool qr_panel(double* W, int64_t lds, int s, int k0, 
             const double u = fma(alpha, rk, sh.D[lane]), x = fma(alpha, alpha, sigma);
             const bool reflect = (__double_as_longlong(sigma) << 1) != 0;   // else nothing to reflect: v = 0
             double nrm = 0.0, gj = 0.0;
-            const bool in_range = reflect ? qr_scalars(alpha, x, nrm, gj) : qr_in_range(x);
+            const bool in_range = reflect ? qr_scalars(alpha, x, nrm, gj) : root_in_range(x);
             if (!in_range) {   // (the same x in every thread of every CTA)
                 if constexpr (!SCALE) return j;
                 if (tries < 2 && isfinite(x)) {

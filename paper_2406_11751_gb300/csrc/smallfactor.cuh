@@ -10,8 +10,7 @@
 // Every element sees the same operations in the same order whatever the launch shape, so one CTA alone gives
 // the bits of the many-CTA form.
 //
-// Bound: the chain of columns.  A dependent FP64 operation takes about 150 clocks on GB300, and a square root and
-// a division about 2000 each, so the pivot's root and its reciprocal are formed in 64-bit fixed point.
+// Bound: the chain of columns; the pivot's root and its reciprocal are formed in 64-bit fixed point (common.cuh).
 #pragma once
 #include "common.cuh"
 
@@ -20,28 +19,14 @@ namespace rpq {
 constexpr int kCb = 32;               // Cholesky block
 constexpr int kCbLd = kCb + 1;
 
-// root = sqrt(x) and inv = 1 / sqrt(x) for x > 0, as in the sketch QR (qr_scalars): x scaled by a power of four into
-// [1, 4), an FP32 seed y good to 2^-20, one step of Halley's iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - x y^2, in fixed
-// point, rounded to FP64; the plain operations outside the safe range.
+// root = sqrt(x) and inv = 1 / sqrt(x) for x > 0: y (1 + h) as well as the root (fixed_root); the plain operations outside
+// its range.
 __device__ __forceinline__ void root_and_inverse(double x, double& root, double& inv) {
-    const unsigned long long xb = static_cast<unsigned long long>(__double_as_longlong(x));
-    const int xe = static_cast<int>(xb >> 52) - 1023, k = xe & ~1;
-    if (xe >= -900 && xe <= 900) {
-        const unsigned long long X = ((xb & ((1ull << 52) - 1)) | (1ull << 52)) << (9 + (xe - k));   // Q61
-        const float yf = fminf(rsqrtf(static_cast<float>(static_cast<uint32_t>(X >> 32)) * 0x1p-29f), 0x1.fffffep-1f);
-        const unsigned long long Y = static_cast<unsigned long long>(__float2uint_rz(yf * 0x1p32f)) << 32;   // Q64
-        const unsigned long long T = __umul64hi(X, Y);                                               // Q61
-        const long long E = static_cast<long long>((1ull << 61) - __umul64hi(T, Y));
-        const long long eh = E >> 20, h = ((E >> 1) + ((3 * ((eh * eh) >> 21)) >> 3)) << 3;          // Q64
-        const unsigned long long N = T + static_cast<unsigned long long>(__mul64hi(static_cast<long long>(T), h));
-        root = __longlong_as_double(
-            static_cast<long long>((static_cast<unsigned long long>(1022 + k / 2) << 52) + ((N + 256) >> 9)));
-        const unsigned long long I =
-            (Y >> 1) + static_cast<unsigned long long>(__mul64hi(static_cast<long long>(Y >> 1), h));   // Q63
-        const int lz = __clzll(static_cast<long long>(I));
-        const unsigned long long M = I << lz;   // rounded below without leaving 64 bits: M may be 2^64 - 1
-        inv = __longlong_as_double(static_cast<long long>(
-            (static_cast<unsigned long long>(1022 - lz - k / 2) << 52) + (M >> 11) + ((M >> 10) & 1)));
+    if (root_in_range(x)) {
+        const FixedRoot r = fixed_root(x);
+        root = fixed_root_value(r);
+        const unsigned long long y = r.Y >> 1;   // Q63
+        inv = from_q63(y + static_cast<unsigned long long>(__mul64hi(static_cast<long long>(y), r.h << 3)), -r.k / 2);
     } else {
         root = sqrt(x);
         inv = 1.0 / root;
