@@ -452,6 +452,12 @@ CLASS_SOURCE = {"rowpass": "rowpass.cuh", "split_update": "ozaki.cu", "split_gem
                 "fp64_syrk": "blocked.cu", "sketch_qr": "sketchqr.cuh", "cholesky": "smallfactor.cuh"}
 
 
+def class_source(cls, mode):
+    """The file whose kernels a class's launches are: in the split mode the row passes are its block solves."""
+    name = "ozaki.cu" if cls == "rowpass" and mode == "split" else CLASS_SOURCE[cls]
+    return os.path.join(ROOT, "paper_2406_11751_gb300", "csrc", name)
+
+
 def class_bytes(cls, mode, m, n):
     """Algorithmic DRAM bytes per step of a kernel class: what its launches must read and write at least
     (FP64 values, each once per launch that needs it)."""
@@ -483,7 +489,7 @@ def measured_peaks():
 
 def kernel_rooflines(phases, calls, fp64_peak_tflops):
     """Roofline entry per kernel class from the per-launch CUDA events of the timed steps: FP64 classes
-    against the FP64 pipe (in-run probe), split classes against the BF16 tensor pipe (sustained cuBLAS
+    against the FP64 pipe (in-run probe), split classes against the 16-bit tensor pipe (sustained cuBLAS BF16
     figure of MEASURED_PEAKS.json: these kernels run inside a seconds-long step) counting the 28 slice
     products of each FP64-accurate product."""
     peaks = measured_peaks()
@@ -725,7 +731,7 @@ def run_ours(args, ws, rank, local):
     c = max(calls, 1)
     fp32_peak = 152 * 128 * 2 * 2.07e9   # FP32 FMA lanes x 2 flop x max SM clock
     if args.mode == "fp32":
-        kname = "k_rowsolve_f32 (FP32 pass 1: A1 = A Rs^-1, one row per thread)"
+        kname = "k_rowsolve_f32 (FP32 pass 1: A1 = A Rs^-1)"
         launches_per_call = 1
         k_ms = phases["pass1"] / c
         k_flops = float(m) * n * n          # n^2/2 FMAs per row
@@ -748,11 +754,9 @@ def run_ours(args, ws, rank, local):
         roofline = dict(rooflines[dom])
         roofline["class"] = dom
         roofline["algorithmic_bytes_per_launch"] = class_bytes(dom, args.mode, m, n) / roofline["launches_per_step"]
-        roofline["traffic"] = traffic_from_profiles(dom, n, os.path.join(
-            ROOT, "paper_2406_11751_gb300", "csrc", CLASS_SOURCE[dom]), m, roofline["launches_per_step"])
         for cls, r in rooflines.items():
-            r["traffic"] = traffic_from_profiles(cls, n, os.path.join(
-                ROOT, "paper_2406_11751_gb300", "csrc", CLASS_SOURCE[cls]), m, r["launches_per_step"])
+            r["traffic"] = traffic_from_profiles(cls, n, class_source(cls, args.mode), m, r["launches_per_step"])
+        roofline["traffic"] = rooflines[dom]["traffic"]
 
     cpu = None
     if not args.no_cpu_baseline and N == 1:
@@ -761,7 +765,7 @@ def run_ours(args, ws, rank, local):
     out = {
         "metric": METRIC, "value": value, "unit": "matrices/s", "n_gpus": N, "steps": K, "warmup": W,
         "ms_per_step": t_ms_max / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": {"fp64": "f64", "split": "f64+bf16", "fp32": "f32+f64"}[args.mode],
+        "dtype": {"fp64": "f64", "split": "f64+f16", "fp32": "f32+f64"}[args.mode],
         "data": "synthetic (A = U diag(sigma) V^T, Haar U/V from torch, sigma log-spaced)",
         "config": {"workload": f"rpCholesky-QR {args.mode.upper()} m={m} n={n} s={s} kappa={args.kappa:g}"
                                + ("" if args.smoothing == "none" else f" smoothing={args.smoothing.upper()}"), "m": m,
@@ -994,7 +998,7 @@ def run_batch(args, ws, rank, local):
     out = {
         "metric": METRIC, "value": value, "unit": "matrices/s", "n_gpus": ws, "steps": K, "warmup": W,
         "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": {"fp64": "f64", "split": "f64+bf16", "fp32": "f32+f64"}[args.mode],
+        "dtype": {"fp64": "f64", "split": "f64+f16", "fp32": "f32+f64"}[args.mode],
         "data": "synthetic (A = U diag(sigma) V^T per manifest entry, Haar U/V from torch)",
         "config": {"workload": f"rpCholesky-QR batch of {count} (m log-uniform 4096..2^20, n in "
                                f"{{8,16,32,64,128}}, s=3n, kappa log-uniform 1..1e14), {args.mode.upper()}, "

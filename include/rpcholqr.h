@@ -62,9 +62,9 @@ typedef enum {
 
 typedef enum {
     RPCHOLQR_FP64 = 0,   /* every step in FP64 (FP64 tensor-core mma.sync m16n8k16 + DFMA)        */
-    RPCHOLQR_SPLIT64 = 1, /* FP64-accurate split precision: sketch QR, Cholesky and the diagonal
-                            blocks of the row solves in FP64; the Gram matrix, the off-diagonal
-                            block update of the row solve (n > 64) and Q = A1 R1^{-1} (explicit
+    RPCHOLQR_SPLIT64 = 1, /* FP64-accurate split precision: sketch QR, Cholesky and the 16-column
+                            diagonal blocks of the row solve in FP64; the Gram matrix, the rest of
+                            the row solve (n > 16) and Q = A1 R1^{-1} (explicit
                             inverse of the well-conditioned R1) as Ozaki-split FP16 tensor-core
                             (tcgen05) products with exact FP32 group sums and int64 combination.
                             Q = A1 R1^{-1} takes that path only while ||R1||_F ||R1^{-1}||_F / n <= 2

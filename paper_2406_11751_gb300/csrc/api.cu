@@ -595,7 +595,7 @@ const char* rpcholqr_status_string(int status) {
 }
 
 // ---- stage images of the wide split passes (np > 128) ---------------------------------------------------
-// Rows of one chunk of images when they cannot cover every row: 8 GiB of images.
+// Rows of one chunk of images when they cannot cover every row: 8 GiB at 16 bytes a value (the digits take 14).
 int64_t image_chunk_rows(int np) {
     int64_t rows = (int64_t{1} << 33) / static_cast<int64_t>(np * 16) / 128 * 128;
     return rows < 128 ? 128 : rows;

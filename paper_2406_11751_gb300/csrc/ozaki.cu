@@ -59,9 +59,9 @@ constexpr int kASlice = kTileM * kKW * 2;  // 8 KB
 constexpr int kBSlice = kTileN * kKW * 2;  // 4 KB
 constexpr int kAStage = kSlices * kASlice; // 56 KB
 constexpr int kBStage = kSlices * kBSlice; // 28 KB
-// k_ozaki_gemm_ws shared memory: two stages (A slices, then B slices: 96 KB each), then the raw FP64 X
+// k_ozaki_gemm_ws shared memory: two stages (A slices, then B slices: 84 KB each), then the raw FP64 X
 // rows of the next stage (row stride kRawLd doubles: 16-byte reads of one row per thread are
-// conflict-free).  At a tile end the drained stage's 96 KB stage the 128 x 64 output tile (row stride
+// conflict-free).  At a tile end the drained stage's 84 KB stage the 128 x 64 output tile (row stride
 // kEpiLd doubles) so that B is read and C written in whole rows.
 constexpr int kStageBytes = kAStage + kBStage;
 constexpr int kRawLd = kKW + 2;
@@ -789,7 +789,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
                 phase[s] ^= 1u;
                 pending[s] = false;
             }
-            // B slices of stage g: one contiguous 32 KB block
+            // B slices of stage g: one contiguous 28 KB block
             const uint8_t* src = yblocks + static_cast<size_t>((tn * nkw + kw) * kSlices) * kBSlice;
             {
                 for (int e = tid; e < kBStage / 16; e += NT) {
@@ -2198,7 +2198,7 @@ cudaError_t launch_ozaki_gemm(bool sub, const double* X, int64_t ldx, const int3
 }
 
 // Stage images of the row slices of X (m x K, ldx; row bounds xexp) for k_ozaki_gemm_ws with aimg:
-// ceil(m / 128) x ceil(K / 32) images of 64 KB (ozaki_image_bytes).
+// ceil(m / 128) x ceil(K / 32) images of 56 KB (ozaki_image_bytes).
 size_t ozaki_image_bytes(int64_t m, int K) {
     return static_cast<size_t>((m + oz::kTileM - 1) / oz::kTileM) * ((K + oz::kKW - 1) / oz::kKW) * oz::kAStage;
 }

@@ -1,11 +1,11 @@
 // Device-side pieces of the sample's Householder QR (step 'factor' of Algorithm alg_2, Section 4), shared by
 // its kernels (sketchqr.cu) and the persistent batched kernel (persist.cu).
 //
-// FP64 on GB300 retires two multiply-adds per clock per SM, and a dependent FP64 instruction takes 64
-// clocks, so this step is bound by the chain of column steps and by how many SMs share the O(s n^2) work.
+// FP64 on GB300 retires two multiply-adds per clock per SM (a warp's instruction takes its scheduler 64 clocks) and a
+// dependent one waits about 150, so this step is bound by the chain of column steps and by how many SMs share the O(s n^2) work.
 // Panels of kQrB columns: the panel is factored by one thread-block cluster with its ROWS shared out (one
 // reduction over the cluster per column), then the columns to its right are updated by every SM:
-//   panel   W[:, panel] -> reflectors H_j = I - g_j v_j v_j^T, v_j = x - beta e_j unscaled,
+//   panel   W[:, panel] -> reflectors H_j = I - g_j v_j v_j^T, v_j = x - beta e_j not normalised,
 //           beta = -sign(alpha) ||x||, g_j = 1 / (||x|| (||x|| + |alpha|)) (no reflection when nothing is
 //           below the diagonal); the reduction for column j gives sigma = sum of squares below the diagonal
 //           and the products of x with every panel column at once: those to the right take the update, those

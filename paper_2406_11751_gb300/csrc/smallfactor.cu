@@ -11,7 +11,7 @@ namespace rpq {
 // columns take part as block columns j <= k, entry (r, c) of R^{-T} at W[c * np + r].
 //   k_chol_panel   CTA c: factor W_kk, then block column k + 1 + c of R, or the identity's block column c - (nb - k - 1);
 //   k_chol_trail   one warp per 16 x 8 tile of the updated blocks.
-// Measured on GB300, Cholesky alone: n = 50 103 -> 85 us, 128 326 -> 200, 512 1.30 -> 0.92 ms, 1000 2.82 -> 2.02 ms; R^{-1}
+// Measured on GB300, Cholesky alone: n = 64 126 -> 81 us, 128 323 -> 198, 512 1.30 -> 0.92 ms, 1000 2.82 -> 2.02 ms; R^{-1}
 // takes no further launches where a warp per column took 0.12 ms (n = 128) to 0.95 ms (512) and a blocked row solve of
 // the identity 21 ms (1000).
 __global__ void k_chol_init(const double* __restrict__ G, int64_t ldg, int n, int np, double* __restrict__ R,

@@ -19,7 +19,7 @@ def matrix(m, n):
 
 
 @pytest.mark.parametrize("mode", ["FP64", "SPLIT64"])
-@pytest.mark.parametrize("m,n,s", [(600, 1, 3), (900, 40, 120), (2000, 130, 390)])
+@pytest.mark.parametrize("m,n,s", [(600, 1, 3), (900, 40, 120), (2000, 130, 390), (14000, 33, 13000)])   # the last: panel in place
 def test_powers_of_two(lib, mode, m, n, s):
     A = matrix(m, n)
     plan = lib.rpcholqr_plan_create(0, m, n, s, mode=getattr(lib, mode))
