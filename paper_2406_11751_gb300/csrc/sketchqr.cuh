@@ -1,8 +1,9 @@
 // Device-side pieces of the sample's Householder QR (step 'factor' of Algorithm alg_2, Section 4), shared by
 // its kernels (sketchqr.cu) and the persistent batched kernel (persist.cu).
 //
-// FP64 on GB300 retires two multiply-adds per clock per SM (a warp's instruction takes its scheduler 64 clocks) and a
-// dependent one waits about 150, so this step is bound by the chain of column steps and by how many SMs share the O(s n^2) work.
+// FP64 on GB300 retires two multiply-adds per clock per SM, one warp's instruction in 64 clocks of its scheduler, and a
+// dependent one waits as long, so this step is bound by the chain of column steps and by how many SMs share the O(s n^2)
+// work.
 // Panels of kQrB columns: the panel is factored by one thread-block cluster with its ROWS shared out (one
 // reduction over the cluster per column), then the columns to its right are updated by every SM:
 //   panel   W[:, panel] -> reflectors H_j = I - g_j v_j v_j^T, v_j = x - beta e_j not normalised,
@@ -139,10 +140,10 @@ __device__ __forceinline__ bool qr_scalars(double alpha, double x, double& nrm, 
 
 // Factor the panel of columns k0 .. k0 + nb - 1 (rows k0 .. s - 1) of W (column-major, ld lds) by the calling
 // CTA as CTA `rank` of `csize` (CLUSTER: a thread-block cluster, csize a power of two <= 16; otherwise one CTA).
-// A column whose remaining norm is outside [2^-450, 2^450] is scaled by a power of two and its products are formed again
-// (at most twice, which brings any column into the range): unscaled, g and the products over- or underflow.  H_j does
-// not depend on the scale of v_j; R's entry takes it back.  Where the sum of squares itself overflows, R's diagonal entry
-// is infinite and the sketch counts as singular.
+// A column whose remaining norm is outside [2^-450, 2^450] is scaled by a power of two and its products are formed again:
+// unscaled, g and the products over- or underflow.  H_j does not depend on the scale of v_j; R's entry takes it back.  A
+// column whose squares below the diagonal all vanish (entries under 2^-537) has nothing to reflect, as one of zeros;
+// where the sum of squares overflows, R's diagonal entry is infinite and the sketch counts as singular.
 // W's panel columns become V (v_j from row j down, vp on the diagonal; g_j = 0 where nothing is reflected) with R
 // above the diagonal; L[j * ldl + k] = v_j^T v_k (k < j), g and betas[k0 + j].  SMEM: panel is shared memory for
 // this CTA's rows (kQrLd doubles each); otherwise the panel is worked on in place.
@@ -256,8 +257,8 @@ __device__ __forceinline__ bool qr_panel(double* W, int64_t lds, int s, int k0, 
     // made.  SCALE is a loop of its own, so that the usual one holds nothing of it (3 us a panel otherwise).
     auto columns = [&](auto scale_t, int j0, int ex) -> int {
         constexpr bool SCALE = decltype(scale_t)::value;
-        int tries = 0;                               // scalings of the current column
-        double unscale = 1.0;                        // what takes them back
+        bool scaled = false;                         // the current column is scaled,
+        double unscale = 1.0;                        // and this takes it back
         for (int j = j0; j < nb;) {
             const int par = ex & 1;
             const bool owner_cta = pg >= 0 && pg < ng, owner = owner_cta && warp == pg % NW;
@@ -308,14 +309,14 @@ __device__ __forceinline__ bool qr_panel(double* W, int64_t lds, int s, int k0, 
             const double u = fma(alpha, rk, sh.D[lane]), x = fma(alpha, alpha, sigma);
             const bool reflect = (__double_as_longlong(sigma) << 1) != 0;   // else nothing to reflect: v = 0
             double nrm = 0.0, gj = 0.0;
-            const bool in_range = reflect ? qr_scalars(alpha, x, nrm, gj) : root_in_range(x);
+            const bool in_range = !reflect || qr_scalars(alpha, x, nrm, gj);
             if (!in_range) {   // (the same x in every thread of every CTA)
                 if constexpr (!SCALE) return j;
-                if (tries < 2 && isfinite(x)) {
+                if (!scaled && isfinite(x)) {
                     const bool up = x < 1.0;
                     const double f = up ? 0x1p500 : 0x1p-600;
-                    unscale *= up ? 0x1p-500 : 0x1p600;
-                    ++tries;
+                    unscale = up ? 0x1p-500 : 0x1p600;
+                    scaled = true;
                     for (int q = warp; q < ng; q += NW) {
                         const int ib = (g0 + q) * rg > j ? (g0 + q) * rg : j;
                         const int ie = (g0 + q + 1) * rg < nrows ? (g0 + q + 1) * rg : nrows;
@@ -357,7 +358,7 @@ __device__ __forceinline__ bool qr_panel(double* W, int64_t lds, int s, int k0, 
             for (int q = warp; q < ng; q += NW) rows_step(std::true_type{}, q, j, w);
             __syncwarp();
             ++j;
-            tries = 0;
+            scaled = false;
             unscale = 1.0;
         }
         return nb;
