@@ -18,7 +18,8 @@
 // F = rint(x 2^{55-E}), and cut into seven signed 8-bit digits, F = sum_{a=1..7} s_a 256^{7-a}, |s_a| <= 128
 // (exact in FP16), so x = 2^E (sum s_a 2^{1-8a} + e), |e| <= 2^-56.  A product of two such operands is
 // sum_{a,b} 2^{2-8(a+b)} S_a S_b; the 28 pairs with a + b <= 8 are kept (the six dropped ones with a + b = 9 are below
-// 6 2^-56 of the scale a term, 2^-56 in the mean square).  Pairs with the same d = a + b share one FP32 accumulator in
+// 6 2^-56 of the scale a term, 2^-56 in the mean square; the first pass's products up to 128 columns keep them as well, see
+// kGroups9).  Pairs with the same d = a + b share one FP32 accumulator in
 // tensor memory: with K <= 128 every partial sum is an integer below 7 128^2 128 < 2^24, so the FP32 accumulation is
 // exact.  The seven accumulators (d = 2..8) are combined exactly in int64 and rounded once to units of 2^-53 of the
 // scale.  (Eight 7-bit digits in BF16 needed 36 pairs, 16 instead of 14 bytes a value and about twice the
@@ -2211,8 +2212,8 @@ void launch_slice_images(const double* X, int64_t ldx, int64_t m, int K, const i
 int32_t ozaki_no_exp() { return kNoExp; }
 
 // Tables of the 64-column diagonal blocks of an n x n T (split_solve_tab_bytes(n)), and the solve of block J's nc columns of
-// m rows with them (X, Y at the block's first column).  Measured on GB300, one 64-column block of 2^21 rows: 3.24 ms
-// (FP64 pipe 66 % busy), against 4.7 ms for four FP64 row passes and three update launches; the row in registers with
+// m rows with them (X, Y at the block's first column).  Measured on GB300, one 64-column block of 2^21 rows: 3.25 ms
+// (FP64 pipe 65 % busy), against 4.7 ms for four FP64 row passes and three update launches; the row in registers with
 // everything unrolled 3.88 (8-column sub-blocks 4.0), one thread per row with rolled loops 3.52.
 size_t split_solve_tab_bytes(int n) { return static_cast<size_t>((n + 63) / 64) * oz::kSsTab; }
 void launch_split_solve_prep(const double* T, int64_t ldt, int n, uint8_t* tab, const int32_t* info, cudaStream_t st) {
