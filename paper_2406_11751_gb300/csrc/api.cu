@@ -53,7 +53,7 @@ cudaError_t launch_ozaki_gemm(bool sub, const double* X, int64_t ldx, const int3
                               const uint8_t* yblocks, const int32_t* yexp, int N, const double* B,
                               int64_t ldb, double* C, int64_t ldc, int64_t m, int32_t* info, int grid,
                               cudaStream_t st, long spin, bool y_upper, const uint8_t* aimg, int img_nkw,
-                              const int32_t* bexp, int64_t ld_bexp);
+                              const int32_t* bexp, int64_t ld_bexp, bool nine);
 size_t ozaki_image_bytes(int64_t m, int K);
 void launch_slice_images(const double* X, int64_t ldx, int64_t m, int K, const int32_t* xexp, uint8_t* img,
                          const int32_t* info, cudaStream_t st);
@@ -916,7 +916,7 @@ static rpcholqr_status ozaki_gemm_internal(rpcholqr_plan p, bool sub, const doub
                                            int64_t ldb, double* C, int64_t ldc, int32_t* info, cudaStream_t st,
                                            bool xexp_ready = false, int64_t row0 = 0, bool y_ready = false,
                                            bool y_upper = false, const uint8_t* aimg = nullptr, int img_nkw = 0,
-                                           const int32_t* bexp = nullptr, int64_t ld_bexp = 0);
+                                           const int32_t* bexp = nullptr, int64_t ld_bexp = 0, bool nine = false);
 
 // Diagonal-block setups for the blocked solve with T (n x n, ld ldt): block J (64 columns, the last
 // one ragged) gets frag + 4096 J and diag + 512 J.
@@ -951,7 +951,8 @@ static rpcholqr_status solve_split(rpcholqr_plan_s* p, const double* X, int64_t 
         if (pm && J == 1) pm->mark(RPCHOLQR_PHASE_PASS1_UPDATE);
         rpcholqr_status rc = RPCHOLQR_OK;
         if (J > 0)
-            rc = ozaki_gemm_internal(p, true, Y, m, c0, ldy, T + c0, nj, ldt, X + c0, ldx, Y + c0, ldy, info, st, true, row0);
+            rc = ozaki_gemm_internal(p, true, Y, m, c0, ldy, T + c0, nj, ldt, X + c0, ldx, Y + c0, ldy, info, st, true, row0, false,
+                                     false, nullptr, 0, nullptr, 0, true);
         if (rc != RPCHOLQR_OK) return rc;
         if (pm && J == 1) pm->mark(RPCHOLQR_PHASE_PASS1_SOLVE2);
         rc = solve_split_block(p, (J == 0 ? X : Y) + c0, J == 0 ? ldx : ldy, Y + c0, ldy, m, nj, J, row0, info, st);
@@ -1140,12 +1141,13 @@ static rpcholqr_status solve_internal(rpcholqr_plan p, const double* X, int64_t 
 // C = X Y (sub = false) or C = B - X Y (sub = true) on the tensor cores; X row bounds computed here.
 // xexp_ready: p->xexp already holds the row bounds of X (written by the row pass that produced X);
 // row0: X's first row within the matrix whose bounds p->xexp holds; y_ready: p->yblocks already holds
-// the slices of this Y; y_upper: Y is upper triangular (the product skips its zero K stages).
+// the slices of this Y; y_upper: Y is upper triangular (the product skips its zero K stages); nine: six more digit pairs (first
+// pass, K <= 128).
 static rpcholqr_status ozaki_gemm_internal(rpcholqr_plan p, bool sub, const double* X, int64_t m, int K,
                                            int64_t ldx, const double* Y, int N, int64_t ldy, const double* B,
                                            int64_t ldb, double* C, int64_t ldc, int32_t* info, cudaStream_t st,
                                            bool xexp_ready, int64_t row0, bool y_ready, bool y_upper,
-                                           const uint8_t* aimg, int img_nkw, const int32_t* bexp, int64_t ld_bexp) {
+                                           const uint8_t* aimg, int img_nkw, const int32_t* bexp, int64_t ld_bexp, bool nine) {
     int32_t* xexp = p->xexp + row0;
     if (!xexp_ready) {
         launch_row_exp(X, ldx, m, K, xexp, st);
@@ -1162,7 +1164,7 @@ static rpcholqr_status ozaki_gemm_internal(rpcholqr_plan p, bool sub, const doub
         KTimer kt(p, st, ozaki_class(sub, K, N), ozaki_flops(sub, y_upper, m, K, N));
         if (launch_ozaki_gemm(sub, X, ldx, xexp, K, p->yblocks, p->yexp, N, B, ldb, C, ldc, m, info, grid, st,
                               static_cast<long>(p->spin_limit), y_upper, aimg,
-                              img_nkw > 0 ? img_nkw : (K + 31) / 32, bexp, ld_bexp) !=
+                              img_nkw > 0 ? img_nkw : (K + 31) / 32, bexp, ld_bexp, nine) !=
             cudaSuccess)
             return RPCHOLQR_ERR_CUDA;
     }

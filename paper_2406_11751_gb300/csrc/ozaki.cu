@@ -283,16 +283,17 @@ __device__ __forceinline__ long long combine_units53_k32(const float (&m)[kGroup
     return combine_ints<53>(v);
 }
 
-// The first pass's products keep the pairs with a + b = 9 too (an eighth accumulator, K <= 128): their error reaches A_1
+// The first pass's products up to 128 columns keep the pairs with a + b = 9 too (an eighth accumulator): their error reaches A_1
 // multiplied by kappa(A), and the dropped pairs were most of it.  Distance of Q from its value in 80 bits, A_1 by this pass and
 // the rest exact, 1200 rows, kappa = 1e5: n = 33 0.97 -> 0.38e-12, 64 1.05 -> 0.34, 100 1.18 -> 0.42, 128 1.10 -> 0.41 (FP64
 // substitution: 0.41, 0.51, 0.59, 0.68).
 constexpr int kGroups9 = kGroups + 1;
-// Its seven group sums and M_9, in units of 2^-53.
+// Its seven group sums and M_9, in units of 2^-53.  |M_2|, |M_3| <= 2^22 with K <= 128, so these two come from the bit patterns
+// (combine_units53_k32): six conversions, the drain's bound, instead of eight.
 __device__ __forceinline__ long long combine_units53_d9(const float (&m)[kGroups9]) {
     int v[kGroups];
 #pragma unroll
-    for (int g = 0; g < kGroups; ++g) v[g] = __float2int_rn(m[g]);
+    for (int g = 0; g < kGroups; ++g) v[g] = g < 2 ? __float_as_int(m[g] + 12582912.0f) - 0x4B400000 : __float2int_rn(m[g]);
     v[6] += (__float2int_rn(m[7]) + 128) >> 8;
     return combine_ints<53>(v);
 }
@@ -391,7 +392,8 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t a_base, uint
     for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
         for (int a = 1; a <= kSlices; ++a) {
-            const int nb = !D9 ? kSlices + 1 - a : a == 1 ? kSlices : a == 2 ? kSlices - 1 : kSlices + 2 - a;
+            const bool start9 = D9 && a == 2 && kk == 0 && first_window;   // its last pair apart, to clear the eighth
+            const int nb = !D9 ? kSlices + 1 - a : a == 1 ? kSlices : a == 2 ? kSlices - start9 : kSlices + 2 - a;
             const int n1 = nb < 4 ? nb : 4;
             const uint64_t ad = a0 + static_cast<uint32_t>(((a - 1) * kASlice + kk * 256) >> 4);
             const uint32_t acc = (first_window && kk == 0 && a == 1) ? 0u : 1u;
@@ -400,10 +402,9 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t a_base, uint
                 mma_f16_n(tmem + (a + 3) * kTileN, ad,
                           b0 + static_cast<uint32_t>((4 * kBSlice) >> 4) + static_cast<uint32_t>(kk * 16),
                           idesc_f16(kTileN * (nb - 4)), acc);
-            if (D9 && a == 2)
+            if (start9)
                 mma_f16_n(tmem + 7 * kTileN, ad,
-                          b0 + static_cast<uint32_t>((6 * kBSlice) >> 4) + static_cast<uint32_t>(kk * 16), idesc_f16(kTileN),
-                          (first_window && kk == 0) ? 0u : 1u);
+                          b0 + static_cast<uint32_t>((6 * kBSlice) >> 4) + static_cast<uint32_t>(kk * 16), idesc_f16(kTileN), 0u);
         }
     }
 }
@@ -570,7 +571,7 @@ __device__ __forceinline__ void prefetch_x(const double* X, int64_t ldx, int64_t
 // Write the finished tile (rows row0 + 0..127, columns 64 tn + 0..63) of C = X Y through the staging
 // buffer W (run by the NT producer threads): each thread puts its row's NC values into W, then the tile
 // is written in whole rows.  The values come from the TMEM accumulators (single window) or from acc (WIN).
-template <bool WIN, bool SUB, bool HALF, int NT, int NC>
+template <bool WIN, bool SUB, bool HALF, bool D9, int NT, int NC>
 __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid, int64_t row0, int tn, int E,
                                                 int N, const int32_t* __restrict__ yexp, const double* B,
                                                 int64_t ldb, double* C, int64_t ldc, int64_t m, double* W,
@@ -589,7 +590,7 @@ __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid
             wr[j] = v;
         }
     } else {
-        constexpr int NG = SUB ? kGroups9 : kGroups;
+        constexpr int NG = D9 ? kGroups9 : kGroups;
 #pragma unroll 1
         for (int c0 = 0; c0 < NC; c0 += 8) {
             float mg[NG][8];
@@ -606,7 +607,7 @@ __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid
                 for (int g = 0; g < NG; ++g) grp[g] = mg[g][j];
                 if (col < N) {
                     long long I;
-                    if constexpr (SUB) I = combine_units53_d9(grp);
+                    if constexpr (D9) I = combine_units53_d9(grp);
                     else I = combine_units<53>(grp);
                     const int ey = yexp[col];
                     const double v = (E > kNoExp && ey > kNoExp) ? scale_pow2(I, E + ey - 53) : 0.0;
@@ -638,6 +639,7 @@ __device__ __forceinline__ void gemm_store_tile(uint32_t tmem, int warp, int tid
 // B, C: m x N FP64 (ldb, ldc); C may equal B.  Persistent grid over 128-row x 64-column tiles.
 // WIN (128 < K <= 2048): the K range is cut into exactness windows of 128, each drained into int64
 // accumulators in units of 2^-53 of the scale (the same resolution as a single window; HALF above K = 1024).
+// D9 (not WIN): the digit pairs with a + b = 9 too, for the first pass (kGroups9).
 // The CTA's (tile, K-stage) sequence is one stream of stages over two shared-memory buffers: stage g is
 // sliced while the MMAs of stage g - 1 run; when stage g opens a new exactness window (or a new tile)
 // the previous window's accumulators are drained (into int64, or out to C at a tile end) before its
@@ -688,7 +690,7 @@ struct StageWalk {
     }
 };
 
-template <bool WIN, bool SUB, bool HALF = false>
+template <bool WIN, bool SUB, bool HALF = false, bool D9 = false>
 __global__ void __launch_bounds__((WIN ? kThreadsWin : kThreads) + 32, 1)
 k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, int K,
                 const uint8_t* __restrict__ yblocks, const int32_t* __restrict__ yexp, int N, const double* B,
@@ -751,7 +753,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
                 }
                 fphase[s] ^= 1u;
                 tc_after_sync();
-                issue_stage<!WIN && SUB>(tmem, smem_u32(stA[s]), smem_u32(stB[s]), (wk.kw & 3) == 0);
+                issue_stage<D9>(tmem, smem_u32(stA[s]), smem_u32(stB[s]), (wk.kw & 3) == 0);
                 mma_commit(&empty_bar[s]);
             }
             // every MMA issued here is complete before the tensor memory is released
@@ -837,7 +839,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
                 tc_after_sync();
                 if (kw == 0) {
                     // every MMA so far is complete: stage sp's buffer stages the output tile
-                    gemm_store_tile<WIN, SUB, HALF, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
+                    gemm_store_tile<WIN, SUB, HALF, D9, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
                                                  reinterpret_cast<double*>(stA[sp]), acc, bits);
                     bits = 0;
 #pragma unroll
@@ -869,7 +871,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
                 }
             if (!timed_out) {
                 tc_after_sync();
-                gemm_store_tile<WIN, SUB, HALF, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
+                gemm_store_tile<WIN, SUB, HALF, D9, NT, NC>(tmem, warp, tid, cur_row0, cur_tn, cur_E, N, yexp, B, ldb, C, ldc, m,
                                              reinterpret_cast<double*>(stA[0]), acc, bits);
             }
         }
@@ -896,7 +898,7 @@ k_ozaki_gemm_ws(const double* X, int64_t ldx, const int32_t* __restrict__ xexp, 
 // warp 9 lane 0 issues the MMAs (7 per K = 16 step: Y's seven 32-column slices are stacked, N = 32 (8 - a)
 // for slice a of X).  Barriers: load[s] (bytes landed) and empty[s] (MMAs of the stage done) per stage
 // buffer; acc_full[b] (the window's MMAs done) and acc_empty[b] (the set read out) per accumulator set.
-// The arithmetic is that of k_ozaki_gemm_ws above K = 128: the same slices, exact group sums per window of 128, the
+// The arithmetic is that of k_ozaki_gemm_ws: the same slices, exact group sums per window of 128, the
 // same int64 combination in units of 2^-53, so the results are the same bits.
 constexpr int kDbN = 32;
 constexpr int kDbBSlice = kDbN * kKW * 2;            // 2 KB: one slice of a 32-column tile's stage
@@ -1907,13 +1909,14 @@ __device__ __forceinline__ void ss_issue(uint32_t tset, uint32_t st, uint32_t B,
     for (int kk = 0; kk < NKK; ++kk)
 #pragma unroll
         for (int s = 1; s <= kSlices; ++s) {
-            // slices 1 .. nb of T: pairs up to s + b = 9; of slice 2's, the last starts the eighth accumulator
-            const int nb = s == 1 ? kSlices : s == 2 ? kSlices - 1 : kSlices + 2 - s;
+            // slices 1 .. nb of T: pairs up to s + b = 9; the first step's last pair of slice 2 starts the eighth accumulator
+            const bool start9 = s == 2 && kk == 0;
+            const int nb = s == 1 ? kSlices : s == 2 ? kSlices - start9 : kSlices + 2 - s;
             const uint64_t ad = a0 + static_cast<uint32_t>(((s - 1) * kASlice + kk * 256) >> 4);
             mma_f16_n(tset + (s - 1) * N, ad, b0 + static_cast<uint32_t>(kk * 16), idesc_f16(N * nb), (kk == 0 && s == 1) ? 0u : 1u);
-            if (s == 2)
+            if (start9)
                 mma_f16_n(tset + 7 * N, ad, b0 + static_cast<uint32_t>((6 * N * kKW * 2) >> 4) + static_cast<uint32_t>(kk * 16),
-                          idesc_f16(N), kk == 0 ? 0u : 1u);
+                          idesc_f16(N), 0u);
         }
     mma_commit(bar);
 }
@@ -2160,7 +2163,7 @@ cudaError_t launch_ozaki_gemm(bool sub, const double* X, int64_t ldx, const int3
                               const uint8_t* yblocks, const int32_t* yexp, int N, const double* B,
                               int64_t ldb, double* C, int64_t ldc, int64_t m, int32_t* info, int grid,
                               cudaStream_t st, long spin, bool y_upper, const uint8_t* aimg, int img_nkw,
-                              const int32_t* bexp, int64_t ld_bexp) {
+                              const int32_t* bexp, int64_t ld_bexp, bool nine) {
     if (K > 64 * oz::kKW) return cudaErrorInvalidValue;   // the totals hold K <= 2048 (add_window)
     const bool win = K > 4 * oz::kKW, half = K > 32 * oz::kKW;
     const int nt = win ? oz::kThreadsWin : oz::kThreads;
@@ -2189,6 +2192,7 @@ cudaError_t launch_ozaki_gemm(bool sub, const double* X, int64_t ldx, const int3
         return cudaGetLastError();
     }
     auto kern = half ? (sub ? oz::k_ozaki_gemm_ws<true, true, true> : oz::k_ozaki_gemm_ws<true, false, true>)
+                : nine && sub && !win ? oz::k_ozaki_gemm_ws<false, true, false, true>
                 : win ? (sub ? oz::k_ozaki_gemm_ws<true, true> : oz::k_ozaki_gemm_ws<true, false>)
                     : (sub ? oz::k_ozaki_gemm_ws<false, true> : oz::k_ozaki_gemm_ws<false, false>);
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::kGemmSmem);
